@@ -158,17 +158,19 @@ cdbm_status cdbm_init(cdbm_ctx *ctx, const double *rho, const double *ux, const 
  */
 cdbm_status cdbm_step(cdbm_ctx *ctx, int nsteps);
 
-/* Enables (default) or disables the small-grid paths of cdbm_step for 1-D grids: the
- * persistent cluster kernel, and for CDBM_FP64 tubes of up to 8192 cells the stage
- * kernel that splits each cell over four threads.  Disabled, those grids step with
- * the one-cell-per-thread stage kernel like any other. */
+/* Enables (default) or disables the small-grid paths of cdbm_step: on 1-D grids the
+ * persistent cluster kernel, and for CDBM_FP64 the stage kernels that split each cell
+ * over four threads (grids of up to about 29000 cells; on 2-D grids the results are the
+ * same bit for bit).  Disabled, those grids step with the one-cell-per-thread stage
+ * kernel like any other. */
 cdbm_status cdbm_set_small_grid_path(cdbm_ctx *ctx, int enable);
 
-/* Enables (default) or disables the row-marching stage kernels on 2-D grids, which
- * carry the y differences of a run of rows in shared memory (and, for
- * CDBM_FP32_DF64, advance two columns per thread with packed FP32x2 arithmetic);
- * disabled, every stage runs one cell per thread.  Both give the same results bit
- * for bit; the switch serves cross-checks and timing.  EINVAL for a NULL context. */
+/* Enables (default) or disables the row-marching stage kernels of the single-precision
+ * states on 2-D grids, which carry the y differences of a run of rows in shared memory
+ * (and, for CDBM_FP32_DF64 and CDBM_FP32_DEV, advance two columns per thread); disabled,
+ * every stage runs one cell per thread.  Both give the same results bit for bit; the
+ * switch serves cross-checks and timing and has no effect on CDBM_FP64, whose stages
+ * never march.  EINVAL for a NULL context. */
 cdbm_status cdbm_set_row_marching(cdbm_ctx *ctx, int enable);
 
 /*

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "cdbm_stage.cuh"
+#include "cdbm_stage_fx.cuh"
 #include "cdbm_internal.h"
 
 using namespace cdbm;
@@ -36,6 +37,7 @@ struct TubeInfo {
     double lx[2][4];                  // per stage: gamma dt c_g / dx_t
     float lx_f[2][4];
     float2 lx_f2[2][4];               // lx_f twice (two-column df64 stage)
+    FxFlux fx[2];                     // per stage: lx in fixed point (CDBM_FP64)
     double sF[2][4];                  // per stage: gamma h F_g (FP32-bulk reference)
     double Fg[4];                     // reference equilibrium per group
     double rhoF, EF;                  // its conserved moments
@@ -51,6 +53,7 @@ struct ClassConsts {
     DFModel dfm;
     DFBlocksT<float2> dfeq2[2];       // the same with each value twice
     DFModelT<float2> dfm2;
+    FxModel fx;                       // fixed-point model constants (CDBM_FP64)
     DevProj dp[2];                    // per stage: conservation projection (CDBM_FP32_DEV)
 };
 
@@ -59,19 +62,14 @@ struct BatchArgs {
     double a_self[2], a_base[2];
     float a_self_f[2], a_base_f[2];
     float2 a_self_f2[2], a_base_f2[2];
+    FxCoef fx[2];                     // fixed-point stage coefficients (CDBM_FP64)
     long long P;                      // total cells: stride between velocity planes
 };
 
-template <typename TS>
-__device__ __forceinline__ TS pick(double d, float f)
-{
-    if constexpr (kSingle<TS>) return f; else return d;
-}
-
 // The 16 values of cell x of a tube; with kSym only the 10 distinct velocities of a
 // y-symmetric state are loaded and the mirror images copied from them.
-template <typename TS, bool kSym>
-__device__ __forceinline__ void load_state(const TS *g, long long P, int x, TS fs[kNV])
+template <bool kSym>
+__device__ __forceinline__ void load_state(const float *g, long long P, int x, float fs[kNV])
 {
 #pragma unroll
     for (int i = 0; i < kNV; ++i)
@@ -83,7 +81,7 @@ __device__ __forceinline__ void load_state(const TS *g, long long P, int x, TS f
     }
 }
 
-// One Runge-Kutta stage (kStage 0 or 1) over the nx cells of one tube by the calling
+// One Runge-Kutta stage (kStage 0 or 1) of a single-precision state over the nx cells of one tube by the calling
 // block.  g, base and out point at the tube's first cell; planes are P apart.  The
 // arithmetic per cell is the flat (Ny = 1) stage of the single-grid kernels, with the
 // equilibrium in double, in df64 (kEq = kEqDF) or in single precision on the moment
@@ -93,26 +91,24 @@ __device__ __forceinline__ void load_state(const TS *g, long long P, int x, TS f
 // velocities are loaded and computed, each result is stored to its plane and to the
 // plane of its mirror image, and the equilibrium drops the terms of j_y = 0.  The
 // values are those of the general form.
-template <typename TS, int kStage, int kEq, bool kSym = false>
-__device__ __forceinline__ void tube_stage(const TS *g, const TS *base, TS *out, long long P,
-                                           const TubeInfo &t, const ClassConsts &C, TS a_self, TS a_base,
+template <int kStage, int kEq, bool kSym = false>
+__device__ __forceinline__ void tube_stage(const float *g, const float *base, float *out, long long P,
+                                           const TubeInfo &t, const ClassConsts &C, float a_self, float a_base,
                                            unsigned *flag)
 {
     constexpr bool kBase = kStage == 1;
     const int nx = t.nx;
-    const double *lx = t.lx[kStage];
     const float *lx_f = t.lx_f[kStage];
     for (int x = threadIdx.x; x < nx; x += blockDim.x) {
         const int xm2 = x >= 2 ? x - 2 : 0, xm1 = x >= 1 ? x - 1 : 0;
         const int xp1 = x + 1 < nx ? x + 1 : nx - 1, xp2 = x + 2 < nx ? x + 2 : nx - 1;
-        TS fs[kNV];
-        load_state<TS, kSym>(g, P, x, fs);
-        TS heq[kNV];
+        float fs[kNV];
+        load_state<kSym>(g, P, x, fs);
+        float heq[kNV];
         if constexpr (kEq == kEqF32) {
             // all 16 values (a symmetric state holds its mirror images in fs)
             f32_equilibrium(C.dfeq[kStage], C.dfm, t.dfs[kStage], C.dp[kStage], fs, heq, flag);
         } else if constexpr (kEq == kEqDF) {
-            static_assert(kSingle<TS>, "df64 equilibrium is for the single-precision state");
             if constexpr (kSym) df_equilibrium_sym(C.dfeq[kStage], C.dfm, t.dfs[kStage], fs, heq, flag);
             else df_equilibrium(C.dfeq[kStage], C.dfm, t.dfs[kStage], fs, heq, flag);
         } else {
@@ -121,28 +117,28 @@ __device__ __forceinline__ void tube_stage(const TS *g, const TS *base, TS *out,
             for (int i = 0; i < kNV; ++i) f[i] = widen(fs[i]);
             double h[kNV];
             if constexpr (kSym) {
-                const Prim s = primitives_sym<kSingle<TS>>(f, C.m, t.rhoF, t.EF, flag);
-                equilibrium_sym<kSingle<TS>>(C.eq[kStage], C.m, s.q.rho, s.q.E, s.q.jx, s.ux, s.ru2, s.p, s.T, h,
+                const Prim s = primitives_sym<true>(f, C.m, t.rhoF, t.EF, flag);
+                equilibrium_sym<true>(C.eq[kStage], C.m, s.q.rho, s.q.E, s.q.jx, s.ux, s.ru2, s.p, s.T, h,
                                              t.sF[kStage]);
             } else {
-                const Prim s = primitives<kSingle<TS>>(f, C.m, t.rhoF, t.EF, flag);
-                equilibrium<kSingle<TS>>(C.eq[kStage], C.m, s.q.rho, s.q.E, s.q.jx, s.q.jy, s.ux, s.uy, s.ru2,
+                const Prim s = primitives<true>(f, C.m, t.rhoF, t.EF, flag);
+                equilibrium<true>(C.eq[kStage], C.m, s.q.rho, s.q.E, s.q.jx, s.q.jy, s.ux, s.uy, s.ru2,
                                          s.jyuy, s.p, s.T, h, t.sF[kStage]);
             }
 #pragma unroll
-            for (int i = 0; i < kNV; ++i) heq[i] = narrow<TS>(h[i]);
+            for (int i = 0; i < kNV; ++i) heq[i] = narrow<float>(h[i]);
         }
 #pragma unroll
         for (int i = 0; i < kNV; ++i) {
             if (kSym && mirror_y(i) != i) continue;
-            TS o = fma_t(a_self, fs[i], heq[i]);
-            if (kBase) o = fma_t(a_base, base[i * P + x], o);
+            float o = fmaf(a_self, fs[i], heq[i]);
+            if (kBase) o = fmaf(a_base, base[i * P + x], o);
             if (dirx(i) != 0) {
-                const TS *gp = g + i * P;
-                const TS u2 = gp[dirx(i) > 0 ? xm2 : xp2];
-                const TS u1 = gp[dirx(i) > 0 ? xm1 : xp1];
-                const TS d1 = gp[dirx(i) > 0 ? xp1 : xm1];
-                o = fma_t(-pick<TS>(lx[i >> 2], lx_f[i >> 2]), nnd(u2, u1, fs[i], d1), o);
+                const float *gp = g + i * P;
+                const float u2 = gp[dirx(i) > 0 ? xm2 : xp2];
+                const float u1 = gp[dirx(i) > 0 ? xm1 : xp1];
+                const float d1 = gp[dirx(i) > 0 ? xp1 : xm1];
+                o = fmaf(-lx_f[i >> 2], nnd(u2, u1, fs[i], d1), o);
             }
             out[i * P + x] = o;
             if (kSym && sym_partner(i) >= 0) out[sym_partner(i) * P + x] = o;
@@ -150,96 +146,93 @@ __device__ __forceinline__ void tube_stage(const TS *g, const TS *base, TS *out,
     }
 }
 
-// The FP64 stage of one tube with the x differences shared: the block covers a chunk
-// of blockDim cells at a time; each thread computes U = f_x - f_{x-s} of its cell once
-// per velocity into a row buffer in shared memory, the chunk's edge threads add the
-// values beyond it (the tube's zero-gradient ends included, through the clamped
-// indices), and each cell reads U of its neighbours there: 4 instead of 6 FP64
-// instructions per x term, with the operands and operations of nnd(), so the result
-// is the same bit for bit.  All threads run the same chunk loop and reach the block
-// barriers.
-template <int kStage, int kThreads, bool kSym = false>
-__device__ __forceinline__ void tube_stage_shared_x(const double *g, const double *base, double *out, long long P,
-                                                    const TubeInfo &t, const ClassConsts &C, double a_self,
-                                                    double a_base, unsigned *flag, double (*row_u)[kThreads + 2])
+// Access to one cell of a tube for fx_rest_of_group(): zero-gradient ends; with kSym a
+// result goes to its plane and to that of its mirror image.
+template <bool kSym>
+struct TubeCell {
+    const double *g, *b;
+    double *out;
+    long long P;
+    int nx, x;
+    template <bool kFlatY>
+    __device__ __forceinline__ FxStencil stencil(int i, int dx, int, double base) const
+    {
+        auto at = [&](int j) { return g[i * P + (j < 0 ? 0 : (j >= nx ? nx - 1 : j))]; };
+        return {at(x), at(x - 2 * dx), at(x - dx), at(x + dx), 0, 0, 0, base};
+    }
+    __device__ __forceinline__ double base(int i) const { return b[i * P + x]; }
+    __device__ __forceinline__ void put(int i, double v) const
+    {
+        out[i * P + x] = v;
+        if (kSym && sym_partner(i) >= 0) out[sym_partner(i) * P + x] = v;
+    }
+};
+
+// The members of group grp of one cell of a tube (kSym: the distinct ones), one per pass.
+template <bool kDiag, int kStage, bool kSym>
+__device__ __forceinline__ void tube_group_fx(const TubeCell<kSym> &cell, const int xs[4], const TubeInfo &t,
+                                              const ClassConsts &C, const FxCoef &k, double a_self, double a_base,
+                                              int grp, const FxGroup h, bool cell_ok, unsigned *flag)
 {
-    // with kSym the mirror images SW, SE (the x-moving ones) are skipped: 8 x terms
-    auto xterm = [](int i) { return dirx(i) != 0 && (!kSym || mirror_y(i) == i); };
     constexpr bool kBase = kStage == 1;
+    const FxK lx = t.fx[kStage].klx[grp];
+    unsigned rest = 0;
+    auto pass = [&](int j, auto transport) {
+        constexpr bool kX = decltype(transport)::value;
+        const double *gp = cell.g + (4 * grp + j) * cell.P;
+        FxStencil v = {};
+        if (kBase) v.base = cell.b[(4 * grp + j) * cell.P + cell.x];
+        v.c = gp[cell.x];
+        if constexpr (kX) {
+            const bool west = kDiag ? j == 1 || j == 2 : j == 2;
+            v.x2 = gp[west ? xs[3] : xs[0]];
+            v.x1 = gp[west ? xs[2] : xs[1]];
+            v.xd = gp[west ? xs[1] : xs[2]];
+        }
+        double o;
+        const bool ok = fx_update<kX, false, kBase>(k, lx, lx, v, h.member(j), h.G, o);
+        if (ok && cell_ok) {
+            cell.out[(4 * grp + j) * cell.P + cell.x] = o;
+            // mirror images: S of N; SE of NE, SW of NW
+            if (kSym && (kDiag || j == 1)) cell.out[(4 * grp + (kDiag ? 3 - j : 3)) * cell.P + cell.x] = o;
+        } else {
+            rest |= 1u << j;
+        }
+    };
+    if constexpr (kDiag) {
+#pragma unroll 1
+        for (int j = 0; j < (kSym ? 2 : 4); ++j) pass(j, std::true_type{});
+    } else {
+#pragma unroll 1
+        for (int j = 0; j < 4; j += 2) pass(j, std::true_type{});
+#pragma unroll 1
+        for (int j = 1; j < (kSym ? 2 : 4); j += 2) pass(j, std::false_type{});     // N, S: no transport
+    }
+    if (rest)
+        fx_rest_of_group<TubeCell<kSym>, kBase, true>(cell, C.eq[kStage], C.m, k, t.fx[kStage],
+                                                      {a_self, a_base, t.lx[kStage], t.lx[kStage]}, grp, rest, cell_ok,
+                                                      h, flag);
+}
+
+// The FP64 stage of one tube (cdbm_stage_fx.cuh), one cell per thread.
+template <int kStage, bool kSym>
+__device__ __forceinline__ void tube_stage_fx(const double *g, const double *base, double *out, long long P,
+                                              const TubeInfo &t, const ClassConsts &C, const FxCoef &k, double a_self,
+                                              double a_base, unsigned *flag)
+{
     const int nx = t.nx;
-    const double *lx = t.lx[kStage];
-    const int tid = threadIdx.x;
-    for (int xb = 0; xb < nx; xb += kThreads) {
-        const int x = xb + tid;
-        const bool active = x < nx;
-        const int xc = active ? x : nx - 1;
-        const int last = (nx - xb < kThreads ? nx - xb : kThreads) - 1;      // last active thread
-        const int xm2 = xc >= 2 ? xc - 2 : 0, xm1 = xc >= 1 ? xc - 1 : 0;
-        const int xp1 = xc + 1 < nx ? xc + 1 : nx - 1, xp2 = xc + 2 < nx ? xc + 2 : nx - 1;
-        double fs[kNV], o[kNV];
-        if (active) {
-            load_state<double, kSym>(g, P, x, fs);
-            double heq[kNV];
-            if constexpr (kSym) {
-                const Prim s = primitives_sym<false>(fs, C.m, 0.0, 0.0, flag);
-                equilibrium_sym<false>(C.eq[kStage], C.m, s.q.rho, s.q.E, s.q.jx, s.ux, s.ru2, s.p, s.T, heq);
-            } else {
-                const Prim s = primitives<false>(fs, C.m, 0.0, 0.0, flag);
-                equilibrium<false>(C.eq[kStage], C.m, s.q.rho, s.q.E, s.q.jx, s.q.jy, s.ux, s.uy, s.ru2, s.jyuy,
-                                   s.p, s.T, heq);
-            }
-            int k = 0;
-#pragma unroll
-            for (int i = 0; i < kNV; ++i) {
-                if (kSym && mirror_y(i) != i) continue;
-                o[i] = fma(a_self, fs[i], heq[i]);
-                if (kBase) o[i] = fma(a_base, base[i * P + x], o[i]);
-                if (xterm(i)) {
-                    row_u[k][tid + 1] = fs[i] - g[i * P + (dirx(i) > 0 ? xm1 : xp1)];   // a of nnd()
-                    ++k;
-                }
-            }
-            if (tid == 0) {                           // U left of the chunk
-                int k2 = 0;
-#pragma unroll
-                for (int i = 0; i < kNV; ++i) {
-                    if (!xterm(i)) continue;
-                    const double *gp = g + i * P;
-                    row_u[k2][0] = dirx(i) > 0 ? gp[xm1] - gp[xm2] : gp[xm1] - fs[i];
-                    ++k2;
-                }
-            }
-            if (tid == last) {                        // U right of the chunk
-                int k2 = 0;
-#pragma unroll
-                for (int i = 0; i < kNV; ++i) {
-                    if (!xterm(i)) continue;
-                    const double *gp = g + i * P;
-                    row_u[k2][last + 2] = dirx(i) > 0 ? gp[xp1] - fs[i] : gp[xp1] - gp[xp2];
-                    ++k2;
-                }
-            }
+    for (int x = threadIdx.x; x < nx; x += blockDim.x) {
+        const int xs[4] = {x >= 2 ? x - 2 : 0, x >= 1 ? x - 1 : 0, x + 1 < nx ? x + 1 : nx - 1, x + 2 < nx ? x + 2 : nx - 1};
+        const TubeCell<kSym> cell = {g, base, out, P, nx, x};
+        const FxCons m = fx_conserved(C.fx, [=](int i) { return g[(kSym ? mirror_y(i) : i) * P + x]; });
+        const EqFactors q = kSym ? eq_factors_sym(C.m, m.rho, m.jx, m.E, flag) : eq_factors(C.m, m.rho, m.jx, m.jy, m.E, flag);
+#pragma unroll 1
+        for (int p = 0; p < 4; p += 2) {
+            tube_group_fx<false, kStage, kSym>(cell, xs, t, C, k, a_self, a_base, p, fx_group<kSym>(C.eq[kStage], q, p),
+                                               m.ok, flag);
+            tube_group_fx<true, kStage, kSym>(cell, xs, t, C, k, a_self, a_base, p + 1,
+                                              fx_group<kSym>(C.eq[kStage], q, p + 1), m.ok, flag);
         }
-        __syncthreads();
-        if (active) {
-            int k = 0;
-#pragma unroll
-            for (int i = 0; i < kNV; ++i) {
-                if (kSym && mirror_y(i) != i) continue;
-                if (xterm(i)) {
-                    const int s = dirx(i);
-                    const double av = row_u[k][tid + 1];          // c - u1
-                    const double bv = row_u[k][tid + 1 + s];      // d1 - c
-                    const double ev = row_u[k][tid + 1 - s];      // u1 - u2
-                    const double tt = minmod(bv, av) - minmod(av, ev);
-                    o[i] = fma(-lx[i >> 2], fma(0.5, tt, av), o[i]);
-                    ++k;
-                }
-                out[i * P + x] = o[i];
-                if (kSym && sym_partner(i) >= 0) out[sym_partner(i) * P + x] = o[i];
-            }
-        }
-        __syncthreads();                              // the next chunk rewrites the buffer
     }
 }
 
@@ -303,33 +296,32 @@ __device__ __forceinline__ void tube_stage2(const float *g, const float *base, f
     }
 }
 
-// Register budget (resident threads per SM the registers must allow): 384 for the
-// double-precision equilibrium (168 registers at 128 threads) and for the two-column
-// df64 one, whose two cells of float arithmetic take about as many.  The symmetric
-// forms keep less live state: 512 for FP64 and FP32_BULK (126 / 116 registers at
-// 128 threads, no spills; 1.97e9 / 3.05e9 against 1.95e9 / 2.90e9 cell-updates/s on
-// the 1024-tube ensemble) and 640 for df64 (96 registers; 1.13e10 against 1.07e10;
-// 768 spilled 380 bytes).  The one-cell deviation equilibrium fits 64 registers
-// without spills, so 1024 (32 warps per SM): 1.50e10 against 1.31e10 at 512 (127
-// registers); 1280 spilled and fell back to 1.32e10.
-constexpr int batch_thread_budget(int eq, bool sym)
+// Register budget (resident threads per SM the registers must allow).
+// FP64 (fixed-point form): 1024 for blocks of 256 threads (64 registers; 3.25e9
+// cell-updates/s on the 1024-tube ensemble at 4 blocks per SM, against 3.12e9 at a
+// budget of 512 or 640), 512 for narrower ones, whose tiles keep fewer warps (2.91e9 at
+// 128 x 4, against 2.69e9 at 1024).
+// FP32_BULK: 384 (168 registers at 128 threads), 512 in the symmetric form, which keeps
+// less live state (116 registers, 3.05e9 against 2.90e9).  Two-column df64: 384, 640 in
+// the symmetric form (96 registers; 1.13e10 against 1.07e10; 768 spilled 380 bytes).  The
+// one-cell deviation equilibrium fits 64 registers without spills, so 1024 (32 warps per
+// SM): 1.50e10 against 1.31e10 at 512 (127 registers); 1280 spilled and fell back to
+// 1.32e10.
+constexpr int batch_thread_budget(bool fp64, int threads, int eq, bool sym)
 {
+    if (fp64) return threads == 256 ? 1024 : 512;
     return eq == kEqF32 ? 1024 : (sym ? (eq == kEqDF ? 640 : 512) : 384);
 }
-constexpr int batch_min_blocks(int threads, int eq, bool sym)
+constexpr int batch_min_blocks(bool fp64, int threads, int eq, bool sym)
 {
-    return batch_thread_budget(eq, sym) / threads > 0 ? batch_thread_budget(eq, sym) / threads : 1;
+    return batch_thread_budget(fp64, threads, eq, sym) / threads > 0 ? batch_thread_budget(fp64, threads, eq, sym) / threads : 1;
 }
 
 template <typename TS, int kThreads, int kEq, bool kSym>
-__global__ void __launch_bounds__(kThreads, batch_min_blocks(kThreads, kEq, kSym)) batch_kernel(TS *f, TS *f1, const TubeInfo *tubes,
+__global__ void __launch_bounds__(kThreads, batch_min_blocks(!kSingle<TS>, kThreads, kEq, kSym)) batch_kernel(TS *f, TS *f1, const TubeInfo *tubes,
                                                          const int *work, const int *work_off, int nsteps,
-                                                         const BatchArgs a, unsigned *flag)
+                                                         const __grid_constant__ BatchArgs a, unsigned *flag)
 {
-    const TS as0 = pick<TS>(a.a_self[0], a.a_self_f[0]), as1 = pick<TS>(a.a_self[1], a.a_self_f[1]);
-    const TS ab0 = pick<TS>(a.a_base[0], a.a_base_f[0]), ab1 = pick<TS>(a.a_base[1], a.a_base_f[1]);
-    // x row buffer of the FP64 stage (a placeholder for the single-precision states)
-    __shared__ double row_u[kSingle<TS> ? 1 : 12][kSingle<TS> ? 1 : kThreads + 2];
     for (int w = work_off[blockIdx.x]; w < work_off[blockIdx.x + 1]; ++w) {
         const TubeInfo &t = tubes[work[w]];
         const ClassConsts &C = a.cls[t.cls];
@@ -337,17 +329,17 @@ __global__ void __launch_bounds__(kThreads, batch_min_blocks(kThreads, kEq, kSym
         TS *f1t = f1 + t.offset;
         for (int s = 0; s < nsteps; ++s) {
             if constexpr (!kSingle<TS>) {
-                tube_stage_shared_x<0, kThreads, kSym>(ft, nullptr, f1t, a.P, t, C, as0, ab0, flag, row_u);
+                tube_stage_fx<0, kSym>(ft, nullptr, f1t, a.P, t, C, a.fx[0], a.a_self[0], a.a_base[0], flag);
                 __syncthreads();
-                tube_stage_shared_x<1, kThreads, kSym>(f1t, ft, ft, a.P, t, C, as1, ab1, flag, row_u);
+                tube_stage_fx<1, kSym>(f1t, ft, ft, a.P, t, C, a.fx[1], a.a_self[1], a.a_base[1], flag);
             } else if constexpr (kEq == kEqDF) {
                 tube_stage2<0, kSym>(ft, nullptr, f1t, a.P, t, C, a.a_self_f2[0], a.a_base_f2[0], flag);
                 __syncthreads();
                 tube_stage2<1, kSym>(f1t, ft, ft, a.P, t, C, a.a_self_f2[1], a.a_base_f2[1], flag);
             } else {
-                tube_stage<TS, 0, kEq, kSym>(ft, nullptr, f1t, a.P, t, C, as0, ab0, flag);
+                tube_stage<0, kEq, kSym>(ft, nullptr, f1t, a.P, t, C, a.a_self_f[0], a.a_base_f[0], flag);
                 __syncthreads();
-                tube_stage<TS, 1, kEq, kSym>(f1t, ft, ft, a.P, t, C, as1, ab1, flag);
+                tube_stage<1, kEq, kSym>(f1t, ft, ft, a.P, t, C, a.a_self_f[1], a.a_base_f[1], flag);
             }
             __syncthreads();
         }
@@ -680,6 +672,7 @@ cdbm_status cdbm_batch_create(int ntubes, const int *nx, const double *dx, const
     for (int s = 0; s < 2; ++s) {
         b->args.a_self[s] = beta[s] - gamma[s] * h;
         b->args.a_base[s] = alpha[s];
+        b->args.fx[s] = fx_coef(b->args.a_self[s], b->args.a_base[s]);
         b->args.a_self_f[s] = (float)b->args.a_self[s];
         b->args.a_base_f[s] = (float)b->args.a_base[s];
         b->args.a_self_f2[s] = make_float2(b->args.a_self_f[s], b->args.a_self_f[s]);
@@ -718,6 +711,7 @@ cdbm_status cdbm_batch_create(int ntubes, const int *nx, const double *dx, const
             }
             C.dfm = df_model(C.m);
             C.dfm2 = df_model_twice(C.dfm);
+            C.fx = fx_model(C.m.c, C.m.w);
             for (int s = 0; s < 2; ++s) C.dp[s] = dev_proj(C.m, gamma[s] * h);
         }
         TubeInfo &ti = b->info[t];
@@ -731,6 +725,7 @@ cdbm_status cdbm_batch_create(int ntubes, const int *nx, const double *dx, const
                 ti.lx_f[s][g] = (float)ti.lx[s][g];
                 ti.lx_f2[s][g] = make_float2(ti.lx_f[s][g], ti.lx_f[s][g]);
             }
+        for (int s = 0; s < 2; ++s) ti.fx[s] = fx_flux(ti.lx[s], ti.lx[s], nx[t] > 1, false);
         b->offs[t + 1] = b->offs[t] + nx[t];
     }
     b->P = b->offs[ntubes];

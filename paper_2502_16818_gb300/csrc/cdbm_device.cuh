@@ -389,4 +389,12 @@ __device__ __forceinline__ int neighbour(int j, int n, int bc)
     return j < 0 ? 0 : (j >= n ? n - 1 : j);
 }
 
+// neighbour() for -2 <= j <= n + 1, without the integer division.
+__device__ __forceinline__ int neighbour_near(int j, int n, int bc)
+{
+    if (bc != 0) return j < 0 ? 0 : (j >= n ? n - 1 : j);
+    if (n == 1) return 0;
+    return j < 0 ? j + n : (j >= n ? j - n : j);
+}
+
 }  // namespace cdbm

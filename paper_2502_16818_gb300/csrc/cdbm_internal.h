@@ -6,6 +6,7 @@
 #include <cstddef>
 
 #include "../../include/cdbm.h"
+#include "cdbm_fixed.h"
 
 namespace cdbm {
 
@@ -127,6 +128,7 @@ struct StageArgs {
     DevProj dp;                   // conservation projection (CDBM_FP32_DEV)
     float2 a_base_f2, a_self_f2;  // a_base_f, a_self_f, lx_f, ly_f twice
     float2 lx_f2[4], ly_f2[4];
+    FxStage fx;                   // fixed-point constants of the FP64 stage
     int nx, ny;
     int bc_x, bc_y;
 };
@@ -189,8 +191,9 @@ StageLaunch stage_launch_config(const StageArgs &a, bool with_base, int sm_count
 // FP64 stage kernel for 1-D grids with each cell split over four threads
 // (cdbm_small1d.cu): kSplitFlatThreads threads per block, 4 nx threads in all.
 constexpr int kSplitFlatThreads = 128;
-constexpr int kSplitFlatMaxCells = 8192;    // measured per stage: 8.8 against 10.0 us at 8192 cells,
-                                            // 16.3 against 10.7 us at 16384
+constexpr int kSplitFlatMaxCells = 4096;    // measured per stage against the fixed-point form with a
+                                            // warp per group: 5.6 / 6.4 us at 2000 cells, 5.4 / 6.3 at
+                                            // 4096, 8.8 / 6.4 at 8192
 void *split_flat_func(bool with_base);
 cudaError_t launch_stage(const StageLaunch &L, const void *g, const void *base, void *out,
                          const StageArgs &a, unsigned *flag, cudaStream_t s);
@@ -233,6 +236,8 @@ void fill_df_consts(StageArgs &a);
 // The conservation projection of a stage whose blocks are scaled by gh = gamma h.
 DevProj dev_proj(const ModelConsts &m, double gh);
 void fill_dev_proj(StageArgs &a, double gh);
+// Fills a.fx from the double constants of a (CDBM_FP64).
+void fill_fx_consts(StageArgs &a);
 // The same constants with each value twice, for the two-column (packed FP32x2) kernels.
 DFBlocksT<float2> df_blocks_twice(const DFBlocks &d);
 DFModelT<float2> df_model_twice(const DFModel &d);

@@ -13,6 +13,7 @@
 // row-marching kernels give each thread one column (two for the df64 and deviation states) over a
 // run of rows.
 #include "cdbm_stage.cuh"
+#include "cdbm_stage_fx.cuh"
 
 namespace cdbm {
 
@@ -67,122 +68,293 @@ __global__ void __launch_bounds__(128) init_kernel(const FieldArgs a, const doub
 
 // out = a_base base + a_self g + gamma h f_eq(g) - sum_r l_r D_r(g) for one cell:
 // macros -> equilibrium -> BGK -> NND transport of all 16 velocities -> update.
-template <typename TS, bool kBase, bool kFlatY, int kEq>
+template <bool kBase, bool kFlatY, int kEq>
 __global__ void __launch_bounds__(kStageThreads, stage_min_blocks(kEq))
-    stage_kernel(const TS *__restrict__ g, const TS *base, TS *out, const StageArgs a, unsigned *flag)
+    stage_kernel(const float *__restrict__ g, const float *base, float *out, const StageArgs a, unsigned *flag)
 {
     const int nx = a.nx, ny = a.ny;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= nx) return;
     const size_t P = (size_t)nx * ny;
-    const int xm2 = neighbour(x - 2, nx, a.bc_x), xm1 = neighbour(x - 1, nx, a.bc_x);
-    const int xp1 = neighbour(x + 1, nx, a.bc_x), xp2 = neighbour(x + 2, nx, a.bc_x);
+    const int xm2 = neighbour_near(x - 2, nx, a.bc_x), xm1 = neighbour_near(x - 1, nx, a.bc_x);
+    const int xp1 = neighbour_near(x + 1, nx, a.bc_x), xp2 = neighbour_near(x + 2, nx, a.bc_x);
     for (int y = blockIdx.y; y < ny; y += gridDim.y) {
         const size_t row = (size_t)y * nx;
         const size_t c = row + x;
         size_t rm2 = 0, rm1 = 0, rp1 = 0, rp2 = 0;
         if (!kFlatY) {
-            rm2 = (size_t)neighbour(y - 2, ny, a.bc_y) * nx + x;
-            rm1 = (size_t)neighbour(y - 1, ny, a.bc_y) * nx + x;
-            rp1 = (size_t)neighbour(y + 1, ny, a.bc_y) * nx + x;
-            rp2 = (size_t)neighbour(y + 2, ny, a.bc_y) * nx + x;
+            rm2 = (size_t)neighbour_near(y - 2, ny, a.bc_y) * nx + x;
+            rm1 = (size_t)neighbour_near(y - 1, ny, a.bc_y) * nx + x;
+            rp1 = (size_t)neighbour_near(y + 1, ny, a.bc_y) * nx + x;
+            rp2 = (size_t)neighbour_near(y + 2, ny, a.bc_y) * nx + x;
         }
-        TS fs[kNV];
+        float fs[kNV];
 #pragma unroll
         for (int i = 0; i < kNV; ++i) fs[i] = __ldg(g + i * P + c);
-        TS heq[kNV];
-        stage_equilibrium<TS, kEq>(a, fs, heq, flag);
+        float heq[kNV];
+        stage_equilibrium<kEq>(a, fs, heq, flag);
 
 #pragma unroll
         for (int i = 0; i < kNV; ++i) {
             const int grp = i >> 2;
-            const TS *gp = g + i * P;
-            TS o = fma_t(a_self_of<TS>(a), fs[i], heq[i]);
-            if (kBase) o = fma_t(a_base_of<TS>(a), base[i * P + c], o);
+            const float *gp = g + i * P;
+            float o = fmaf(a.a_self_f, fs[i], heq[i]);
+            if (kBase) o = fmaf(a.a_base_f, base[i * P + c], o);
             if (dirx(i) != 0) {
-                const TS u2 = __ldg(gp + row + (dirx(i) > 0 ? xm2 : xp2));
-                const TS u1 = __ldg(gp + row + (dirx(i) > 0 ? xm1 : xp1));
-                const TS d1 = __ldg(gp + row + (dirx(i) > 0 ? xp1 : xm1));
-                o = fma_t(-lx_of<TS>(a, grp), nnd(u2, u1, fs[i], d1), o);
+                const float u2 = __ldg(gp + row + (dirx(i) > 0 ? xm2 : xp2));
+                const float u1 = __ldg(gp + row + (dirx(i) > 0 ? xm1 : xp1));
+                const float d1 = __ldg(gp + row + (dirx(i) > 0 ? xp1 : xm1));
+                o = fmaf(-a.lx_f[grp], nnd(u2, u1, fs[i], d1), o);
             }
             if (!kFlatY && diry(i) != 0) {
-                const TS u2 = __ldg(gp + (diry(i) > 0 ? rm2 : rp2));
-                const TS u1 = __ldg(gp + (diry(i) > 0 ? rm1 : rp1));
-                const TS d1 = __ldg(gp + (diry(i) > 0 ? rp1 : rm1));
-                o = fma_t(-ly_of<TS>(a, grp), nnd(u2, u1, fs[i], d1), o);
+                const float u2 = __ldg(gp + (diry(i) > 0 ? rm2 : rp2));
+                const float u1 = __ldg(gp + (diry(i) > 0 ? rm1 : rp1));
+                const float d1 = __ldg(gp + (diry(i) > 0 ? rp1 : rm1));
+                o = fmaf(-a.ly_f[grp], nnd(u2, u1, fs[i], d1), o);
             }
             out[i * P + c] = o;
         }
     }
 }
 
-// Same stage for 2-D grids with the y-direction differences shared along a run of
-// rows.  A block covers kStageThreads columns and a run of R = ceil(ny / gridDim.y)
-// rows; each thread marches up its column.  For a velocity with y-sign s the
-// upwind-ordered difference U_y = f_y - f_{y-s} and N_y = minmod(U_{y+s}, U_y) give
-// the transport difference U_y + (N_y - N_{y-s}) / 2, which is the nnd() expression
-// with a = U_y, b = U_{y-s}, e = U_{y+s}.  Each row computes one new U and one new N
-// per velocity and carries them to the next row in shared memory, so a y-term costs
-// 4 instead of 6 arithmetic instructions, with the same operations as stage_kernel.
+// Row pointers and offsets of a cell's stencil.  The row pointers are uniform over a
+// block, the offsets in a row 32 bits wide (kWide: 64 bits, for rows of 2^29 cells and
+// more), which saves the 64-bit address arithmetic of about 100 loads per cell.
+template <bool kWide>
+struct GridStencil {
+    using Off = std::conditional_t<kWide, size_t, unsigned>;
+    Off c, m2, m1, p1, p2;
+    size_t row, rm2, rm1, rp1, rp2;
+    __device__ __forceinline__ GridStencil(int x, int nx, int bc)
+        : c((Off)8 * x), m2((Off)8 * neighbour_near(x - 2, nx, bc)), m1((Off)8 * neighbour_near(x - 1, nx, bc)),
+          p1((Off)8 * neighbour_near(x + 1, nx, bc)), p2((Off)8 * neighbour_near(x + 2, nx, bc))
+    {
+    }
+    template <bool kFlatY>
+    __device__ __forceinline__ void at_row(int y, int nx, int ny, int bc)
+    {
+        row = (size_t)y * nx;
+        if (!kFlatY) {
+            rm2 = (size_t)neighbour_near(y - 2, ny, bc) * nx;
+            rm1 = (size_t)neighbour_near(y - 1, ny, bc) * nx;
+            rp1 = (size_t)neighbour_near(y + 1, ny, bc) * nx;
+            rp2 = (size_t)neighbour_near(y + 2, ny, bc) * nx;
+        }
+    }
+    static __device__ __forceinline__ double get(const double *p, Off o) { return __ldg((const double *)((const char *)p + o)); }
+};
+
+// Access to one cell of a grid for fx_rest_of_group().
+struct GridCell {
+    const double *g, *b;
+    double *out;
+    int nx, ny, bc_x, bc_y, x, y;
+    __device__ __forceinline__ size_t at(int i) const { return (size_t)i * nx * ny + (size_t)y * nx + x; }
+    // any direction signs, 0 included
+    template <bool kFlatY>
+    __device__ __forceinline__ FxStencil stencil(int i, int dx, int dy, double base) const
+    {
+        const double *gp = g + (size_t)i * nx * ny, *gr = gp + (size_t)y * nx;
+        FxStencil v = {gr[x], gr[neighbour_near(x - 2 * dx, nx, bc_x)], gr[neighbour_near(x - dx, nx, bc_x)],
+                       gr[neighbour_near(x + dx, nx, bc_x)], 0, 0, 0, base};
+        if (!kFlatY) {
+            v.y2 = gp[(size_t)neighbour_near(y - 2 * dy, ny, bc_y) * nx + x];
+            v.y1 = gp[(size_t)neighbour_near(y - dy, ny, bc_y) * nx + x];
+            v.yd = gp[(size_t)neighbour_near(y + dy, ny, bc_y) * nx + x];
+        }
+        return v;
+    }
+    __device__ __forceinline__ double base(int i) const { return b[at(i)]; }
+    __device__ __forceinline__ void put(int i, double v) const { out[at(i)] = v; }
+};
+
+// The four members of group grp of one cell: loads, update and stores, one member per
+// pass.  The passes differ in the offsets of the neighbours only and share their code:
+// unrolled, the members' independent chains overlap (6.9 ms per 4096^2 step at 12
+// warps per SM, 7.0 as here at 32), but the code outgrows the instruction cache as soon
+// as other paths run beside it (1500 x 1300 piecewise-constant fields: 1.9 against
+// 1.27 ms).
+template <bool kDiag, bool kFlatY, bool kBase, bool kWide>
+__device__ __forceinline__ void fx_grid_group(const double *g, const double *base, double *out, const StageArgs &a,
+                                              const GridStencil<kWide> &st, size_t P, int x, int y, int grp,
+                                              const FxGroup h, bool cell_ok, bool live, unsigned *flag)
+{
+    using St = GridStencil<kWide>;
+    unsigned rest = 0;
+    auto pass = [&](int j, auto transport) {
+        constexpr bool kX = decltype(transport)::value, kY = kDiag && !kFlatY && kX;
+        const size_t plane = (4 * grp + j) * P;
+        const double *gp = g + plane, *gr = gp + st.row;
+        FxStencil v = {};
+        if (kBase) v.base = *(const double *)((const char *)(base + plane + st.row) + st.c);
+        v.c = St::get(gr, st.c);
+        if constexpr (kX && (kDiag || kFlatY)) {
+            const bool west = kDiag ? j == 1 || j == 2 : j == 2;
+            v.x2 = St::get(gr, west ? st.p2 : st.m2);
+            v.x1 = St::get(gr, west ? st.p1 : st.m1);
+            v.xd = St::get(gr, west ? st.m1 : st.p1);
+            if constexpr (kY) {
+                v.y2 = St::get(gp + (j < 2 ? st.rm2 : st.rp2), st.c);
+                v.y1 = St::get(gp + (j < 2 ? st.rm1 : st.rp1), st.c);
+                v.yd = St::get(gp + (j < 2 ? st.rp1 : st.rm1), st.c);
+            }
+        } else if constexpr (kX) {     // E, W along x; N, S along y
+            const bool up = j & 1, neg = j >= 2;
+            v.x2 = St::get(gp + (up ? (neg ? st.rp2 : st.rm2) : st.row), up ? st.c : (neg ? st.p2 : st.m2));
+            v.x1 = St::get(gp + (up ? (neg ? st.rp1 : st.rm1) : st.row), up ? st.c : (neg ? st.p1 : st.m1));
+            v.xd = St::get(gp + (up ? (neg ? st.rm1 : st.rp1) : st.row), up ? st.c : (neg ? st.m1 : st.p1));
+        }
+        const FxK kx = !kDiag && !kFlatY && (j & 1) ? a.fx.l.kly[grp] : a.fx.l.klx[grp];
+        double o;
+        const bool ok = fx_update<kX, kY, kBase>(a.fx.k, kx, a.fx.l.kly[grp], v, h.member(j), h.G, o);
+        if (live && ok && cell_ok) *(double *)((char *)(out + plane + st.row) + st.c) = o;
+        else rest |= 1u << j;
+    };
+    if constexpr (!kDiag && kFlatY) {
+#pragma unroll 1
+        for (int j = 0; j < 4; j += 2) pass(j, std::true_type{});
+#pragma unroll 1
+        for (int j = 1; j < 4; j += 2) pass(j, std::false_type{});    // N, S of a 1-D grid: no transport
+    } else {
+#pragma unroll 1
+        for (int j = 0; j < 4; ++j) pass(j, std::true_type{});
+    }
+    if (rest && live)
+        fx_rest_of_group<GridCell, kBase, kFlatY>({g, base, out, a.nx, a.ny, a.bc_x, a.bc_y, x, y}, a.eq, a.m, a.fx.k,
+                                                  a.fx.l, {a.a_self, a.a_base, a.lx, a.ly}, grp, rest, cell_ok, h, flag);
+}
+
+// Stage in double precision, one cell per thread (cdbm_stage_fx.cuh).  Bound by the
+// issue of about 4100 integer instructions per cell and stage (against 246 / 262 FP64
+// instructions of 64 cycles each); 64 registers for 32 warps per SM, which hide the
+// latency of its dependent chains (7.1 ms per 4096^2 step; 7.6 at 24 warps, 8.2 at 16).
+constexpr int kFxMinBlocks = 8;
+template <bool kBase, bool kFlatY, bool kWide>
+__global__ void __launch_bounds__(kStageThreads, kFxMinBlocks)
+    stage_fx_kernel(const double *__restrict__ g, const double *base, double *out, const __grid_constant__ StageArgs a,
+                    unsigned *flag)
+{
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= a.nx) return;
+    const size_t P = (size_t)a.nx * a.ny;
+    GridStencil<kWide> st(x, a.nx, a.bc_x);
+    for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
+        st.template at_row<kFlatY>(y, a.nx, a.ny, a.bc_y);
+        const double *own = g + st.row + x;
+        const FxCons m = fx_conserved(a.fx.m, [=](int i) { return __ldg(own + i * P); });
+        const EqFactors q = eq_factors(a.m, m.rho, m.jx, m.jy, m.E, flag);
+#pragma unroll 1
+        for (int p = 0; p < 4; p += 2) {
+            fx_grid_group<false, kFlatY, kBase>(g, base, out, a, st, P, x, y, p, fx_group(a.eq, q, p), m.ok, true, flag);
+            fx_grid_group<true, kFlatY, kBase>(g, base, out, a, st, P, x, y, p + 1, fx_group(a.eq, q, p + 1), m.ok, true,
+                                               flag);
+        }
+    }
+}
+
+// The same stage with the four velocity groups of 32 cells on the four warps of a block:
+// on a small grid the time of a stage is the chain of one thread, which this shortens
+// about threefold.  The warps exchange the groups' largest exponents and sums through
+// shared memory, and each forms the moments and the factors of the equilibrium; the
+// values are those of stage_fx_kernel.
+template <bool kBase, bool kFlatY>
+__global__ void __launch_bounds__(128)
+    stage_fx_split_kernel(const double *__restrict__ g, const double *base, double *out,
+                          const __grid_constant__ StageArgs a, unsigned *flag)
+{
+    __shared__ uint32_t keys[4][32];
+    __shared__ int64_t sums[4][3][32];
+    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    const int x0 = blockIdx.x * 32 + lane;
+    const bool live = x0 < a.nx;
+    const int x = live ? x0 : a.nx - 1;              // idle lanes mirror the last cell
+    const size_t P = (size_t)a.nx * a.ny;
+    GridStencil<true> st(x, a.nx, a.bc_x);
+    for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
+        st.template at_row<kFlatY>(y, a.nx, a.ny, a.bc_y);
+        const double *own = g + (size_t)(4 * grp) * P + st.row + x;
+        double f[4];
+        uint32_t key = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            f[j] = __ldg(own + j * P);
+            key = fx_max(key, fx_key(f[j]));
+        }
+        keys[grp][lane] = key;
+        __syncthreads();
+        const int top = (int)(fx_max(fx_max(keys[0][lane], keys[1][lane]), fx_max(keys[2][lane], keys[3][lane])) >> 21);
+        int64_t q4[4], s0, sx, sy;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) q4[j] = fx_from(f[j], top);
+        fx_group_sums(grp, q4, s0, sx, sy);
+        sums[grp][0][lane] = s0;
+        sums[grp][1][lane] = sx;
+        sums[grp][2][lane] = sy;
+        __syncthreads();
+        FxMoments mo = kFxNoMoments;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) fx_add_sums(a.fx.m, h, sums[h][0][lane], sums[h][1][lane], sums[h][2][lane], mo);
+        const FxCons m = fx_round_moments(a.fx.m, mo, top);
+        const EqFactors q = eq_factors(a.m, m.rho, m.jx, m.jy, m.E, flag);
+        const FxGroup h = fx_group(a.eq, q, grp);
+        if ((grp & 1) == 0) fx_grid_group<false, kFlatY, kBase>(g, base, out, a, st, P, x, y, grp, h, m.ok, live, flag);
+        else fx_grid_group<true, kFlatY, kBase>(g, base, out, a, st, P, x, y, grp, h, m.ok, live, flag);
+        // the next row writes keys[] only after every warp has passed the second barrier
+    }
+}
+
+// Stage of the CDBM_FP32_BULK state on 2-D grids with the y-direction differences shared
+// along a run of rows.  A block covers kStageThreads columns and a run of
+// R = ceil(ny / gridDim.y) rows; each thread marches up its column.  For a velocity with
+// y-sign s the upwind-ordered difference U_y = f_y - f_{y-s} and
+// N_y = minmod(U_{y+s}, U_y) give the transport difference U_y + (N_y - N_{y-s}) / 2,
+// which is the nnd() expression with a = U_y, b = U_{y-s}, e = U_{y+s}.  Each row
+// computes one new U and one new N per velocity and carries them to the next row in
+// shared memory, so a y-term costs 4 instead of 6 arithmetic instructions, with the same
+// operations as stage_kernel.
 constexpr int kNY = 12;                             // velocities with a y-component
-constexpr size_t kMarchRowBytes = 2 * 12 * (kStageThreads + 2) * sizeof(double);   // FP64 x row buffers
 __host__ __device__ constexpr int yvel(int k)       // k-th velocity with diry != 0
 {
     return k < 2 ? 1 + 2 * k : (k < 6 ? k + 2 : (k < 8 ? 9 + 2 * (k - 6) : k + 4));
 }
 
-template <typename TS, bool kBase, int kEq>
-__global__ void __launch_bounds__(kStageThreads, stage_min_blocks(kEq))
-    stage_march_kernel(const TS *__restrict__ g, const TS *base, TS *out, const StageArgs a, unsigned *flag)
+template <bool kBase>
+__global__ void __launch_bounds__(kStageThreads, stage_min_blocks(kEqDouble))
+    stage_march_kernel(const float *__restrict__ g, const float *base, float *out, const StageArgs a, unsigned *flag)
 {
-    // In double precision the x differences are shared as well: each thread computes
-    // U_x = f_x - f_{x-s} of its cell once per velocity and reads U_{x+s}, U_{x-s} of
-    // its neighbours from a row buffer (double-buffered in dynamic shared memory, so
-    // one block barrier per row; the edge threads add the halo values), so an x-term
-    // costs 4 FP64 instructions plus a share of the halo instead of 6.  The operands and operations are those of nnd(), so the
-    // result is the same bit for bit.  In single precision the FP32 arithmetic is not
-    // the scarce unit and the plain three-load form is kept.
-    constexpr bool kShareX = !kSingle<TS>;
-    constexpr int kNXV = 12;                          // velocities with an x component
-    __shared__ TS carry_u[kNY][kStageThreads];
-    __shared__ TS carry_n[kNY][kStageThreads];
-    extern __shared__ __align__(16) unsigned char march_dyn[];   // [2][kNXV][kStageThreads + 2] TS
-    TS(*const row_buf)[kStageThreads + 2] = reinterpret_cast<TS(*)[kStageThreads + 2]>(march_dyn);
+    __shared__ float carry_u[kNY][kStageThreads];
+    __shared__ float carry_n[kNY][kStageThreads];
     const int nx = a.nx, ny = a.ny;
     const int tid = threadIdx.x;
     const int x = blockIdx.x * blockDim.x + tid;
-    const bool active = x < nx;
-    if (!kShareX && !active) return;
+    if (x >= nx) return;                              // no block barriers below
     const int R = (ny + gridDim.y - 1) / gridDim.y;
     const int y0 = blockIdx.y * R;
     const int y1 = y0 + R < ny ? y0 + R : ny;
-    if (y0 >= y1) return;                             // the same for the whole block
-    const int last = (nx - (int)(blockIdx.x * blockDim.x) < (int)blockDim.x
-                          ? nx - (int)(blockIdx.x * blockDim.x) : (int)blockDim.x) - 1;   // last active thread
+    if (y0 >= y1) return;
     const size_t P = (size_t)nx * ny;
-    const int xc = active ? x : nx - 1;               // inactive threads only pass the barriers
-    const int xm2 = neighbour(xc - 2, nx, a.bc_x), xm1 = neighbour(xc - 1, nx, a.bc_x);
-    const int xp1 = neighbour(xc + 1, nx, a.bc_x), xp2 = neighbour(xc + 2, nx, a.bc_x);
+    const int xm2 = neighbour_near(x - 2, nx, a.bc_x), xm1 = neighbour_near(x - 1, nx, a.bc_x);
+    const int xp1 = neighbour_near(x + 1, nx, a.bc_x), xp2 = neighbour_near(x + 2, nx, a.bc_x);
 
     // prologue: U_{y0} and N_{y0 - 1} for s = +1, N_{y0} for s = -1
-    if (active) {
+    {
         const size_t r0 = (size_t)y0 * nx + x;
-        const size_t rm1 = (size_t)neighbour(y0 - 1, ny, a.bc_y) * nx + x;
-        const size_t rm2 = (size_t)neighbour(y0 - 2, ny, a.bc_y) * nx + x;
-        const size_t rp1 = (size_t)neighbour(y0 + 1, ny, a.bc_y) * nx + x;
+        const size_t rm1 = (size_t)neighbour_near(y0 - 1, ny, a.bc_y) * nx + x;
+        const size_t rm2 = (size_t)neighbour_near(y0 - 2, ny, a.bc_y) * nx + x;
+        const size_t rp1 = (size_t)neighbour_near(y0 + 1, ny, a.bc_y) * nx + x;
 #pragma unroll
         for (int k = 0; k < kNY; ++k) {
             const int i = yvel(k);
-            const TS *gp = g + i * P;
-            const TS f0 = __ldg(gp + r0), fm1 = __ldg(gp + rm1);
+            const float *gp = g + i * P;
+            const float f0 = __ldg(gp + r0), fm1 = __ldg(gp + rm1);
             if (diry(i) > 0) {
-                const TS u = f0 - fm1;                    // U_{y0}
-                const TS um = fm1 - __ldg(gp + rm2);      // U_{y0-1}
+                const float u = f0 - fm1;                 // U_{y0}
+                const float um = fm1 - __ldg(gp + rm2);   // U_{y0-1}
                 carry_u[k][tid] = u;
                 carry_n[k][tid] = minmod(u, um);          // N_{y0-1}
             } else {
-                const TS u = f0 - __ldg(gp + rp1);        // U_{y0}
-                const TS um = fm1 - f0;                   // U_{y0-1}
+                const float u = f0 - __ldg(gp + rp1);     // U_{y0}
+                const float um = fm1 - f0;                // U_{y0-1}
                 carry_u[k][tid] = u;
                 carry_n[k][tid] = minmod(um, u);          // N_{y0}
             }
@@ -191,103 +363,49 @@ __global__ void __launch_bounds__(kStageThreads, stage_min_blocks(kEq))
 
     for (int y = y0; y < y1; ++y) {
         const size_t row = (size_t)y * nx;
-        const size_t c = row + xc;
-        // row y writes buffer y & 1; its readers have passed the next row's barrier
-        // before row y + 2 writes the same buffer again
-        TS(*const row_u)[kStageThreads + 2] = row_buf + (kShareX ? (y & 1) * kNXV : 0);
-        TS fs[kNV], o[kNV];
-        if (active) {
+        const size_t c = row + x;
+        float fs[kNV], o[kNV], heq[kNV];
 #pragma unroll
-            for (int i = 0; i < kNV; ++i) fs[i] = __ldg(g + i * P + c);
-            TS heq[kNV];
-            stage_equilibrium<TS, kEq>(a, fs, heq, flag);
-            int k = 0;
+        for (int i = 0; i < kNV; ++i) fs[i] = __ldg(g + i * P + c);
+        stage_equilibrium<kEqDouble>(a, fs, heq, flag);
 #pragma unroll
-            for (int i = 0; i < kNV; ++i) {
-                o[i] = fma_t(a_self_of<TS>(a), fs[i], heq[i]);
-                if (kBase) o[i] = fma_t(a_base_of<TS>(a), base[i * P + c], o[i]);
-                if (dirx(i) != 0) {
-                    const TS *gp = g + i * P + row;
-                    const TS u1 = __ldg(gp + (dirx(i) > 0 ? xm1 : xp1));
-                    if constexpr (kShareX) {
-                        row_u[k][tid + 1] = fs[i] - u1;            // U at x: the upwind-ordered a of nnd()
-                    } else {
-                        const TS u2 = __ldg(gp + (dirx(i) > 0 ? xm2 : xp2));
-                        const TS d1 = __ldg(gp + (dirx(i) > 0 ? xp1 : xm1));
-                        o[i] = fma_t(-lx_of<TS>(a, i >> 2), nnd(u2, u1, fs[i], d1), o[i]);
-                    }
-                    ++k;
-                }
+        for (int i = 0; i < kNV; ++i) {
+            o[i] = fmaf(a.a_self_f, fs[i], heq[i]);
+            if (kBase) o[i] = fmaf(a.a_base_f, base[i * P + c], o[i]);
+            if (dirx(i) != 0) {
+                const float *gp = g + i * P + row;
+                const float u1 = __ldg(gp + (dirx(i) > 0 ? xm1 : xp1));
+                const float u2 = __ldg(gp + (dirx(i) > 0 ? xm2 : xp2));
+                const float d1 = __ldg(gp + (dirx(i) > 0 ? xp1 : xm1));
+                o[i] = fmaf(-a.lx_f[i >> 2], nnd(u2, u1, fs[i], d1), o[i]);
             }
         }
-        if constexpr (kShareX) {
-            // Halo of the row buffer: U_{x-1} left of the block and U_{x+1} right of it (the
-            // e or b of nnd() of the edge cells).  One branch taken by the edge threads only,
-            // so the other warps do not issue these instructions.
-            if (active && tid == 0) {
-                int k = 0;
+        const size_t rp1 = (size_t)neighbour_near(y + 1, ny, a.bc_y) * nx + x;
+        const size_t rp2 = (size_t)neighbour_near(y + 2, ny, a.bc_y) * nx + x;
 #pragma unroll
-                for (int i = 0; i < kNV; ++i) {
-                    if (dirx(i) == 0) continue;
-                    const TS *gp = g + i * P + row;
-                    row_u[k][0] = dirx(i) > 0 ? __ldg(gp + xm1) - __ldg(gp + xm2) : __ldg(gp + xm1) - fs[i];
-                    ++k;
-                }
+        for (int k = 0; k < kNY; ++k) {
+            const int i = yvel(k);
+            const float *gp = g + i * P;
+            const float u = carry_u[k][tid];
+            const float n = carry_n[k][tid];
+            float t;
+            if (diry(i) > 0) {
+                const float un = __ldg(gp + rp1) - fs[i];                // U_{y+1}
+                const float nn = minmod(un, u);                          // N_y
+                t = nn - n;                                              // N_y - N_{y-1}
+                carry_u[k][tid] = un;
+                carry_n[k][tid] = nn;
+            } else {
+                const float un = __ldg(gp + rp1) - __ldg(gp + rp2);      // U_{y+1}
+                const float nn = minmod(u, un);                          // N_{y+1}
+                t = n - nn;                                              // N_y - N_{y+1}
+                carry_u[k][tid] = un;
+                carry_n[k][tid] = nn;
             }
-            if (active && tid == last) {
-                int k = 0;
-#pragma unroll
-                for (int i = 0; i < kNV; ++i) {
-                    if (dirx(i) == 0) continue;
-                    const TS *gp = g + i * P + row;
-                    row_u[k][last + 2] = dirx(i) > 0 ? __ldg(gp + xp1) - fs[i] : __ldg(gp + xp1) - __ldg(gp + xp2);
-                    ++k;
-                }
-            }
-            __syncthreads();
-            if (active) {
-                int k = 0;
-#pragma unroll
-                for (int i = 0; i < kNV; ++i) {
-                    if (dirx(i) == 0) continue;
-                    const int s = dirx(i);
-                    const TS av = row_u[k][tid + 1];              // c - u1
-                    const TS bv = row_u[k][tid + 1 + s];          // d1 - c
-                    const TS ev = row_u[k][tid + 1 - s];          // u1 - u2
-                    const TS t = minmod(bv, av) - minmod(av, ev);
-                    o[i] = fma_t(-lx_of<TS>(a, i >> 2), fma_t((TS)0.5, t, av), o[i]);
-                    ++k;
-                }
-            }
+            o[i] = fmaf(-a.ly_f[i >> 2], fmaf(0.5f, t, u), o[i]);
         }
-        if (active) {
-            const size_t rp1 = (size_t)neighbour(y + 1, ny, a.bc_y) * nx + x;
-            const size_t rp2 = (size_t)neighbour(y + 2, ny, a.bc_y) * nx + x;
 #pragma unroll
-            for (int k = 0; k < kNY; ++k) {
-                const int i = yvel(k);
-                const TS *gp = g + i * P;
-                const TS u = carry_u[k][tid];
-                const TS n = carry_n[k][tid];
-                TS t;
-                if (diry(i) > 0) {
-                    const TS un = __ldg(gp + rp1) - fs[i];                  // U_{y+1}
-                    const TS nn = minmod(un, u);                            // N_y
-                    t = nn - n;                                             // N_y - N_{y-1}
-                    carry_u[k][tid] = un;
-                    carry_n[k][tid] = nn;
-                } else {
-                    const TS un = __ldg(gp + rp1) - __ldg(gp + rp2);        // U_{y+1}
-                    const TS nn = minmod(u, un);                            // N_{y+1}
-                    t = n - nn;                                             // N_y - N_{y+1}
-                    carry_u[k][tid] = un;
-                    carry_n[k][tid] = nn;
-                }
-                o[i] = fma_t(-ly_of<TS>(a, i >> 2), fma_t((TS)0.5, t, u), o[i]);
-            }
-#pragma unroll
-            for (int i = 0; i < kNV; ++i) out[i * P + c] = o[i];
-        }
+        for (int i = 0; i < kNV; ++i) out[i * P + c] = o[i];
     }
 }
 
@@ -348,10 +466,10 @@ __global__ void __launch_bounds__(kStageThreads, kMarch2MinBlocks)
     const int y1 = y0 + R < ny ? y0 + R : ny;
     if (y0 >= y1) return;
     const size_t P = (size_t)nx * ny;
-    const int m2a = neighbour(x0 - 2, nx, a.bc_x), m1a = neighbour(x0 - 1, nx, a.bc_x);
-    const int p1a = neighbour(x0 + 1, nx, a.bc_x), p2a = neighbour(x0 + 2, nx, a.bc_x);
-    const int m2b = neighbour(x1 - 2, nx, a.bc_x), m1b = neighbour(x1 - 1, nx, a.bc_x);
-    const int p1b = neighbour(x1 + 1, nx, a.bc_x), p2b = neighbour(x1 + 2, nx, a.bc_x);
+    const int m2a = neighbour_near(x0 - 2, nx, a.bc_x), m1a = neighbour_near(x0 - 1, nx, a.bc_x);
+    const int p1a = neighbour_near(x0 + 1, nx, a.bc_x), p2a = neighbour_near(x0 + 2, nx, a.bc_x);
+    const int m2b = neighbour_near(x1 - 2, nx, a.bc_x), m1b = neighbour_near(x1 - 1, nx, a.bc_x);
+    const int p1b = neighbour_near(x1 + 1, nx, a.bc_x), p2b = neighbour_near(x1 + 2, nx, a.bc_x);
     const float2 half2 = make_float2(0.5f, 0.5f);
     // the two cells of a row, and an arbitrary pair of columns of a row
     auto ld = [&](const float *p) -> float2 {
@@ -390,9 +508,9 @@ __global__ void __launch_bounds__(kStageThreads, kMarch2MinBlocks)
     // prologue: U_{y0} and N_{y0 - 1} for s = +1, N_{y0} for s = -1
     {
         const size_t r0 = (size_t)y0 * nx;
-        const size_t rm1 = (size_t)neighbour(y0 - 1, ny, a.bc_y) * nx;
-        const size_t rm2 = (size_t)neighbour(y0 - 2, ny, a.bc_y) * nx;
-        const size_t rp1 = (size_t)neighbour(y0 + 1, ny, a.bc_y) * nx;
+        const size_t rm1 = (size_t)neighbour_near(y0 - 1, ny, a.bc_y) * nx;
+        const size_t rm2 = (size_t)neighbour_near(y0 - 2, ny, a.bc_y) * nx;
+        const size_t rp1 = (size_t)neighbour_near(y0 + 1, ny, a.bc_y) * nx;
 #pragma unroll
         for (int k = 0; k < kNY; ++k) {
             const int i = yvel(k);
@@ -415,8 +533,8 @@ __global__ void __launch_bounds__(kStageThreads, kMarch2MinBlocks)
     stage_row(0, (size_t)y0 * nx);
     for (int y = y0, b = 0; y < y1; ++y, b ^= 1) {
         const size_t row = (size_t)y * nx;
-        const size_t rp1 = (size_t)neighbour(y + 1, ny, a.bc_y) * nx;
-        const size_t rp2 = (size_t)neighbour(y + 2, ny, a.bc_y) * nx;
+        const size_t rp1 = (size_t)neighbour_near(y + 1, ny, a.bc_y) * nx;
+        const size_t rp2 = (size_t)neighbour_near(y + 2, ny, a.bc_y) * nx;
         // With the deviation equilibrium the kernel is bound by load latency. So
         // row y+2 and, in the second stage, the next base row are prefetched into L2
         // without holding registers. Row y+2 is what the downward velocities read in
@@ -846,16 +964,30 @@ void *stage_march2_func(bool with_base, bool vec, bool dev)
     return dev ? stage_march2_func_t<kEqF32>(with_base, vec) : stage_march2_func_t<kEqDF>(with_base, vec);
 }
 
-template <typename TS, int kEq>
+void *fx_func(bool with_base, bool flat, bool wide)
+{
+    if (wide) {
+        if (with_base) return flat ? (void *)stage_fx_kernel<true, true, true> : (void *)stage_fx_kernel<true, false, true>;
+        return flat ? (void *)stage_fx_kernel<false, true, true> : (void *)stage_fx_kernel<false, false, true>;
+    }
+    if (with_base) return flat ? (void *)stage_fx_kernel<true, true, false> : (void *)stage_fx_kernel<true, false, false>;
+    return flat ? (void *)stage_fx_kernel<false, true, false> : (void *)stage_fx_kernel<false, false, false>;
+}
+
+void *fx_split_func(bool with_base, bool flat)
+{
+    if (with_base) return flat ? (void *)stage_fx_split_kernel<true, true> : (void *)stage_fx_split_kernel<true, false>;
+    return flat ? (void *)stage_fx_split_kernel<false, true> : (void *)stage_fx_split_kernel<false, false>;
+}
+
+template <int kEq>
 void *stage_func(bool march, bool with_base, bool flat)
 {
-    if constexpr (kEq == kEqDouble) {   // the single-precision equilibria march with stage_march2_kernel
-        if (march)
-            return with_base ? (void *)stage_march_kernel<TS, true, kEq> : (void *)stage_march_kernel<TS, false, kEq>;
+    if constexpr (kEq == kEqDouble) {   // the other equilibria march with stage_march2_kernel
+        if (march) return with_base ? (void *)stage_march_kernel<true> : (void *)stage_march_kernel<false>;
     }
-    if (with_base)
-        return flat ? (void *)stage_kernel<TS, true, true, kEq> : (void *)stage_kernel<TS, true, false, kEq>;
-    return flat ? (void *)stage_kernel<TS, false, true, kEq> : (void *)stage_kernel<TS, false, false, kEq>;
+    if (with_base) return flat ? (void *)stage_kernel<true, true, kEq> : (void *)stage_kernel<true, false, kEq>;
+    return flat ? (void *)stage_kernel<false, true, kEq> : (void *)stage_kernel<false, false, kEq>;
 }
 
 }  // namespace
@@ -950,6 +1082,28 @@ StageLaunch stage_launch_config(const StageArgs &a, bool with_base, int sm_count
         L.grid = dim3((unsigned)((4 * (size_t)a.nx + kSplitFlatThreads - 1) / kSplitFlatThreads), 1, 1);
         return L;
     }
+    if (prec == CDBM_FP64) {
+        const unsigned rows = a.ny < 65535 ? a.ny : 65535;
+        // Below half of the threads that stage_fx_kernel keeps resident the time is the
+        // chain of one thread: four threads per cell.  Per stage, split against one
+        // thread per cell: 8.8 / 17.0 us at 64^2, 14.3 / 16.9 at 128^2, 20.8 / 25.4 at
+        // 160^2, 38.2 / 36.2 at 256^2.
+        if (allow_split && cells <= (size_t)sm_count * kFxMinBlocks * kStageThreads / 2) {
+            L.func = fx_split_func(with_base, flat);
+            L.block = dim3(128, 1, 1);
+            L.grid = dim3((unsigned)((a.nx + 31) / 32), rows, 1);
+            return L;
+        }
+        // the widest block whose padding past the row's end is least
+        unsigned w = kStageThreads;
+        auto pad = [&](unsigned t) { return ((size_t)a.nx + t - 1) / t * t; };
+        for (unsigned t = kStageThreads / 2; t >= 32; t /= 2)
+            if (pad(t) < pad(w)) w = t;
+        L.func = fx_func(with_base, flat, a.nx >= (1 << 29));
+        L.block = dim3(w, 1, 1);
+        L.grid = dim3((unsigned)(pad(w) / w), rows, 1);
+        return L;
+    }
     // The df64 and single-precision deviation equilibria march two columns per thread
     // (stage_march2_kernel).
     const bool pair = prec == CDBM_FP32_DF64 || prec == CDBM_FP32_DEV;
@@ -972,15 +1126,7 @@ StageLaunch stage_launch_config(const StageArgs &a, bool with_base, int sm_count
     }
     if (march) {
         L.func = pair ? stage_march2_func(with_base, (a.nx & 1) == 0, prec == CDBM_FP32_DEV)
-                 : prec == CDBM_FP32_BULK ? stage_func<float, kEqDouble>(true, with_base, false)
-                                          : stage_func<double, kEqDouble>(true, with_base, false);
-        if (prec == CDBM_FP64) {
-            // the double-buffered x row buffer of stage_march_kernel<double>
-            L.smem = kMarchRowBytes;
-            if (cudaFuncSetAttribute(L.func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem) !=
-                cudaSuccess)
-                cudaGetLastError();   // the launch then reports the error
-        }
+                      : stage_func<kEqDouble>(true, with_base, false);
         if (pair) {
             // rows staged by cp.async: dynamic shared memory beside the static carries
             L.smem = kMarch2StageBytes;
@@ -993,10 +1139,9 @@ StageLaunch stage_launch_config(const StageArgs &a, bool with_base, int sm_count
         L.grid = dim3(xblocks, yblocks < 65535 ? yblocks : 65535, 1);
         return L;
     }
-    L.func = prec == CDBM_FP32_DEV    ? stage_func<float, kEqF32>(false, with_base, flat)
-             : prec == CDBM_FP32_DF64 ? stage_func<float, kEqDF>(false, with_base, flat)
-             : prec == CDBM_FP32_BULK ? stage_func<float, kEqDouble>(false, with_base, flat)
-                                      : stage_func<double, kEqDouble>(false, with_base, flat);
+    L.func = prec == CDBM_FP32_DEV    ? stage_func<kEqF32>(false, with_base, flat)
+             : prec == CDBM_FP32_DF64 ? stage_func<kEqDF>(false, with_base, flat)
+                                      : stage_func<kEqDouble>(false, with_base, flat);
     // Small grids: narrower blocks so that more SMs share the cells.
     int threads = kStageThreads;
     while (threads > 32 && cells < (size_t)sm_count * threads * 2) threads >>= 1;
@@ -1092,6 +1237,7 @@ DFShiftT<float2> df_shift_twice(const DFShift &d)
 
 void fill_df_consts(StageArgs &a)
 {
+    fill_fx_consts(a);
     a.d.b = df_blocks(a.eq);
     a.d.m = df_model(a.m);
     a.d.r = df_shift(a.sF, a.rhoF, a.EF);
@@ -1105,6 +1251,13 @@ void fill_df_consts(StageArgs &a)
         a.lx_f2[g] = make_float2(a.lx_f[g], a.lx_f[g]);
         a.ly_f2[g] = make_float2(a.ly_f[g], a.ly_f[g]);
     }
+}
+
+void fill_fx_consts(StageArgs &a)
+{
+    a.fx.m = fx_model(a.m.c, a.m.w);
+    a.fx.k = fx_coef(a.a_self, a.a_base);
+    a.fx.l = fx_flux(a.lx, a.ly, a.nx > 1, a.ny > 1);
 }
 
 DevProj dev_proj(const ModelConsts &m, double gh)

@@ -41,8 +41,8 @@ __device__ __forceinline__ TS cluster_value(const cg::cluster_group &cl, const T
 // stencil values (and the base) are gathered into registers before the first store,
 // so the loads of the edge cells from the neighbouring CTAs overlap instead of each
 // waiting behind a store the compiler cannot prove independent.
-template <typename TS, bool kBase, int kEq>
-__device__ __forceinline__ void cluster_stage(const cg::cluster_group &cl, const TS *src, const TS *base, TS *dst,
+template <bool kBase, int kEq>
+__device__ __forceinline__ void cluster_stage(const cg::cluster_group &cl, const float *src, const float *base, float *dst,
                                               const StageArgs &a, int chunk, int rank, int x0, int len,
                                               unsigned *flag)
 {
@@ -50,7 +50,7 @@ __device__ __forceinline__ void cluster_stage(const cg::cluster_group &cl, const
     const int nx = a.nx;
     for (int lx = threadIdx.x; lx < len; lx += blockDim.x) {
         const int gx = x0 + lx;
-        TS fs[kNV], bs[kNV], up2[kNX], up1[kNX], dn1[kNX];
+        float fs[kNV], bs[kNV], up2[kNX], up1[kNX], dn1[kNX];
 #pragma unroll
         for (int i = 0; i < kNV; ++i) {
             fs[i] = src[i * chunk + lx];
@@ -61,15 +61,15 @@ __device__ __forceinline__ void cluster_stage(const cg::cluster_group &cl, const
 #pragma unroll
             for (int i = 0; i < kNV; ++i) {
                 if (dirx(i) == 0) continue;
-                const TS *p = src + i * chunk + lx;
+                const float *p = src + i * chunk + lx;
                 up2[k] = p[dirx(i) > 0 ? -2 : 2];
                 up1[k] = p[dirx(i) > 0 ? -1 : 1];
                 dn1[k] = p[dirx(i) > 0 ? 1 : -1];
                 ++k;
             }
         } else {
-            const int xm2 = neighbour(gx - 2, nx, a.bc_x), xm1 = neighbour(gx - 1, nx, a.bc_x);
-            const int xp1 = neighbour(gx + 1, nx, a.bc_x), xp2 = neighbour(gx + 2, nx, a.bc_x);
+            const int xm2 = neighbour_near(gx - 2, nx, a.bc_x), xm1 = neighbour_near(gx - 1, nx, a.bc_x);
+            const int xp1 = neighbour_near(gx + 1, nx, a.bc_x), xp2 = neighbour_near(gx + 2, nx, a.bc_x);
             int k = 0;
 #pragma unroll
             for (int i = 0; i < kNV; ++i) {
@@ -80,15 +80,15 @@ __device__ __forceinline__ void cluster_stage(const cg::cluster_group &cl, const
                 ++k;
             }
         }
-        TS heq[kNV];
-        stage_equilibrium<TS, kEq>(a, fs, heq, flag);
+        float heq[kNV];
+        stage_equilibrium<kEq>(a, fs, heq, flag);
         int k = 0;
 #pragma unroll
         for (int i = 0; i < kNV; ++i) {
-            TS o = fma_t(a_self_of<TS>(a), fs[i], heq[i]);
-            if (kBase) o = fma_t(a_base_of<TS>(a), bs[i], o);
+            float o = fmaf(a.a_self_f, fs[i], heq[i]);
+            if (kBase) o = fmaf(a.a_base_f, bs[i], o);
             if (dirx(i) != 0) {
-                o = fma_t(-lx_of<TS>(a, i >> 2), nnd(up2[k], up1[k], fs[i], dn1[k]), o);
+                o = fmaf(-a.lx_f[i >> 2], nnd(up2[k], up1[k], fs[i], dn1[k]), o);
                 ++k;
             }
             dst[i * chunk + lx] = o;
@@ -96,13 +96,13 @@ __device__ __forceinline__ void cluster_stage(const cg::cluster_group &cl, const
     }
 }
 
-template <typename TS, int kEq>
-__global__ void __launch_bounds__(256) small1d_kernel(TS *f, int nsteps, const StageArgs a0, const StageArgs a1,
+template <int kEq>
+__global__ void __launch_bounds__(256) small1d_kernel(float *f, int nsteps, const StageArgs a0, const StageArgs a1,
                                                       unsigned *flag, int chunk)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TS *s0 = reinterpret_cast<TS *>(smem_raw);     // state f^n, [16][chunk]
-    TS *s1 = s0 + kNV * chunk;                     // stage buffer
+    float *s0 = reinterpret_cast<float *>(smem_raw);     // state f^n, [16][chunk]
+    float *s1 = s0 + kNV * chunk;                     // stage buffer
     const cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const int nx = a0.nx;
@@ -114,9 +114,9 @@ __global__ void __launch_bounds__(256) small1d_kernel(TS *f, int nsteps, const S
     }
     cl.sync();
     for (int s = 0; s < nsteps; ++s) {
-        cluster_stage<TS, false, kEq>(cl, s0, nullptr, s1, a0, chunk, rank, x0, len, flag);
+        cluster_stage<false, kEq>(cl, s0, nullptr, s1, a0, chunk, rank, x0, len, flag);
         cl.sync();
-        cluster_stage<TS, true, kEq>(cl, s1, s0, s0, a1, chunk, rank, x0, len, flag);
+        cluster_stage<true, kEq>(cl, s1, s0, s0, a1, chunk, rank, x0, len, flag);
         cl.sync();
     }
     for (int k = threadIdx.x; k < kNV * len; k += blockDim.x) {
@@ -218,8 +218,8 @@ __device__ __forceinline__ void split_stage(const cg::cluster_group &cl, const d
         bs[j] = with_base ? base[(4 * g + j) * chunk + lx] : 0.0;
     }
     const bool inner = lx >= 2 && lx + 2 < len;
-    const int xm2 = neighbour(gx - 2, nx, a.bc_x), xm1 = neighbour(gx - 1, nx, a.bc_x);
-    const int xp1 = neighbour(gx + 1, nx, a.bc_x), xp2 = neighbour(gx + 2, nx, a.bc_x);
+    const int xm2 = neighbour_near(gx - 2, nx, a.bc_x), xm1 = neighbour_near(gx - 1, nx, a.bc_x);
+    const int xp1 = neighbour_near(gx + 1, nx, a.bc_x), xp2 = neighbour_near(gx + 2, nx, a.bc_x);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int i = 4 * g + j;
@@ -269,8 +269,8 @@ __global__ void __launch_bounds__(kSplitFlatThreads) stage_split_flat_kernel(con
         q[j] = g[(4 * gq + j) * P + x];
         bs[j] = kBase ? base[(4 * gq + j) * P + x] : 0.0;
     }
-    const int xm2 = neighbour(x - 2, nx, a.bc_x), xm1 = neighbour(x - 1, nx, a.bc_x);
-    const int xp1 = neighbour(x + 1, nx, a.bc_x), xp2 = neighbour(x + 2, nx, a.bc_x);
+    const int xm2 = neighbour_near(x - 2, nx, a.bc_x), xm1 = neighbour_near(x - 1, nx, a.bc_x);
+    const int xp1 = neighbour_near(x + 1, nx, a.bc_x), xp2 = neighbour_near(x + 2, nx, a.bc_x);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int i = 4 * gq + j;
@@ -343,8 +343,8 @@ __device__ __forceinline__ void split_stage_df(const cg::cluster_group &cl, cons
         bs[j] = kBase ? base[(8 * h + j) * chunk + lx] : 0.0f;
     }
     const bool inner = lx >= 2 && lx + 2 < len;
-    const int xm2 = neighbour(gx - 2, nx, a.bc_x), xm1 = neighbour(gx - 1, nx, a.bc_x);
-    const int xp1 = neighbour(gx + 1, nx, a.bc_x), xp2 = neighbour(gx + 2, nx, a.bc_x);
+    const int xm2 = neighbour_near(gx - 2, nx, a.bc_x), xm1 = neighbour_near(gx - 1, nx, a.bc_x);
+    const int xp1 = neighbour_near(gx + 1, nx, a.bc_x), xp2 = neighbour_near(gx + 2, nx, a.bc_x);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const int i = 8 * h + j;
@@ -419,17 +419,17 @@ __global__ void __launch_bounds__(256) small1d_split_df_kernel(float *f, int nst
     }
 }
 
-template <typename TS, int kEq>
-void *small1d_func() { return (void *)small1d_kernel<TS, kEq>; }
+template <int kEq>
+void *small1d_func() { return (void *)small1d_kernel<kEq>; }
 
 constexpr int kSplitDfMaxChunk = 128;     // two threads per cell within 256 threads
 
 void *small1d_func_of(int prec, int chunk)
 {
     if (prec == CDBM_FP32_DF64)
-        return chunk <= kSplitDfMaxChunk ? (void *)small1d_split_df_kernel : small1d_func<float, kEqDF>();
-    if (prec == CDBM_FP32_DEV) return small1d_func<float, kEqF32>();
-    if (prec == CDBM_FP32_BULK) return small1d_func<float, kEqDouble>();
+        return chunk <= kSplitDfMaxChunk ? (void *)small1d_split_df_kernel : small1d_func<kEqDF>();
+    if (prec == CDBM_FP32_DEV) return small1d_func<kEqF32>();
+    if (prec == CDBM_FP32_BULK) return small1d_func<kEqDouble>();
     return (void *)small1d_split_kernel;
 }
 
