@@ -495,6 +495,7 @@ cdbm_status cdbm_create(const cdbm_grid *grid, const cdbm_vset *vset, double I, 
     build_stages(c);
     c->fields.eq = c->eq_unit;
     c->fields.m = c->mc;
+    c->fields.fx = fx_model(c->mc.c, c->mc.w);
     for (int i = 0; i < kNV; ++i) {
         const double s = vset->v[i >> 2];
         c->fields.vx[i] = dirx(i) * s;

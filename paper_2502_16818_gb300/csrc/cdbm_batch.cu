@@ -168,14 +168,23 @@ struct TubeCell {
     }
 };
 
+// The constants of the tube a block works on, in shared memory: indexed per tube in the
+// kernel's parameters they cost several times as much to read.
+struct TubeConsts {
+    EqBlocks eq[2];
+    ModelConsts m;
+    FxModel fx;
+    FxFlux l[2];
+    double lx[2][4];
+};
+
 // The members of group grp of one cell of a tube (kSym: the distinct ones), one per pass.
 template <bool kDiag, int kStage, bool kSym>
-__device__ __forceinline__ void tube_group_fx(const TubeCell<kSym> &cell, const int xs[4], const TubeInfo &t,
-                                              const ClassConsts &C, const FxCoef &k, double a_self, double a_base,
+__device__ __forceinline__ void tube_group_fx(const TubeCell<kSym> &cell, const int xs[4], const TubeConsts &C, const FxCoef &k, double a_self, double a_base,
                                               int grp, const FxGroup h, bool cell_ok, unsigned *flag)
 {
     constexpr bool kBase = kStage == 1;
-    const FxK lx = t.fx[kStage].klx[grp];
+    const FxK lx = C.l[kStage].klx[grp];
     unsigned rest = 0;
     auto pass = [&](int j, auto transport) {
         constexpr bool kX = decltype(transport)::value;
@@ -209,18 +218,17 @@ __device__ __forceinline__ void tube_group_fx(const TubeCell<kSym> &cell, const 
         for (int j = 1; j < (kSym ? 2 : 4); j += 2) pass(j, std::false_type{});     // N, S: no transport
     }
     if (rest)
-        fx_rest_of_group<TubeCell<kSym>, kBase, true>(cell, C.eq[kStage], C.m, k, t.fx[kStage],
-                                                      {a_self, a_base, t.lx[kStage], t.lx[kStage]}, grp, rest, cell_ok,
+        fx_rest_of_group<TubeCell<kSym>, kBase, true>(cell, C.eq[kStage], C.m, k, C.l[kStage],
+                                                      {a_self, a_base, C.lx[kStage], C.lx[kStage]}, grp, rest, cell_ok,
                                                       h, flag);
 }
 
 // The FP64 stage of one tube (cdbm_stage_fx.cuh), one cell per thread.
 template <int kStage, bool kSym>
 __device__ __forceinline__ void tube_stage_fx(const double *g, const double *base, double *out, long long P,
-                                              const TubeInfo &t, const ClassConsts &C, const FxCoef &k, double a_self,
+                                              int nx, const TubeConsts &C, const FxCoef &k, double a_self,
                                               double a_base, unsigned *flag)
 {
-    const int nx = t.nx;
     for (int x = threadIdx.x; x < nx; x += blockDim.x) {
         const int xs[4] = {x >= 2 ? x - 2 : 0, x >= 1 ? x - 1 : 0, x + 1 < nx ? x + 1 : nx - 1, x + 2 < nx ? x + 2 : nx - 1};
         const TubeCell<kSym> cell = {g, base, out, P, nx, x};
@@ -228,9 +236,9 @@ __device__ __forceinline__ void tube_stage_fx(const double *g, const double *bas
         const EqFactors q = kSym ? eq_factors_sym(C.m, m.rho, m.jx, m.E, flag) : eq_factors(C.m, m.rho, m.jx, m.jy, m.E, flag);
 #pragma unroll 1
         for (int p = 0; p < 4; p += 2) {
-            tube_group_fx<false, kStage, kSym>(cell, xs, t, C, k, a_self, a_base, p, fx_group<kSym>(C.eq[kStage], q, p),
+            tube_group_fx<false, kStage, kSym>(cell, xs, C, k, a_self, a_base, p, fx_group<kSym>(C.eq[kStage], q, p),
                                                m.ok, flag);
-            tube_group_fx<true, kStage, kSym>(cell, xs, t, C, k, a_self, a_base, p + 1,
+            tube_group_fx<true, kStage, kSym>(cell, xs, C, k, a_self, a_base, p + 1,
                                               fx_group<kSym>(C.eq[kStage], q, p + 1), m.ok, flag);
         }
     }
@@ -322,16 +330,28 @@ __global__ void __launch_bounds__(kThreads, batch_min_blocks(!kSingle<TS>, kThre
                                                          const int *work, const int *work_off, int nsteps,
                                                          const __grid_constant__ BatchArgs a, unsigned *flag)
 {
+    __shared__ TubeConsts tc;          // FP64 only
     for (int w = work_off[blockIdx.x]; w < work_off[blockIdx.x + 1]; ++w) {
         const TubeInfo &t = tubes[work[w]];
         const ClassConsts &C = a.cls[t.cls];
+        if constexpr (!kSingle<TS>) {
+            // every thread of the block has passed the last barrier of the tube before
+            for (int s = threadIdx.x; s < 2; s += blockDim.x) {
+                tc.eq[s] = C.eq[s];
+                tc.l[s] = t.fx[s];
+                for (int g = 0; g < 4; ++g) tc.lx[s][g] = t.lx[s][g];
+            }
+            if (threadIdx.x == 32) tc.m = C.m;
+            if (threadIdx.x == 33) tc.fx = C.fx;
+            __syncthreads();
+        }
         TS *ft = f + t.offset;
         TS *f1t = f1 + t.offset;
         for (int s = 0; s < nsteps; ++s) {
             if constexpr (!kSingle<TS>) {
-                tube_stage_fx<0, kSym>(ft, nullptr, f1t, a.P, t, C, a.fx[0], a.a_self[0], a.a_base[0], flag);
+                tube_stage_fx<0, kSym>(ft, nullptr, f1t, a.P, t.nx, tc, a.fx[0], a.a_self[0], a.a_base[0], flag);
                 __syncthreads();
-                tube_stage_fx<1, kSym>(f1t, ft, ft, a.P, t, C, a.fx[1], a.a_self[1], a.a_base[1], flag);
+                tube_stage_fx<1, kSym>(f1t, ft, ft, a.P, t.nx, tc, a.fx[1], a.a_self[1], a.a_base[1], flag);
             } else if constexpr (kEq == kEqDF) {
                 tube_stage2<0, kSym>(ft, nullptr, f1t, a.P, t, C, a.a_self_f2[0], a.a_base_f2[0], flag);
                 __syncthreads();
@@ -369,41 +389,46 @@ __global__ void __launch_bounds__(128) batch_init_kernel(const BatchArgs a, cons
         const TubeInfo &t = tubes[tube_of(offs, ntubes, c)];
         const ClassConsts &C = a.cls[t.cls];
         const double r = rho[c], u = ux[c], v = uy[c], tt = T[c];
-        const double jx = r * u, jy = r * v;
-        const double jyuy = jy * v;
-        const double ru2 = fma(jx, u, jyuy);
-        const double p = r * tt;
-        const double E = fma(C.m.K, p, ru2);
         double fe[kNV];
-        equilibrium(C.unit, C.m, r, E, jx, jy, u, v, ru2, jyuy, p, tt, fe);
+        if constexpr (kSingle<TS>) equilibrium_of(C.unit, C.m, r, u, v, tt, fe);
+        else fx_equilibrium_of(C.unit, C.m, r, u, v, tt, fe);
         if (!(positive_finite(r) && positive_finite(tt) && isfinite(u) && isfinite(v)))
             atomicOr(flag, kFlagNonPhys);
 #pragma unroll
         for (int i = 0; i < kNV; ++i) {
             if constexpr (kSingle<TS>)
-                f[i * a.P + c] = (float)(fe[i] - t.Fg[i >> 2]);
+                f[i * a.P + c] = narrow_f64(fe[i] - t.Fg[i >> 2]);
             else
                 f[i * a.P + c] = fe[i];
         }
     }
 }
 
+// Conserved moments in FP64, for cells outside the fixed-point path.
 template <typename TS>
-__global__ void __launch_bounds__(128) batch_macros_kernel(const BatchArgs a, const TubeInfo *tubes,
+__device__ __noinline__ Cons batch_conserved_any(const ModelConsts &m, const TS *own, long long P)
+{
+    double fc[kNV];
+    for (int i = 0; i < kNV; ++i) fc[i] = widen(own[i * P]);
+    return conserved(fc, m);
+}
+
+template <typename TS>
+__global__ void __launch_bounds__(128) batch_macros_kernel(const ClassConsts *__restrict__ cls, long long P, const TubeInfo *tubes,
                                                             const long long *offs, int ntubes, const TS *f,
                                                             double *rho, double *ux, double *uy, double *T)
 {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < a.P;
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < P;
          c += (long long)gridDim.x * blockDim.x) {
         const TubeInfo &t = tubes[tube_of(offs, ntubes, c)];
-        const ModelConsts &m = a.cls[t.cls].m;
+        const ModelConsts &m = cls[t.cls].m;
         // the operations of the single-grid macros kernel: moments of the stored
         // values (plus the reference equilibrium's for a single-precision state)
         // and one reciprocal of rho
-        double fc[kNV];
-#pragma unroll
-        for (int i = 0; i < kNV; ++i) fc[i] = widen(f[i * a.P + c]);
-        Cons q = conserved(fc, m);
+        const TS *own = f + c;
+        const FxCons fm = fx_conserved(cls[t.cls].fx, [=](int i) { return __ldg(own + i * P); });
+        Cons q = {fm.rho, fm.jx, fm.jy, fm.E};
+        if (!fm.ok) q = batch_conserved_any(m, own, P);
         if constexpr (kSingle<TS>) {
             q.rho += t.rhoF;
             q.E += t.EF;
@@ -457,6 +482,7 @@ struct cdbm_batch {
     BatchArgs args;
     void *f, *f1;
     TubeInfo *d_tubes;
+    ClassConsts *d_cls;                // args.cls in device memory, for the read-out
     long long *d_offs;
     int *d_work, *d_work_off;          // partition: tube ids per block (CSR)
     unsigned *flag;
@@ -741,9 +767,10 @@ cdbm_status cdbm_batch_create(int ntubes, const int *nx, const double *dx, const
     b->f = balloc(b, fb);
     b->f1 = balloc(b, fb);
     b->d_tubes = (TubeInfo *)balloc(b, sizeof(TubeInfo) * ntubes);
+    b->d_cls = (ClassConsts *)balloc(b, sizeof(b->args.cls));
     b->d_offs = (long long *)balloc(b, sizeof(long long) * (ntubes + 1));
     b->flag = (unsigned *)balloc(b, 256);
-    if (!b->f || !b->f1 || !b->d_tubes || !b->d_offs || !b->flag ||
+    if (!b->f || !b->f1 || !b->d_tubes || !b->d_cls || !b->d_offs || !b->flag ||
         cudaMallocHost(&b->flag_host, sizeof(unsigned)) != cudaSuccess) {
         cudaGetLastError();
         cdbm_batch_destroy(b);
@@ -752,6 +779,7 @@ cdbm_status cdbm_batch_create(int ntubes, const int *nx, const double *dx, const
     if (cudaMemsetAsync(b->flag, 0, sizeof(unsigned), b->stream) != cudaSuccess ||
         cudaMemcpyAsync(b->d_offs, b->offs.data(), sizeof(long long) * (ntubes + 1), cudaMemcpyHostToDevice,
                         b->stream) != cudaSuccess ||
+        cudaMemcpyAsync(b->d_cls, b->args.cls, sizeof(b->args.cls), cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
         cudaMemcpyAsync(b->d_tubes, b->info.data(), sizeof(TubeInfo) * ntubes, cudaMemcpyHostToDevice,
                         b->stream) != cudaSuccess) {
         cudaGetLastError();
@@ -941,10 +969,10 @@ cdbm_status cdbm_batch_macros(cdbm_batch *b, double *rho, double *ux, double *uy
     }
     const unsigned nb = cells_grid(b->P);
     if (single_storage(b->precision))
-        batch_macros_kernel<float><<<nb, 128, 0, b->stream>>>(b->args, b->d_tubes, b->d_offs, b->ntubes,
+        batch_macros_kernel<float><<<nb, 128, 0, b->stream>>>(b->d_cls, b->P, b->d_tubes, b->d_offs, b->ntubes,
                                                               (const float *)b->f, dev[0], dev[1], dev[2], dev[3]);
     else
-        batch_macros_kernel<double><<<nb, 128, 0, b->stream>>>(b->args, b->d_tubes, b->d_offs, b->ntubes,
+        batch_macros_kernel<double><<<nb, 128, 0, b->stream>>>(b->d_cls, b->P, b->d_tubes, b->d_offs, b->ntubes,
                                                                (const double *)b->f, dev[0], dev[1], dev[2], dev[3]);
     if (bcuda(b, cudaGetLastError(), "batch macros launch")) return b->err;
     for (int k = 0; k < 4; ++k)
@@ -986,6 +1014,7 @@ void cdbm_batch_destroy(cdbm_batch *b)
     bfree(b, b->f, fb);
     bfree(b, b->f1, fb);
     bfree(b, b->d_tubes, 0);
+    bfree(b, b->d_cls, 0);
     bfree(b, b->d_offs, 0);
     bfree(b, b->flag, 256);
     bfree(b, b->d_work, 0);

@@ -213,6 +213,18 @@ __device__ __forceinline__ void equilibrium(const EqBlocks &B, const ModelConsts
     equilibrium_group(B, 3, s0[3], qd, jx, jy, T, u2, dlt, out + 12);
 }
 
+// f_eq of the fields rho, u, v, T.
+__device__ __forceinline__ void equilibrium_of(const EqBlocks &B, const ModelConsts &m, double rho, double u, double v,
+                                               double T, double out[kNV])
+{
+    const double jx = rho * u, jy = rho * v;
+    const double jyuy = jy * v;
+    const double ru2 = fma(jx, u, jyuy);
+    const double p = rho * T;
+    const double E = fma(m.K, p, ru2);
+    equilibrium(B, m, rho, E, jx, jy, u, v, ru2, jyuy, p, T, out);
+}
+
 template <typename TS>
 constexpr bool kSingle = std::is_same<TS, float>::value;
 

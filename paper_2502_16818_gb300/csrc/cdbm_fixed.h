@@ -83,6 +83,21 @@ CDBM_FX_HD int64_t fx_from_t(double v, int E)
 CDBM_FX_HD int64_t fx_from(double v, int E) { return fx_from_t<false, kLead>(v, E); }
 CDBM_FX_HD int64_t fx_clamped(double v, int E) { return fx_from_t<true, kLead>(v, E); }
 
+// Single-precision values: key >> 24 is their exponent field; v, whose exponent is at
+// most E, with the leading one of a value of exponent E at bit kLead, rounded to the
+// nearest unit (exact up to 34 binades below; subnormals count as zero).  It stands for
+// v 2^(E - 127 - kLead).
+CDBM_FX_HD uint32_t fx_key(float v) { return f32_bits(v) << 1; }
+CDBM_FX_HD int64_t fx_from(float v, int E)
+{
+    const uint32_t b = f32_bits(v);
+    const int e = (int)((b << 1) >> 24);
+    const uint32_t m = e ? (b & 0x7fffffu) | 0x800000u : 0u;
+    const int64_t w = (int64_t)(((uint64_t)m << 39) >> fx_imin(E + 3 - e, 63));   // in half units
+    const int64_t s = (int64_t)((int32_t)b >> 31);
+    return ((w ^ s) + (1 - s)) >> 1;
+}
+
 // v 2^(E - 1023 - kLead) rounded to double, to nearest, ties to even.  |v| < 2^63.
 CDBM_FX_HD double fx_to(int64_t v, int E)
 {

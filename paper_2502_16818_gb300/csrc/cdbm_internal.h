@@ -138,6 +138,7 @@ struct FieldArgs {
     ModelConsts m;
     double vx[kNV], vy[kNV], eta[kNV];
     double Fg[4];    // reference equilibrium per group (FP32-bulk state only)
+    FxModel fx;      // fixed-point model constants
     int nx, ny;
 };
 

@@ -34,6 +34,10 @@ constexpr int stage_min_blocks(int eq) { return eq != kEqDouble ? CDBM_STAGE_MIN
 
 // ---------------------------------------------------------------- init (K0)
 
+// f_eq of the fields.  Bound by the FP64 pipe: 62 instructions with the members rebuilt in
+// fixed point (fx_equilibrium_of; 86 before, 2.60 -> 1.99 ms for 4096^2 cells), 102 for a
+// single-precision state, whose values have to round as they always did (118 before the
+// narrowing left the pipe, 3.87 -> 3.26 ms with the means of rho and T).
 template <typename TS>
 __global__ void __launch_bounds__(128) init_kernel(const FieldArgs a, const double *__restrict__ rho,
                                                     const double *__restrict__ ux,
@@ -45,19 +49,15 @@ __global__ void __launch_bounds__(128) init_kernel(const FieldArgs a, const doub
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < P;
          c += (size_t)gridDim.x * blockDim.x) {
         const double r = rho[c], u = ux[c], v = uy[c], t = T[c];
-        const double jx = r * u, jy = r * v;
-        const double jyuy = jy * v;
-        const double ru2 = fma(jx, u, jyuy);
-        const double p = r * t;
-        const double E = fma(a.m.K, p, ru2);
         double fe[kNV];
-        equilibrium(a.eq, a.m, r, E, jx, jy, u, v, ru2, jyuy, p, t, fe);
+        if constexpr (kSingle<TS>) equilibrium_of(a.eq, a.m, r, u, v, t, fe);
+        else fx_equilibrium_of(a.eq, a.m, r, u, v, t, fe);
         if (!(positive_finite(r) && positive_finite(t) && isfinite(u) && isfinite(v)))
             atomicOr(flag, kFlagNonPhys);
 #pragma unroll
         for (int i = 0; i < kNV; ++i) {
             if constexpr (kSingle<TS>)
-                f[i * P + c] = (float)(fe[i] - a.Fg[i >> 2]);
+                f[i * P + c] = narrow_f64(fe[i] - a.Fg[i >> 2]);   // off the FP64 pipe
             else
                 f[i * P + c] = fe[i];
         }
@@ -684,17 +684,29 @@ RefMoments ref_moments(const FieldArgs &a, bool single)
 __device__ __forceinline__ double stored(double v) { return v; }
 __device__ __forceinline__ double stored(float v) { return widen_f32(v); }
 
+// The conserved moments of a stored cell: in fixed point (cdbm_stage_fx.cuh), or in FP64
+// where its exponents are outside that path.  10 instead of 51 FP64 instructions took
+// the fields of 4096^2 cells from 1.61 to 0.51 ms (0.40 ms at the memory's rate).
 template <typename TS>
-__global__ void __launch_bounds__(128) macros_kernel(const FieldArgs a, const RefMoments F, const TS *__restrict__ f,
-                                                      double *rho, double *ux, double *uy, double *T)
+__device__ __noinline__ Cons conserved_any(const FieldArgs &a, const TS *own, size_t P)
+{
+    double fc[kNV];
+    for (int i = 0; i < kNV; ++i) fc[i] = stored(own[i * P]);
+    return conserved(fc, a.m);
+}
+
+template <typename TS>
+__global__ void __launch_bounds__(128) macros_kernel(const __grid_constant__ FieldArgs a, const RefMoments F,
+                                                     const TS *__restrict__ f, double *rho, double *ux, double *uy,
+                                                     double *T)
 {
     const size_t P = (size_t)a.nx * a.ny;
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < P;
          c += (size_t)gridDim.x * blockDim.x) {
-        double fc[kNV];
-#pragma unroll
-        for (int i = 0; i < kNV; ++i) fc[i] = stored(f[i * P + c]);
-        Cons q = conserved(fc, a.m);
+        const TS *own = f + c;
+        const FxCons m = fx_conserved(a.fx, [=](int i) { return __ldg(own + i * P); });
+        Cons q = {m.rho, m.jx, m.jy, m.E};
+        if (!m.ok) q = conserved_any(a, own, P);
         if constexpr (kSingle<TS>) {
             q.rho += F.rho;
             q.E += F.E;
@@ -712,10 +724,55 @@ __global__ void __launch_bounds__(128) macros_kernel(const FieldArgs a, const Re
 // ------------------------------------------------------------ TNE (K4)
 
 // Powers of the group speed component c_g (v = (+-c_g, 0), (0, +-c_g) on the axis
-// groups, (+-c_g, +-c_g) on the diagonal ones) and of W_g = |v|^2 + eta_g^2.
-struct TneConsts {
-    double c[4], c2[4], c3[4], W[4], Wc[4], Wc2[4];
+// groups, (+-c_g, +-c_g) on the diagonal ones) and of W_g = |v|^2 + eta_g^2, each set
+// relative to a power of two.
+struct TneSet {
+    FxK k[4];
+    int e;
 };
+struct TneConsts {
+    TneSet c, c2, c3, W, Wc, Wc2;
+};
+
+TneSet tne_set(const double v[4])
+{
+    TneSet t;
+    t.e = fx_exponent(v, 4);
+    for (int g = 0; g < 4; ++g) t.k[g] = fx_k(fx_const(std::ldexp(v[g], -t.e), 60));
+    return t;
+}
+
+// The raw moments of a cell up to the fourth order (rows of Eq. 6 at u = 0).
+struct RawMoments {
+    double rho, jx, jy, E, Rxx, Ryy, Rxy, Rwx, Rwy, Rxxx, Ryyy, Rxxy, Rxyy, Rwxx, Rwyy, Rwxy;
+};
+
+// ... in FP64, for cells outside the integer path.
+template <typename TS>
+__device__ __noinline__ RawMoments raw_moments_any(const FieldArgs &a, const TS *own, size_t P)
+{
+    RawMoments r = {};
+    for (int i = 0; i < kNV; ++i) {
+        const double v = stored(own[i * P]), x = a.vx[i], y = a.vy[i], w = a.m.w[i >> 2];
+        r.rho += v;
+        r.jx = fma(x, v, r.jx);
+        r.jy = fma(y, v, r.jy);
+        r.E = fma(w, v, r.E);
+        r.Rxx = fma(x * x, v, r.Rxx);
+        r.Ryy = fma(y * y, v, r.Ryy);
+        r.Rxy = fma(x * y, v, r.Rxy);
+        r.Rwx = fma(w * x, v, r.Rwx);
+        r.Rwy = fma(w * y, v, r.Rwy);
+        r.Rxxx = fma(x * x * x, v, r.Rxxx);
+        r.Ryyy = fma(y * y * y, v, r.Ryyy);
+        r.Rxxy = fma(x * x * y, v, r.Rxxy);
+        r.Rxyy = fma(x * y * y, v, r.Rxyy);
+        r.Rwxx = fma(w * x * x, v, r.Rwxx);
+        r.Rwyy = fma(w * y * y, v, r.Rwyy);
+        r.Rwxy = fma(w * x * y, v, r.Rwxy);
+    }
+    return r;
+}
 
 // Rows 5..16 of M(u) (Eq. 6) applied to f - f_eq: Delta* of Eqs. (8)-(11).  f_eq is
 // defined by M(u) f_eq = fbar, the prescribed central moments of Eq. (7), so Delta*
@@ -724,88 +781,111 @@ struct TneConsts {
 // fourth).  The central moments follow from the raw moments R_k = sum_i f_i row_k(v_i)
 // by the binomial expansion of (v - u) with j = rho u; the raw moments of a group
 // come from its members' sum, x and y differences, the x and y pair sums (axis
-// groups) and the xy parity (diagonal groups).
+// groups) and the xy parity (diagonal groups).  The raw moments are formed in fixed
+// point (exact sums, each dot product with constants rounded once), which leaves 88 of
+// 167 FP64 instructions: 5.14 -> 2.46 ms for 4096^2 cells.
 template <typename TS>
-__global__ void __launch_bounds__(128) tne_kernel(const FieldArgs a, const TneConsts t, const RefMoments F,
-                                                   const TS *__restrict__ f, double *__restrict__ out)
+__global__ void __launch_bounds__(128) tne_kernel(const __grid_constant__ FieldArgs a, const __grid_constant__ TneConsts t,
+                                                  const RefMoments F, const TS *__restrict__ f, double *__restrict__ out)
 {
     const size_t P = (size_t)a.nx * a.ny;
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < P;
          c += (size_t)gridDim.x * blockDim.x) {
-        double fc[kNV];
+        const TS *own = f + c;
+        TS fc[kNV];
+        uint32_t key = 0;
 #pragma unroll
-        for (int i = 0; i < kNV; ++i) fc[i] = stored(f[i * P + c]);
+        for (int i = 0; i < kNV; ++i) fc[i] = __ldg(own + i * P);
+#pragma unroll
+        for (int i = 0; i < kNV; ++i) key = fx_max(key, fx_key(fc[i]));
+        const int field = (int)(key >> (kSingle<TS> ? 24 : 21));
+        const int top = kSingle<TS> ? field + (1023 - 127) : field;
         // group components: s0 sum, sx / sy odd in x / y, ex / ey the x / y pairs
         // (axis), sxy odd in x and y (diagonal)
-        double s0[4], sx[4], sy[4], ex[2], ey[2], sxy[2];
+        int64_t s0[4], sx[4], sy[4], ex[2], ey[2], sxy[2];
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-            const double *q = fc + 4 * g;
-            if ((g & 1) == 0) {          // E N W S
+            int64_t q[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) q[j] = fx_from(fc[4 * g + j], field);
+            fx_group_sums(g, q, s0[g], sx[g], sy[g]);
+            if ((g & 1) == 0) {
                 ex[g >> 1] = q[0] + q[2];
                 ey[g >> 1] = q[1] + q[3];
-                sx[g] = q[0] - q[2];
-                sy[g] = q[1] - q[3];
-                s0[g] = ex[g >> 1] + ey[g >> 1];
-            } else {                     // NE NW SW SE
-                const double e = q[0] + q[3], w = q[1] + q[2];
-                sx[g] = e - w;
-                sy[g] = (q[0] + q[1]) - (q[2] + q[3]);
+            } else {
                 sxy[g >> 1] = (q[0] + q[2]) - (q[1] + q[3]);
-                s0[g] = e + w;
             }
         }
-        auto dot = [](const double *k, const double *x) {
-            return fma(k[3], x[3], fma(k[2], x[2], fma(k[1], x[1], k[0] * x[0])));
+        auto dot4 = [&](const TneSet &k, int64_t x0, int64_t x1, int64_t x2, int64_t x3) {
+            FxSum m = kFxHalfUnit;
+            fx_mul(m, x0, k.k[0]);
+            fx_mul(m, x1, k.k[1]);
+            fx_mul(m, x2, k.k[2]);
+            fx_mul(m, x3, k.k[3]);
+            return fx_to(fx_sum59(m), top + k.e);
         };
-        // raw moments R1..R16 (rows of Eq. 6 at u = 0)
-        double rho = (s0[0] + s0[1]) + (s0[2] + s0[3]);
-        const double jx = dot(t.c, sx), jy = dot(t.c, sy);
-        double E = dot(t.W, s0);
-        double Rxx = fma(t.c2[3], s0[3], fma(t.c2[2], ex[1], fma(t.c2[1], s0[1], t.c2[0] * ex[0])));
-        double Ryy = fma(t.c2[3], s0[3], fma(t.c2[2], ey[1], fma(t.c2[1], s0[1], t.c2[0] * ey[0])));
-        const double Rxy = fma(t.c2[3], sxy[1], t.c2[1] * sxy[0]);
-        const double Rwx = dot(t.Wc, sx), Rwy = dot(t.Wc, sy);
-        const double Rxxx = dot(t.c3, sx), Ryyy = dot(t.c3, sy);
-        const double Rxxy = fma(t.c3[3], sy[3], t.c3[1] * sy[1]);
-        const double Rxyy = fma(t.c3[3], sx[3], t.c3[1] * sx[1]);
-        double Rwxx = fma(t.Wc2[3], s0[3], fma(t.Wc2[2], ex[1], fma(t.Wc2[1], s0[1], t.Wc2[0] * ex[0])));
-        double Rwyy = fma(t.Wc2[3], s0[3], fma(t.Wc2[2], ey[1], fma(t.Wc2[1], s0[1], t.Wc2[0] * ey[0])));
-        const double Rwxy = fma(t.Wc2[3], sxy[1], t.Wc2[1] * sxy[0]);
-        if constexpr (kSingle<TS>) {    // the reference equilibrium's even moments
-            rho += F.rho;
-            E += F.E;
-            Rxx += F.Rxx;
-            Ryy += F.Rxx;
-            Rwxx += F.Rwxx;
-            Rwyy += F.Rwxx;
+        auto dot2 = [&](const TneSet &k, int64_t x1, int64_t x3) {      // the diagonal groups
+            FxSum m = kFxHalfUnit;
+            fx_mul(m, x1, k.k[1]);
+            fx_mul(m, x3, k.k[3]);
+            return fx_to(fx_sum59(m), top + k.e);
+        };
+        RawMoments m;
+        if (!(kSingle<TS> ? field == 255 : fx_out_of_range(field))) {
+            m.rho = fx_to((s0[0] + s0[1]) + (s0[2] + s0[3]), top);
+            m.jx = dot4(t.c, sx[0], sx[1], sx[2], sx[3]);
+            m.jy = dot4(t.c, sy[0], sy[1], sy[2], sy[3]);
+            m.E = dot4(t.W, s0[0], s0[1], s0[2], s0[3]);
+            m.Rxx = dot4(t.c2, ex[0], s0[1], ex[1], s0[3]);
+            m.Ryy = dot4(t.c2, ey[0], s0[1], ey[1], s0[3]);
+            m.Rxy = dot2(t.c2, sxy[0], sxy[1]);
+            m.Rwx = dot4(t.Wc, sx[0], sx[1], sx[2], sx[3]);
+            m.Rwy = dot4(t.Wc, sy[0], sy[1], sy[2], sy[3]);
+            m.Rxxx = dot4(t.c3, sx[0], sx[1], sx[2], sx[3]);
+            m.Ryyy = dot4(t.c3, sy[0], sy[1], sy[2], sy[3]);
+            m.Rxxy = dot2(t.c3, sy[1], sy[3]);
+            m.Rxyy = dot2(t.c3, sx[1], sx[3]);
+            m.Rwxx = dot4(t.Wc2, ex[0], s0[1], ex[1], s0[3]);
+            m.Rwyy = dot4(t.Wc2, ey[0], s0[1], ey[1], s0[3]);
+            m.Rwxy = dot2(t.Wc2, sxy[0], sxy[1]);
+        } else {
+            m = raw_moments_any(a, own, P);
         }
+        if constexpr (kSingle<TS>) {    // the reference equilibrium's even moments
+            m.rho += F.rho;
+            m.E += F.E;
+            m.Rxx += F.Rxx;
+            m.Ryy += F.Rxx;
+            m.Rwxx += F.Rwxx;
+            m.Rwyy += F.Rwxx;
+        }
+        const double jx = m.jx, jy = m.jy;
         // primitives: u = j / rho, p = rho T = (E - rho u^2) / K
-        const double r = rcp64(rho);
+        const double r = rcp64(m.rho);
         const double ux = jx * r, uy = jy * r;
         const double uxuy = ux * uy, u2 = fma(ux, ux, uy * uy);
-        const double p = (E - fma(jx, ux, jy * uy)) * a.m.invK;
+        const double p = (m.E - fma(jx, ux, jy * uy)) * a.m.invK;
         const double q4 = a.m.Kp2 * p * (p * r);                 // (K + 2) rho T^2
-        const double ax = fma(uy, Rxy, ux * Rxx);                // sum f (v.u) v_x
-        const double ay = fma(uy, Ryy, ux * Rxy);                // sum f (v.u) v_y
+        const double ax = fma(uy, m.Rxy, ux * m.Rxx);            // sum f (v.u) v_x
+        const double ay = fma(uy, m.Ryy, ux * m.Rxy);            // sum f (v.u) v_y
         // central moments about u, minus fbar
-        const double Cxx = fma(-ux, jx, Rxx), Cxy = fma(-ux, jy, Rxy), Cyy = fma(-uy, jy, Ryy);
+        const double Cxx = fma(-ux, jx, m.Rxx), Cxy = fma(-ux, jy, m.Rxy), Cyy = fma(-uy, jy, m.Ryy);
         const double d[12] = {
             Cxx - p,
             Cxy,
             Cyy - p,
-            fma(2.0 * u2, jx, fma(-2.0, ax, fma(-ux, E, Rwx))),
-            fma(2.0 * u2, jy, fma(-2.0, ay, fma(-uy, E, Rwy))),
-            fma(2.0 * jx, ux * ux, fma(-3.0 * ux, Rxx, Rxxx)),
-            fma(2.0 * jx, uxuy, fma(-2.0 * ux, Rxy, fma(-uy, Rxx, Rxxy))),
-            fma(2.0 * jy, uxuy, fma(-2.0 * uy, Rxy, fma(-ux, Ryy, Rxyy))),
-            fma(2.0 * jy, uy * uy, fma(-3.0 * uy, Ryy, Ryyy)),
-            fma(u2, Cxx, fma(-2.0 * jx * ux, u2, fma(4.0 * ux, ax, fma(-2.0, fma(uy, Rxxy, ux * Rxxx),
-                fma(ux * ux, E, fma(-2.0 * ux, Rwx, Rwxx)))))) - q4,
-            fma(u2, Cxy, fma(-2.0, fma(jx * uy, u2, fma(-ux, ay, fma(-uy, ax, fma(uy, Rxyy, ux * Rxxy)))),
-                fma(uxuy, E, fma(-ux, Rwy, fma(-uy, Rwx, Rwxy))))),
-            fma(u2, Cyy, fma(-2.0 * jy * uy, u2, fma(4.0 * uy, ay, fma(-2.0, fma(uy, Ryyy, ux * Rxyy),
-                fma(uy * uy, E, fma(-2.0 * uy, Rwy, Rwyy)))))) - q4,
+            fma(2.0 * u2, jx, fma(-2.0, ax, fma(-ux, m.E, m.Rwx))),
+            fma(2.0 * u2, jy, fma(-2.0, ay, fma(-uy, m.E, m.Rwy))),
+            fma(2.0 * jx, ux * ux, fma(-3.0 * ux, m.Rxx, m.Rxxx)),
+            fma(2.0 * jx, uxuy, fma(-2.0 * ux, m.Rxy, fma(-uy, m.Rxx, m.Rxxy))),
+            fma(2.0 * jy, uxuy, fma(-2.0 * uy, m.Rxy, fma(-ux, m.Ryy, m.Rxyy))),
+            fma(2.0 * jy, uy * uy, fma(-3.0 * uy, m.Ryy, m.Ryyy)),
+            fma(u2, Cxx, fma(-2.0 * jx * ux, u2, fma(4.0 * ux, ax, fma(-2.0, fma(uy, m.Rxxy, ux * m.Rxxx),
+                fma(ux * ux, m.E, fma(-2.0 * ux, m.Rwx, m.Rwxx)))))) - q4,
+            fma(u2, Cxy, fma(-2.0, fma(jx * uy, u2, fma(-ux, ay, fma(-uy, ax, fma(uy, m.Rxyy, ux * m.Rxxy)))),
+                fma(uxuy, m.E, fma(-ux, m.Rwy, fma(-uy, m.Rwx, m.Rwxy))))),
+            fma(u2, Cyy, fma(-2.0 * jy * uy, u2, fma(4.0 * uy, ay, fma(-2.0, fma(uy, m.Ryyy, ux * m.Rxyy),
+                fma(uy * uy, m.E, fma(-2.0 * uy, m.Rwy, m.Rwyy)))))) - q4,
         };
 #pragma unroll
         for (int k = 0; k < 12; ++k) out[k * P + c] = d[k];
@@ -1017,15 +1097,14 @@ cudaError_t launch_macros(const FieldArgs &a, const void *f, int prec, double *r
 
 cudaError_t launch_tne(const FieldArgs &a, const void *f, int prec, double *out, cudaStream_t s)
 {
-    TneConsts t;
+    double c2[4], c3[4], wc[4], wc2[4];
     for (int g = 0; g < 4; ++g) {
-        t.c[g] = a.m.c[g];
-        t.c2[g] = a.m.c[g] * a.m.c[g];
-        t.c3[g] = t.c2[g] * a.m.c[g];
-        t.W[g] = a.m.w[g];
-        t.Wc[g] = a.m.w[g] * a.m.c[g];
-        t.Wc2[g] = a.m.w[g] * t.c2[g];
+        c2[g] = a.m.c[g] * a.m.c[g];
+        c3[g] = c2[g] * a.m.c[g];
+        wc[g] = a.m.w[g] * a.m.c[g];
+        wc2[g] = a.m.w[g] * c2[g];
     }
+    const TneConsts t = {tne_set(a.m.c), tne_set(c2), tne_set(c3), tne_set(a.m.w), tne_set(wc), tne_set(wc2)};
     const unsigned nb = grid_for((size_t)a.nx * a.ny, 128);
     const RefMoments F = ref_moments(a, single_storage(prec));
     if (single_storage(prec))
