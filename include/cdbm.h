@@ -160,7 +160,7 @@ cdbm_status cdbm_step(cdbm_ctx *ctx, int nsteps);
 
 /* Enables (default) or disables the small-grid paths of cdbm_step: on 1-D grids the
  * persistent cluster kernel, and for CDBM_FP64 the stage kernels that split each cell
- * over four threads (grids of up to about 29000 cells; on 2-D grids the results are the
+ * over four or two threads (grids of up to about 67000 cells; on 2-D grids the results are the
  * same bit for bit).  Disabled, those grids step with the one-cell-per-thread stage
  * kernel like any other. */
 cdbm_status cdbm_set_small_grid_path(cdbm_ctx *ctx, int enable);

@@ -390,8 +390,7 @@ __global__ void __launch_bounds__(128) batch_init_kernel(const BatchArgs a, cons
         const ClassConsts &C = a.cls[t.cls];
         const double r = rho[c], u = ux[c], v = uy[c], tt = T[c];
         double fe[kNV];
-        if constexpr (kSingle<TS>) equilibrium_of(C.unit, C.m, r, u, v, tt, fe);
-        else fx_equilibrium_of(C.unit, C.m, r, u, v, tt, fe);
+        equilibrium_of(C.unit, C.m, r, u, v, tt, fe);
         if (!(positive_finite(r) && positive_finite(tt) && isfinite(u) && isfinite(v)))
             atomicOr(flag, kFlagNonPhys);
 #pragma unroll

@@ -164,7 +164,8 @@ char *thread_error_buffer();
 cudaError_t launch_init(const FieldArgs &a, const double *rho, const double *ux,
                         const double *uy, const double *T, void *f, int prec, unsigned *flag,
                         cudaStream_t s);
-cudaError_t launch_macros(const FieldArgs &a, const void *f, int prec, double *rho, double *ux,
+// in_double: the sums of a CDBM_FP64 state in FP64 (the read-out of a recorded run).
+cudaError_t launch_macros(const FieldArgs &a, const void *f, int prec, bool in_double, double *rho, double *ux,
                           double *uy, double *T, cudaStream_t s);
 cudaError_t launch_tne(const FieldArgs &a, const void *f, int prec, double *out, cudaStream_t s);
 cudaError_t launch_sums(const FieldArgs &a, const void *f, int prec, double *partials, int nblocks,
@@ -189,12 +190,14 @@ struct StageLaunch {
 StageLaunch stage_launch_config(const StageArgs &a, bool with_base, int sm_count, int prec,
                                 bool allow_march = true, bool allow_split = true);
 
+// The all-FP64 stage kernels (cdbm_stage_double.cu) of the run that the adjoint
+// differentiates.
+StageLaunch double_stage_launch_config(const StageArgs &a, bool with_base, int sm_count, bool allow_march,
+                                       bool allow_split);
+
 // FP64 stage kernel for 1-D grids with each cell split over four threads
 // (cdbm_small1d.cu): kSplitFlatThreads threads per block, 4 nx threads in all.
 constexpr int kSplitFlatThreads = 128;
-constexpr int kSplitFlatMaxCells = 4096;    // measured per stage against the fixed-point form with a
-                                            // warp per group: 5.6 / 6.4 us at 2000 cells, 5.4 / 6.3 at
-                                            // 4096, 8.8 / 6.4 at 8192
 void *split_flat_func(bool with_base);
 cudaError_t launch_stage(const StageLaunch &L, const void *g, const void *base, void *out,
                          const StageArgs &a, unsigned *flag, cudaStream_t s);

@@ -34,10 +34,11 @@ constexpr int stage_min_blocks(int eq) { return eq != kEqDouble ? CDBM_STAGE_MIN
 
 // ---------------------------------------------------------------- init (K0)
 
-// f_eq of the fields.  Bound by the FP64 pipe: 62 instructions with the members rebuilt in
-// fixed point (fx_equilibrium_of; 86 before, 2.60 -> 1.99 ms for 4096^2 cells), 102 for a
-// single-precision state, whose values have to round as they always did (118 before the
-// narrowing left the pipe, 3.87 -> 3.26 ms with the means of rho and T).
+// f_eq of the fields.  Bound by the FP64 pipe: 86 instructions (2.60 ms for 4096^2 cells),
+// 102 for a single-precision state (118 before the narrowing left the pipe, 3.87 -> 3.26
+// ms with the means of rho and T).  Rebuilding the members in fixed point took 62 and
+// 1.99 ms, but the initial state is also the adjoint's, whose dL/dtau must not change
+// (cdbm_stage_double.cu).
 template <typename TS>
 __global__ void __launch_bounds__(128) init_kernel(const FieldArgs a, const double *__restrict__ rho,
                                                     const double *__restrict__ ux,
@@ -50,8 +51,7 @@ __global__ void __launch_bounds__(128) init_kernel(const FieldArgs a, const doub
          c += (size_t)gridDim.x * blockDim.x) {
         const double r = rho[c], u = ux[c], v = uy[c], t = T[c];
         double fe[kNV];
-        if constexpr (kSingle<TS>) equilibrium_of(a.eq, a.m, r, u, v, t, fe);
-        else fx_equilibrium_of(a.eq, a.m, r, u, v, t, fe);
+        equilibrium_of(a.eq, a.m, r, u, v, t, fe);
         if (!(positive_finite(r) && positive_finite(t) && isfinite(u) && isfinite(v)))
             atomicOr(flag, kFlagNonPhys);
 #pragma unroll
@@ -174,7 +174,7 @@ struct GridCell {
 // warps per SM, 7.0 as here at 32), but the code outgrows the instruction cache as soon
 // as other paths run beside it (1500 x 1300 piecewise-constant fields: 1.9 against
 // 1.27 ms).
-template <bool kDiag, bool kFlatY, bool kBase, bool kWide>
+template <int kUnroll, bool kDiag, bool kFlatY, bool kBase, bool kWide>
 __device__ __forceinline__ void fx_grid_group(const double *g, const double *base, double *out, const StageArgs &a,
                                               const GridStencil<kWide> &st, size_t P, int x, int y, int grp,
                                               const FxGroup h, bool cell_ok, bool live, unsigned *flag)
@@ -211,12 +211,12 @@ __device__ __forceinline__ void fx_grid_group(const double *g, const double *bas
         else rest |= 1u << j;
     };
     if constexpr (!kDiag && kFlatY) {
-#pragma unroll 1
+#pragma unroll kUnroll
         for (int j = 0; j < 4; j += 2) pass(j, std::true_type{});
-#pragma unroll 1
+#pragma unroll kUnroll
         for (int j = 1; j < 4; j += 2) pass(j, std::false_type{});    // N, S of a 1-D grid: no transport
     } else {
-#pragma unroll 1
+#pragma unroll kUnroll
         for (int j = 0; j < 4; ++j) pass(j, std::true_type{});
     }
     if (rest && live)
@@ -245,60 +245,77 @@ __global__ void __launch_bounds__(kStageThreads, kFxMinBlocks)
         const EqFactors q = eq_factors(a.m, m.rho, m.jx, m.jy, m.E, flag);
 #pragma unroll 1
         for (int p = 0; p < 4; p += 2) {
-            fx_grid_group<false, kFlatY, kBase>(g, base, out, a, st, P, x, y, p, fx_group(a.eq, q, p), m.ok, true, flag);
-            fx_grid_group<true, kFlatY, kBase>(g, base, out, a, st, P, x, y, p + 1, fx_group(a.eq, q, p + 1), m.ok, true,
+            fx_grid_group<1, false, kFlatY, kBase>(g, base, out, a, st, P, x, y, p, fx_group(a.eq, q, p), m.ok, true, flag);
+            fx_grid_group<1, true, kFlatY, kBase>(g, base, out, a, st, P, x, y, p + 1, fx_group(a.eq, q, p + 1), m.ok, true,
                                                flag);
         }
     }
 }
 
-// The same stage with the four velocity groups of 32 cells on the four warps of a block:
-// on a small grid the time of a stage is the chain of one thread, which this shortens
-// about threefold.  The warps exchange the groups' largest exponents and sums through
-// shared memory, and each forms the moments and the factors of the equilibrium; the
-// values are those of stage_fx_kernel.
-template <bool kBase, bool kFlatY>
-__global__ void __launch_bounds__(128)
+// The same stage with the velocity groups of a cell on kWays (4 or 2) warps of a block:
+// on a small grid the time of a stage is the chain of one thread, which this shortens.
+// The warps of 32 cells exchange their groups' largest exponents and sums through shared
+// memory, and each forms the moments and the factors of the equilibrium; the values are
+// those of stage_fx_kernel.  With few warps per SM the members' passes are unrolled so
+// that their chains overlap.  Blocks per SM (registers): 6 for four ways and 4 for two, so
+// that the sizes below which each is used fit one wave (at 4 blocks, four ways jumped
+// from 15.5 us at 128^2 to 24 us at 144^2).
+template <int kWays, bool kBase, bool kFlatY>
+__global__ void __launch_bounds__(128, kWays == 4 ? 6 : 4)
     stage_fx_split_kernel(const double *__restrict__ g, const double *base, double *out,
                           const __grid_constant__ StageArgs a, unsigned *flag)
 {
-    __shared__ uint32_t keys[4][32];
-    __shared__ int64_t sums[4][3][32];
-    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-    const int x0 = blockIdx.x * 32 + lane;
+    constexpr int kCells = 128 / kWays, kGroups = 4 / kWays;
+    __shared__ uint32_t keys[kWays][kCells];
+    __shared__ int64_t sums[4][3][kCells];
+    const int warp = threadIdx.x >> 5;
+    const int way = warp % kWays, at = warp / kWays * 32 + (threadIdx.x & 31);
+    const int x0 = blockIdx.x * kCells + at;
     const bool live = x0 < a.nx;
     const int x = live ? x0 : a.nx - 1;              // idle lanes mirror the last cell
     const size_t P = (size_t)a.nx * a.ny;
     GridStencil<true> st(x, a.nx, a.bc_x);
     for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
         st.template at_row<kFlatY>(y, a.nx, a.ny, a.bc_y);
-        const double *own = g + (size_t)(4 * grp) * P + st.row + x;
-        double f[4];
+        const double *own = g + (size_t)(4 * kGroups * way) * P + st.row + x;
+        double f[4 * kGroups];
         uint32_t key = 0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < 4 * kGroups; ++j) {
             f[j] = __ldg(own + j * P);
             key = fx_max(key, fx_key(f[j]));
         }
-        keys[grp][lane] = key;
+        keys[way][at] = key;
         __syncthreads();
-        const int top = (int)(fx_max(fx_max(keys[0][lane], keys[1][lane]), fx_max(keys[2][lane], keys[3][lane])) >> 21);
-        int64_t q4[4], s0, sx, sy;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) q4[j] = fx_from(f[j], top);
-        fx_group_sums(grp, q4, s0, sx, sy);
-        sums[grp][0][lane] = s0;
-        sums[grp][1][lane] = sx;
-        sums[grp][2][lane] = sy;
+        for (int w = 0; w < kWays; ++w) key = fx_max(key, keys[w][at]);
+        const int top = (int)(key >> 21);
+#pragma unroll
+        for (int k = 0; k < kGroups; ++k) {
+            const int grp = kGroups * way + k;
+            int64_t q4[4], s0, sx, sy;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) q4[j] = fx_from(f[4 * k + j], top);
+            fx_group_sums(grp, q4, s0, sx, sy);
+            sums[grp][0][at] = s0;
+            sums[grp][1][at] = sx;
+            sums[grp][2][at] = sy;
+        }
         __syncthreads();
         FxMoments mo = kFxNoMoments;
 #pragma unroll
-        for (int h = 0; h < 4; ++h) fx_add_sums(a.fx.m, h, sums[h][0][lane], sums[h][1][lane], sums[h][2][lane], mo);
+        for (int h = 0; h < 4; ++h) fx_add_sums(a.fx.m, h, sums[h][0][at], sums[h][1][at], sums[h][2][at], mo);
         const FxCons m = fx_round_moments(a.fx.m, mo, top);
         const EqFactors q = eq_factors(a.m, m.rho, m.jx, m.jy, m.E, flag);
-        const FxGroup h = fx_group(a.eq, q, grp);
-        if ((grp & 1) == 0) fx_grid_group<false, kFlatY, kBase>(g, base, out, a, st, P, x, y, grp, h, m.ok, live, flag);
-        else fx_grid_group<true, kFlatY, kBase>(g, base, out, a, st, P, x, y, grp, h, m.ok, live, flag);
+        const int grp = kGroups * way;
+        if (kGroups == 2 || (grp & 1) == 0)
+            fx_grid_group<4, false, kFlatY, kBase>(g, base, out, a, st, P, x, y, grp, fx_group(a.eq, q, grp), m.ok,
+                                                         live, flag);
+        if (kGroups == 2 || (grp & 1) == 1) {
+            const int odd = grp | 1;
+            fx_grid_group<4, true, kFlatY, kBase>(g, base, out, a, st, P, x, y, odd, fx_group(a.eq, q, odd), m.ok,
+                                                        live, flag);
+        }
         // the next row writes keys[] only after every warp has passed the second barrier
     }
 }
@@ -695,7 +712,8 @@ __device__ __noinline__ Cons conserved_any(const FieldArgs &a, const TS *own, si
     return conserved(fc, a.m);
 }
 
-template <typename TS>
+// kDouble: all in FP64, for the read-out of a recorded run (cdbm_stage_double.cu).
+template <typename TS, bool kDouble>
 __global__ void __launch_bounds__(128) macros_kernel(const __grid_constant__ FieldArgs a, const RefMoments F,
                                                      const TS *__restrict__ f, double *rho, double *ux, double *uy,
                                                      double *T)
@@ -704,9 +722,17 @@ __global__ void __launch_bounds__(128) macros_kernel(const __grid_constant__ Fie
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < P;
          c += (size_t)gridDim.x * blockDim.x) {
         const TS *own = f + c;
-        const FxCons m = fx_conserved(a.fx, [=](int i) { return __ldg(own + i * P); });
-        Cons q = {m.rho, m.jx, m.jy, m.E};
-        if (!m.ok) q = conserved_any(a, own, P);
+        Cons q;
+        if constexpr (kDouble) {
+            double fc[kNV];
+#pragma unroll
+            for (int i = 0; i < kNV; ++i) fc[i] = stored(__ldg(own + i * P));
+            q = conserved(fc, a.m);
+        } else {
+            const FxCons m = fx_conserved(a.fx, [=](int i) { return __ldg(own + i * P); });
+            q = {m.rho, m.jx, m.jy, m.E};
+            if (!m.ok) q = conserved_any(a, own, P);
+        }
         if constexpr (kSingle<TS>) {
             q.rho += F.rho;
             q.E += F.E;
@@ -1054,10 +1080,12 @@ void *fx_func(bool with_base, bool flat, bool wide)
     return flat ? (void *)stage_fx_kernel<false, true, false> : (void *)stage_fx_kernel<false, false, false>;
 }
 
+template <int kWays>
 void *fx_split_func(bool with_base, bool flat)
 {
-    if (with_base) return flat ? (void *)stage_fx_split_kernel<true, true> : (void *)stage_fx_split_kernel<true, false>;
-    return flat ? (void *)stage_fx_split_kernel<false, true> : (void *)stage_fx_split_kernel<false, false>;
+    if (with_base)
+        return flat ? (void *)stage_fx_split_kernel<kWays, true, true> : (void *)stage_fx_split_kernel<kWays, true, false>;
+    return flat ? (void *)stage_fx_split_kernel<kWays, false, true> : (void *)stage_fx_split_kernel<kWays, false, false>;
 }
 
 template <int kEq>
@@ -1083,15 +1111,17 @@ cudaError_t launch_init(const FieldArgs &a, const double *rho, const double *ux,
     return cudaGetLastError();
 }
 
-cudaError_t launch_macros(const FieldArgs &a, const void *f, int prec, double *rho, double *ux,
+cudaError_t launch_macros(const FieldArgs &a, const void *f, int prec, bool in_double, double *rho, double *ux,
                           double *uy, double *T, cudaStream_t s)
 {
     const unsigned nb = grid_for((size_t)a.nx * a.ny, 128);
     const RefMoments F = ref_moments(a, single_storage(prec));
     if (single_storage(prec))
-        macros_kernel<float><<<nb, 128, 0, s>>>(a, F, (const float *)f, rho, ux, uy, T);
+        macros_kernel<float, false><<<nb, 128, 0, s>>>(a, F, (const float *)f, rho, ux, uy, T);
+    else if (in_double)
+        macros_kernel<double, true><<<nb, 128, 0, s>>>(a, F, (const double *)f, rho, ux, uy, T);
     else
-        macros_kernel<double><<<nb, 128, 0, s>>>(a, F, (const double *)f, rho, ux, uy, T);
+        macros_kernel<double, false><<<nb, 128, 0, s>>>(a, F, (const double *)f, rho, ux, uy, T);
     return cudaGetLastError();
 }
 
@@ -1154,8 +1184,10 @@ StageLaunch stage_launch_config(const StageArgs &a, bool with_base, int sm_count
     StageLaunch L;
     const bool flat = (a.ny == 1);
     const size_t cells = (size_t)a.nx * a.ny;
-    if (allow_split && flat && prec == CDBM_FP64 && a.nx <= kSplitFlatMaxCells) {
-        // short FP64 tubes: four threads per cell shorten the dependent chain of a stage
+    if (allow_split && flat && prec == CDBM_FP64 && a.nx <= sm_count * kSplitFlatThreads / 4) {
+        // Short FP64 tubes, up to one block of the all-FP64 kernel with four threads per
+        // cell on each SM (4864 cells): 5.4-5.6 us per stage, against 6.9 us in fixed
+        // point; with two blocks on an SM 8.8 against 7.3 us.
         L.func = split_flat_func(with_base);
         L.block = dim3(kSplitFlatThreads, 1, 1);
         L.grid = dim3((unsigned)((4 * (size_t)a.nx + kSplitFlatThreads - 1) / kSplitFlatThreads), 1, 1);
@@ -1163,14 +1195,17 @@ StageLaunch stage_launch_config(const StageArgs &a, bool with_base, int sm_count
     }
     if (prec == CDBM_FP64) {
         const unsigned rows = a.ny < 65535 ? a.ny : 65535;
-        // Below half of the threads that stage_fx_kernel keeps resident the time is the
-        // chain of one thread: four threads per cell.  Per stage, split against one
-        // thread per cell: 8.8 / 17.0 us at 64^2, 14.3 / 16.9 at 128^2, 20.8 / 25.4 at
-        // 160^2, 38.2 / 36.2 at 256^2.
-        if (allow_split && cells <= (size_t)sm_count * kFxMinBlocks * kStageThreads / 2) {
-            L.func = fx_split_func(with_base, flat);
+        // While the grid leaves most of the SMs' threads idle, the time is the chain of
+        // one thread, and the cell is split over four or two.  us per stage with four
+        // threads per cell, two and one: 9.4 / 12.6 / 24.5 at 64^2, 13.6 / 14.9 / 25.0 at
+        // 112^2, 15.6 / 14.6 / 24.4 at 128^2, 27.5 / 21.2 / 28.1 at 192^2, 40.6 / 34.8 /
+        // 37.5 at 256^2, 44.3 / 42.3 / 39.8 at 270^2.
+        if (allow_split && cells <= (size_t)sm_count * 440) {
+            const bool four = cells <= (size_t)sm_count * 88;
+            const unsigned per = four ? 32 : 64;
+            L.func = four ? fx_split_func<4>(with_base, flat) : fx_split_func<2>(with_base, flat);
             L.block = dim3(128, 1, 1);
-            L.grid = dim3((unsigned)((a.nx + 31) / 32), rows, 1);
+            L.grid = dim3((unsigned)(((size_t)a.nx + per - 1) / per), rows, 1);
             return L;
         }
         // the widest block whose padding past the row's end is least

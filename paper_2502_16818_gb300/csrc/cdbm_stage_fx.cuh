@@ -184,37 +184,6 @@ __device__ __forceinline__ FxGroup fx_group(const EqBlocks &B, const EqFactors &
     return {A + U, D - V, A - U, D + V, G};
 }
 
-// equilibrium_of() with the members rebuilt in fixed point: 62 instead of 86 FP64
-// instructions.
-__device__ __forceinline__ void fx_equilibrium_of(const EqBlocks &B, const ModelConsts &m, double rho, double u, double v,
-                                                  double T, double out[kNV])
-{
-    EqFactors q;
-    q.rho = rho;
-    q.jx = rho * u;
-    q.jy = rho * v;
-    q.T = T;
-    const double jyuy = __dmul_rn(q.jy, v), P = __dmul_rn(rho, T), v2 = __dmul_rn(v, v);
-    q.ru2 = fma(q.jx, u, jyuy);
-    q.E = fma(m.K, P, q.ru2);
-    q.u2 = fma(u, u, v2);
-    q.dlt = fma(u, u, -v2);
-    q.m1416 = fma(T, fma(m.Kp6, q.ru2, __dmul_rn(m.twoKp2, P)), __dmul_rn(q.ru2, q.u2));
-    q.W4 = fma(m.Kp4, T, q.u2);
-    q.d57 = fma(q.jx, u, -jyuy);
-    q.m6 = q.jx * v;
-    bool ok = true;
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        const FxGroup h = fx_group(B, q, g);
-        ok = ok && !fx_out_of_range(h.G);
-        const int E = h.G - (kGroupLead - kLead);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) out[4 * g + j] = fx_to(h.member(j), E);
-    }
-    if (!ok) equilibrium_of(B, m, rho, u, v, T, out);
-}
-
 // ---- update of a velocity ----
 
 // Cell, its upwind-ordered neighbours (two up, one up, one down) along x and y, and its
