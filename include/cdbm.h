@@ -151,18 +151,17 @@ cdbm_status cdbm_init(cdbm_ctx *ctx, const double *rho, const double *ux, const 
  * 16 velocities -> stage update).  Launches are replayed from a CUDA graph.  A 1-D
  * grid (ny = 1) small enough for one thread-block cluster (at most 16 x 64 cells for
  * CDBM_FP64, 16 x 256 for the three single-precision states) instead runs all nsteps
- * in one persistent launch with its state in the cluster's shared memory; the
- * results are the same bit for bit for the single-precision states and the same to
- * rounding for CDBM_FP64, whose cluster kernel splits each cell over four threads.
+ * in one persistent launch with its state in the cluster's shared memory, with the same
+ * results bit for bit.
  * Asynchronous; a non-physical state is reported by the next cdbm_sync.
  */
 cdbm_status cdbm_step(cdbm_ctx *ctx, int nsteps);
 
 /* Enables (default) or disables the small-grid paths of cdbm_step: on 1-D grids the
  * persistent cluster kernel, and for CDBM_FP64 the stage kernels that split each cell
- * over four or two threads (grids of up to about 67000 cells; on 2-D grids the results are the
- * same bit for bit).  Disabled, those grids step with the one-cell-per-thread stage
- * kernel like any other. */
+ * over 16 or two threads (grids of up to about 67000 cells).  Disabled, those grids step
+ * with the one-cell-per-thread stage kernel like any other, with the same results bit
+ * for bit. */
 cdbm_status cdbm_set_small_grid_path(cdbm_ctx *ctx, int enable);
 
 /* Enables (default) or disables the row-marching stage kernels of the single-precision
@@ -355,10 +354,8 @@ void cdbm_batch_destroy(cdbm_batch *b);
  *                  cdbm_get_state or an equilibrium the caller built), advanced in
  *                  place by nsteps >= 0 two-stage TVD Runge-Kutta steps.  The result
  *                  matches cdbm_step's on the same state to rounding (within 1e-12
- *                  relative max-norm): both apply the same per-cell operations, but
- *                  on a short 1-D grid cdbm_step may run them in its cluster kernel,
- *                  whose compiled arithmetic can round differently.  On 2-D grids
- *                  both run the same stage kernels and agree bit for bit.
+ *                  relative max-norm): both apply the same per-cell operations.  On
+ *                  2-D grids both run the same stage kernels and agree bit for bit.
  *   cuda_stream  : stream for the work (NULL = legacy stream).
  * Scratch: the stage-1 buffer and the error flag live in one fixed device array of
  * the library (16 * CDBM_NOALLOC_MAX_CELLS doubles plus 256 bytes, i.e. 4 MiB), which

@@ -838,10 +838,6 @@ cdbm_status cdbm_adjoint_forward(cdbm_ctx *c, int nsteps, int every)
         if (cuda_check(c, cudaMemcpyAsync(c->ckpt[k], c->f, fb, cudaMemcpyDeviceToDevice, c->stream), "checkpoint"))
             return c->err;
         const int n = (k + 1) * every <= nsteps ? every : nsteps - k * every;
-        if (c->small.ok && c->small_enabled) {
-            if (cdbm_step(c, n)) return c->err;      // the cluster kernel is FP64 throughout
-            continue;
-        }
         for (int s = 0; s < n; ++s) {
             cudaError_t e = launch_stage(c->adj_launch[0], c->f, nullptr, c->f1, c->stage[0], c->flag, c->stream);
             if (e == cudaSuccess)

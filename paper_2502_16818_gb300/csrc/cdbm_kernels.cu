@@ -252,47 +252,42 @@ __global__ void __launch_bounds__(kStageThreads, kFxMinBlocks)
     }
 }
 
-// The same stage with the velocity groups of a cell on kWays (4 or 2) warps of a block:
-// on a small grid the time of a stage is the chain of one thread, which this shortens.
-// The warps of 32 cells exchange their groups' largest exponents and sums through shared
-// memory, and each forms the moments and the factors of the equilibrium; the values are
-// those of stage_fx_kernel.  With few warps per SM the members' passes are unrolled so
-// that their chains overlap.  Blocks per SM (registers): 6 for four ways and 4 for two, so
-// that the sizes below which each is used fit one wave (at 4 blocks, four ways jumped
-// from 15.5 us at 128^2 to 24 us at 144^2).
-template <int kWays, bool kBase, bool kFlatY>
-__global__ void __launch_bounds__(128, kWays == 4 ? 6 : 4)
+// The same stage with a cell on two threads: on a grid of some ten thousand cells the time
+// of a stage is the chain of one thread, which this shortens.  Two warps of a block have
+// two velocity groups of 32 cells each; they exchange the groups' largest exponents and
+// sums through shared memory, and each forms the moments and the factors of the
+// equilibrium.  The values are those of stage_fx_kernel.  With few warps per SM the
+// members' passes are unrolled so that their chains overlap.
+template <bool kBase, bool kFlatY>
+__global__ void __launch_bounds__(128, 4)
     stage_fx_split_kernel(const double *__restrict__ g, const double *base, double *out,
                           const __grid_constant__ StageArgs a, unsigned *flag)
 {
-    constexpr int kCells = 128 / kWays, kGroups = 4 / kWays;
-    __shared__ uint32_t keys[kWays][kCells];
-    __shared__ int64_t sums[4][3][kCells];
+    __shared__ uint32_t keys[2][64];
+    __shared__ int64_t sums[4][3][64];
     const int warp = threadIdx.x >> 5;
-    const int way = warp % kWays, at = warp / kWays * 32 + (threadIdx.x & 31);
-    const int x0 = blockIdx.x * kCells + at;
+    const int way = warp & 1, at = (warp >> 1) * 32 + (threadIdx.x & 31);
+    const int x0 = blockIdx.x * 64 + at;
     const bool live = x0 < a.nx;
     const int x = live ? x0 : a.nx - 1;              // idle lanes mirror the last cell
     const size_t P = (size_t)a.nx * a.ny;
     GridStencil<true> st(x, a.nx, a.bc_x);
     for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
         st.template at_row<kFlatY>(y, a.nx, a.ny, a.bc_y);
-        const double *own = g + (size_t)(4 * kGroups * way) * P + st.row + x;
-        double f[4 * kGroups];
+        const double *own = g + (size_t)(8 * way) * P + st.row + x;
+        double f[8];
         uint32_t key = 0;
 #pragma unroll
-        for (int j = 0; j < 4 * kGroups; ++j) {
+        for (int j = 0; j < 8; ++j) {
             f[j] = __ldg(own + j * P);
             key = fx_max(key, fx_key(f[j]));
         }
         keys[way][at] = key;
         __syncthreads();
+        const int top = (int)(fx_max(keys[0][at], keys[1][at]) >> 21);
 #pragma unroll
-        for (int w = 0; w < kWays; ++w) key = fx_max(key, keys[w][at]);
-        const int top = (int)(key >> 21);
-#pragma unroll
-        for (int k = 0; k < kGroups; ++k) {
-            const int grp = kGroups * way + k;
+        for (int k = 0; k < 2; ++k) {
+            const int grp = 2 * way + k;
             int64_t q4[4], s0, sx, sy;
 #pragma unroll
             for (int j = 0; j < 4; ++j) q4[j] = fx_from(f[4 * k + j], top);
@@ -307,16 +302,37 @@ __global__ void __launch_bounds__(128, kWays == 4 ? 6 : 4)
         for (int h = 0; h < 4; ++h) fx_add_sums(a.fx.m, h, sums[h][0][at], sums[h][1][at], sums[h][2][at], mo);
         const FxCons m = fx_round_moments(a.fx.m, mo, top);
         const EqFactors q = eq_factors(a.m, m.rho, m.jx, m.jy, m.E, flag);
-        const int grp = kGroups * way;
-        if (kGroups == 2 || (grp & 1) == 0)
-            fx_grid_group<4, false, kFlatY, kBase>(g, base, out, a, st, P, x, y, grp, fx_group(a.eq, q, grp), m.ok,
-                                                         live, flag);
-        if (kGroups == 2 || (grp & 1) == 1) {
-            const int odd = grp | 1;
-            fx_grid_group<4, true, kFlatY, kBase>(g, base, out, a, st, P, x, y, odd, fx_group(a.eq, q, odd), m.ok,
-                                                        live, flag);
-        }
+        const int grp = 2 * way;
+        fx_grid_group<4, false, kFlatY, kBase>(g, base, out, a, st, P, x, y, grp, fx_group(a.eq, q, grp), m.ok, live, flag);
+        fx_grid_group<4, true, kFlatY, kBase>(g, base, out, a, st, P, x, y, grp + 1, fx_group(a.eq, q, grp + 1), m.ok, live,
+                                              flag);
         // the next row writes keys[] only after every warp has passed the second barrier
+    }
+}
+
+// The same stage with a cell on 16 threads (fx_cell16): 512 threads per 32 cells of a row.
+template <bool kBase, bool kFlatY>
+__global__ void __launch_bounds__(512, 2)
+    stage_fx_cell16_kernel(const double *__restrict__ g, const double *base, double *out,
+                           const __grid_constant__ StageArgs a, unsigned *flag)
+{
+    __shared__ FxCells16 s;
+    const int w = threadIdx.x >> 5, i = cell16_velocity(w);
+    const int x0 = blockIdx.x * 32 + (int)(threadIdx.x & 31);
+    const bool live = x0 < a.nx;
+    const int x = live ? x0 : a.nx - 1;              // idle lanes mirror the last cell
+    for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
+        const GridCell cell = {g, base, out, a.nx, a.ny, a.bc_x, a.bc_y, x, y};
+        const FxStencil v = cell.stencil<kFlatY>(i, dirx(i), kFlatY ? 0 : diry(i), kBase ? cell.base(i) : 0.0);
+        double o;
+        const bool ok = fx_cell16<kFlatY, kBase>(a, s, w, 0, i, v, flag, o);
+        if (live) {
+            if (ok) cell.put(i, o);
+            else
+                fx_double_group<GridCell, kBase, kFlatY>(cell, a.eq, a.m, {a.a_self, a.a_base, a.lx, a.ly}, i >> 2,
+                                                         1u << (i & 3), flag);
+        }
+        // the next row's first write to what this row still reads (s.h) follows two barriers
     }
 }
 
@@ -1080,12 +1096,16 @@ void *fx_func(bool with_base, bool flat, bool wide)
     return flat ? (void *)stage_fx_kernel<false, true, false> : (void *)stage_fx_kernel<false, false, false>;
 }
 
-template <int kWays>
 void *fx_split_func(bool with_base, bool flat)
 {
-    if (with_base)
-        return flat ? (void *)stage_fx_split_kernel<kWays, true, true> : (void *)stage_fx_split_kernel<kWays, true, false>;
-    return flat ? (void *)stage_fx_split_kernel<kWays, false, true> : (void *)stage_fx_split_kernel<kWays, false, false>;
+    if (with_base) return flat ? (void *)stage_fx_split_kernel<true, true> : (void *)stage_fx_split_kernel<true, false>;
+    return flat ? (void *)stage_fx_split_kernel<false, true> : (void *)stage_fx_split_kernel<false, false>;
+}
+
+void *fx_cell16_func(bool with_base, bool flat)
+{
+    if (with_base) return flat ? (void *)stage_fx_cell16_kernel<true, true> : (void *)stage_fx_cell16_kernel<true, false>;
+    return flat ? (void *)stage_fx_cell16_kernel<false, true> : (void *)stage_fx_cell16_kernel<false, false>;
 }
 
 template <int kEq>
@@ -1184,27 +1204,19 @@ StageLaunch stage_launch_config(const StageArgs &a, bool with_base, int sm_count
     StageLaunch L;
     const bool flat = (a.ny == 1);
     const size_t cells = (size_t)a.nx * a.ny;
-    if (allow_split && flat && prec == CDBM_FP64 && a.nx <= sm_count * kSplitFlatThreads / 4) {
-        // Short FP64 tubes, up to one block of the all-FP64 kernel with four threads per
-        // cell on each SM (4864 cells): 5.4-5.6 us per stage, against 6.9 us in fixed
-        // point; with two blocks on an SM 8.8 against 7.3 us.
-        L.func = split_flat_func(with_base);
-        L.block = dim3(kSplitFlatThreads, 1, 1);
-        L.grid = dim3((unsigned)((4 * (size_t)a.nx + kSplitFlatThreads - 1) / kSplitFlatThreads), 1, 1);
-        return L;
-    }
     if (prec == CDBM_FP64) {
         const unsigned rows = a.ny < 65535 ? a.ny : 65535;
         // While the grid leaves most of the SMs' threads idle, the time is the chain of
-        // one thread, and the cell is split over four or two.  us per stage with four
-        // threads per cell, two and one: 9.4 / 12.6 / 24.5 at 64^2, 13.6 / 14.9 / 25.0 at
-        // 112^2, 15.6 / 14.6 / 24.4 at 128^2, 27.5 / 21.2 / 28.1 at 192^2, 40.6 / 34.8 /
-        // 37.5 at 256^2, 44.3 / 42.3 / 39.8 at 270^2.
+        // one thread, and the cell is split over 16 or two.  us per stage with 16 threads
+        // per cell, two and one: 5.6 / 12.7 / 24.5 at 64^2, 12.8 / 14.9 / 24.4 at 128^2,
+        // 22.9 / 21.3 / 28.1 at 192^2, 29.8 / 33.3 / 35.7 at 220^2, 37.6 / 35.0 / 37.5 at
+        // 256^2, 42.3 (two) / 39.8 at 270^2; tubes of 2000 cells 4.5 / 9.9 / 20, of 20000
+        // 11.3 / 13.0 / 20, of 30000 15.0 / 13.3 / 20.
         if (allow_split && cells <= (size_t)sm_count * 440) {
-            const bool four = cells <= (size_t)sm_count * 88;
-            const unsigned per = four ? 32 : 64;
-            L.func = four ? fx_split_func<4>(with_base, flat) : fx_split_func<2>(with_base, flat);
-            L.block = dim3(128, 1, 1);
+            const bool many = cells <= (size_t)sm_count * (flat ? 170 : 318);
+            const unsigned per = many ? 32 : 64;
+            L.func = many ? fx_cell16_func(with_base, flat) : fx_split_func(with_base, flat);
+            L.block = dim3(many ? 512 : 128, 1, 1);
             L.grid = dim3((unsigned)(((size_t)a.nx + per - 1) / per), rows, 1);
             return L;
         }

@@ -16,6 +16,7 @@
 #include <cooperative_groups.h>
 
 #include "cdbm_stage.cuh"
+#include "cdbm_stage_fx.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -125,8 +126,7 @@ __global__ void __launch_bounds__(256) small1d_kernel(float *f, int nsteps, cons
     }
 }
 
-// The arithmetic of one cell's group g in the four-thread split (the FP64 cluster
-// kernel and the flat split stage kernel): from the group's four values q, its base
+// The arithmetic of one cell's group g in the four-thread split: from the group's four values q, its base
 // values bs and x stencil values, the four updated values o.  The four threads of a
 // cell are lanes 4c .. 4c + 3 of one warp.
 __device__ __forceinline__ void split_cell(const StageArgs &a, int g, const double q[4], const double bs[4],
@@ -190,61 +190,6 @@ __device__ __forceinline__ void split_cell(const StageArgs &a, int g, const doub
     }
 }
 
-// FP64 variant with the work of a cell split over four threads, one per velocity
-// group: thread 4c + g of the CTA handles group g of cell c.  A stage of one cell
-// is a chain of dependent FP64 instructions whose latency, not throughput, bounds a
-// small grid (one warp per SM); splitting the cell shortens the chain about fourfold.
-// The four threads exchange their group components (s0, sx, sy) by warp shuffles and
-// each forms the moments, primitive variables and the shared part of the
-// equilibrium with the operations of conserved(), primitives() and equilibrium() in
-// the same order; each then builds and updates its own group's four velocities.
-// The compiler may fuse a multiply and an add differently than in the
-// one-thread-per-cell kernels, so the two agree to rounding, not bit for bit.
-__device__ __forceinline__ void split_stage(const cg::cluster_group &cl, const double *src, const double *base,
-                                            double *dst, const StageArgs &a, bool with_base, int chunk, int rank,
-                                            int x0, int len, unsigned *flag)
-{
-    const int t = threadIdx.x;
-    const int g = t & 3;                              // velocity group of this thread
-    const int lx0 = t >> 2;
-    const bool live = lx0 < len;
-    const int lx = live ? lx0 : len - 1;              // idle threads mirror the last cell
-    const int gx = x0 + lx;
-    const int nx = a.nx;
-    double q[4], bs[4], up2[4], up1[4], dn1[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        q[j] = src[(4 * g + j) * chunk + lx];
-        bs[j] = with_base ? base[(4 * g + j) * chunk + lx] : 0.0;
-    }
-    const bool inner = lx >= 2 && lx + 2 < len;
-    const int xm2 = neighbour_near(gx - 2, nx, a.bc_x), xm1 = neighbour_near(gx - 1, nx, a.bc_x);
-    const int xp1 = neighbour_near(gx + 1, nx, a.bc_x), xp2 = neighbour_near(gx + 2, nx, a.bc_x);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int i = 4 * g + j;
-        const int sx = dirx(i);
-        if (sx == 0) {
-            up2[j] = up1[j] = dn1[j] = 0.0;
-        } else if (inner) {
-            const double *p = src + i * chunk + lx;
-            up2[j] = p[sx > 0 ? -2 : 2];
-            up1[j] = p[sx > 0 ? -1 : 1];
-            dn1[j] = p[sx > 0 ? 1 : -1];
-        } else {
-            up2[j] = cluster_value(cl, src, chunk, rank, i, sx > 0 ? xm2 : xp2);
-            up1[j] = cluster_value(cl, src, chunk, rank, i, sx > 0 ? xm1 : xp1);
-            dn1[j] = cluster_value(cl, src, chunk, rank, i, sx > 0 ? xp1 : xm1);
-        }
-    }
-    double o[4];
-    split_cell(a, g, q, bs, up2, up1, dn1, with_base, live, flag, o);
-    if (live) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) dst[(4 * g + j) * chunk + lx] = o[j];
-    }
-}
-
 // One FP64 stage of a 1-D grid as an ordinary launch with each cell split over four
 // threads (split_cell), for tubes too long for the cluster kernel.  With one thread
 // per cell a tube of a few thousand cells leaves about a warp per SM, and the chain
@@ -288,12 +233,68 @@ __global__ void __launch_bounds__(kSplitFlatThreads) stage_split_flat_kernel(con
     }
 }
 
-__global__ void __launch_bounds__(256) small1d_split_kernel(double *f, int nsteps, const StageArgs a0,
-                                                            const StageArgs a1, unsigned *flag, int chunk)
+// Access to one cell of the cluster's state for fx_double_group().
+struct ClusterCell {
+    const double *src, *b;
+    double *dst;
+    int chunk, rank, nx, bc, x;
+    __device__ double at(int i, int gx) const
+    {
+        return cluster_value(cg::this_cluster(), src, chunk, rank, i, gx);
+    }
+    template <bool kFlatY>
+    __device__ FxStencil stencil(int i, int dx, int, double base) const
+    {
+        return {at(i, x), at(i, neighbour_near(x - 2 * dx, nx, bc)), at(i, neighbour_near(x - dx, nx, bc)),
+                at(i, neighbour_near(x + dx, nx, bc)), 0, 0, 0, base};
+    }
+    __device__ double base(int i) const { return b[i * chunk + (x - rank * chunk)]; }
+    __device__ void put(int i, double v) const { dst[i * chunk + (x - rank * chunk)] = v; }
+};
+
+// FP64 stage in the cluster, a cell on 16 threads (fx_cell16): warp w of the CTA has
+// the velocity cell16_velocity(w mod 16) of the cells 32 (w / 16) .. + 31 of the CTA's chunk.
+template <bool kBase>
+__device__ __forceinline__ void cluster_stage16(const cg::cluster_group &cl, const double *src, const double *base,
+                                                double *dst, const StageArgs &a, FxCells16 *s, int chunk, int rank, int x0,
+                                                int len, unsigned *flag)
+{
+    const int w = threadIdx.x >> 5, i = cell16_velocity(w & 15), set = w >> 4, nx = a.nx;
+    const int l0 = 32 * set + (int)(threadIdx.x & 31);
+    const bool live = l0 < len;
+    const int lx = live ? l0 : len - 1;               // idle lanes mirror the last cell
+    const int gx = x0 + lx;
+    const double c = src[i * chunk + lx];
+    FxStencil v = {c, c, c, c, 0, 0, 0, kBase ? base[i * chunk + lx] : 0.0};
+    const int d = dirx(i);
+    if (d != 0) {
+        if (lx >= 2 && lx + 2 < len) {
+            const double *p = src + i * chunk + lx;
+            v.x2 = p[-2 * d];
+            v.x1 = p[-d];
+            v.xd = p[d];
+        } else {
+            v.x2 = cluster_value(cl, src, chunk, rank, i, neighbour_near(gx - 2 * d, nx, a.bc_x));
+            v.x1 = cluster_value(cl, src, chunk, rank, i, neighbour_near(gx - d, nx, a.bc_x));
+            v.xd = cluster_value(cl, src, chunk, rank, i, neighbour_near(gx + d, nx, a.bc_x));
+        }
+    }
+    double o;
+    const bool ok = fx_cell16<true, kBase>(a, s[set], w & 15, set, i, v, flag, o);
+    if (!live) return;
+    if (ok) dst[i * chunk + lx] = o;
+    else
+        fx_double_group<ClusterCell, kBase, true>({src, base, dst, chunk, rank, nx, a.bc_x, gx}, a.eq, a.m,
+                                                  {a.a_self, a.a_base, a.lx, a.ly}, i >> 2, 1u << (i & 3), flag);
+}
+
+__global__ void __launch_bounds__(1024) small1d_fx_kernel(double *f, int nsteps, const __grid_constant__ StageArgs a0,
+                                                          const __grid_constant__ StageArgs a1, unsigned *flag, int chunk)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *s0 = reinterpret_cast<double *>(smem_raw);
     double *s1 = s0 + kNV * chunk;
+    FxCells16 *cells = reinterpret_cast<FxCells16 *>(s1 + kNV * chunk);
     const cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const int nx = a0.nx;
@@ -305,9 +306,9 @@ __global__ void __launch_bounds__(256) small1d_split_kernel(double *f, int nstep
     }
     cl.sync();
     for (int s = 0; s < nsteps; ++s) {
-        split_stage(cl, s0, nullptr, s1, a0, false, chunk, rank, x0, len, flag);
+        cluster_stage16<false>(cl, s0, nullptr, s1, a0, cells, chunk, rank, x0, len, flag);
         cl.sync();
-        split_stage(cl, s1, s0, s0, a1, true, chunk, rank, x0, len, flag);
+        cluster_stage16<true>(cl, s1, s0, s0, a1, cells, chunk, rank, x0, len, flag);
         cl.sync();
     }
     for (int k = threadIdx.x; k < kNV * len; k += blockDim.x) {
@@ -430,7 +431,7 @@ void *small1d_func_of(int prec, int chunk)
         return chunk <= kSplitDfMaxChunk ? (void *)small1d_split_df_kernel : small1d_func<kEqDF>();
     if (prec == CDBM_FP32_DEV) return small1d_func<kEqF32>();
     if (prec == CDBM_FP32_BULK) return small1d_func<kEqDouble>();
-    return (void *)small1d_split_kernel;
+    return (void *)small1d_fx_kernel;
 }
 
 }  // namespace
@@ -447,24 +448,30 @@ Small1D small1d_config(const StageArgs &a, int prec)
     // Used while each CTA holds at most two warps' worth of cells (FP64) or eight
     // (single precision).  Measured per stage on 64-4096-cell tubes: single
     // precision with the df64 equilibrium 2.7-3.2 us against 4.3-5.8 us for one
-    // launch per stage; FP64 9.3 us against 10.0 us, because there one warp's chain
-    // of dependent FP64 instructions, not the launch, sets the time of a stage.  With
-    // 128 FP64 cells per CTA (512 threads) a 2000-cell tube took 15.6 us per stage in
-    // the cluster against 10.0 us with one launch per stage on all SMs.
+    // launch per stage; FP64 4.0-5.2 us on 500-1000 cells, against 4.6 us per launch on
+    // all SMs: 1024 threads hold 64 cells.
     const int per_cta_max = prec == CDBM_FP64 ? 64 : 256;
     const int C = (a.nx + per_cta_max - 1) / per_cta_max > kMaxCluster ? 0 : kMaxCluster;
     if (C == 0) return L;
     int cluster = a.nx < C ? a.nx : C;
     const int chunk = (a.nx + cluster - 1) / cluster;
     cluster = (a.nx + chunk - 1) / chunk;            // no empty CTAs
-    const size_t smem = 2 * kNV * (size_t)chunk * storage_bytes(prec);
-    // FP64: four threads per cell (split_stage), df64: two (split_stage_df, up to
-    // kSplitDfMaxChunk cells), all cells of the CTA in one pass
-    const int per_cell = prec == CDBM_FP64 ? 4 : (prec == CDBM_FP32_DF64 && chunk <= kSplitDfMaxChunk ? 2 : 1);
+    const int sets = (chunk + 31) / 32;               // FP64: 32 cells on 16 warps each
+    const size_t smem = 2 * kNV * (size_t)chunk * storage_bytes(prec) +
+                        (prec == CDBM_FP64 ? sets * sizeof(FxCells16) : 0);
+    // df64: two threads per cell (split_stage_df, up to kSplitDfMaxChunk cells), all cells
+    // of the CTA in one pass
+    const int per_cell = prec == CDBM_FP32_DF64 && chunk <= kSplitDfMaxChunk ? 2 : 1;
     int threads = ((per_cell * chunk + 31) / 32) * 32;
     if (threads > 256) threads = 256;
+    if (prec == CDBM_FP64) threads = 512 * sets;
     void *func = small1d_func_of(prec, chunk);
     if (cluster > 8 && cudaFuncSetAttribute(func, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return L;
+    }
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return L;
     }

@@ -12,9 +12,8 @@
 //   - each velocity is updated in one of two ways that evaluate the same sum of
 //     products: where its stencil, base value and result share one sign and exponent
 //     (fx_update; the usual case in smooth flow), differences are differences of the
-//     doubles' bits, and the increment is added to them; elsewhere (fx_update_any) the
-//     operands are brought to the largest exponent of the cell, its upwind neighbours,
-//     its base value and its group's equilibrium.
+//     doubles' bits, and the increment is added to them; elsewhere (fx_transport_any,
+//     fx_relax_any) the operands are brought to the largest exponent among them.
 //     Relaxation and transport are rounded one after the other: differences too small
 //     to move a value by half a unit leave it unchanged, as in double arithmetic.  (With
 //     one rounding of the whole sum, differences of one unit ahead of the Ma = 15 shock
@@ -199,34 +198,48 @@ __device__ __forceinline__ int64_t fx_shift(int64_t h, int n)
     return (h >> n) + (int64_t)((((uint32_t)h << 1) >> fx_imin(n, 31)) & 1u);
 }
 
-// Any operands.  ok: in range.  The two outer stencil values enter the result only
-// through minmod, which a value three binades above the top exponent cannot win, so
-// those are clamped.  Where the velocity has no component along an axis the neighbours
-// are the cell itself.  One body for both axes keeps the code small: unrolled over axes
-// and members it takes longer to fetch than to run (2.9 against 1.8 ms per step of
-// piecewise-constant 1500 x 1300 fields).
-template <bool kFlatY, bool kBase>
-__device__ __forceinline__ double fx_update_any(const FxCoef &k, FxC lx, FxC ly, const FxStencil &v, int64_t h, int G,
-                                                bool &ok)
+// Any operands: the transport -sum l D in fixed point at the top exponent E of the cell
+// and its upwind neighbours.  The two outer stencil values enter it only through minmod,
+// which a value three binades above that exponent cannot win, so those are clamped.
+// Where the velocity has no component along an axis the neighbours are the cell itself.
+// One body for both axes keeps the code small: unrolled over axes and members it takes
+// longer to fetch than to run (2.9 against 1.8 ms per step of piecewise-constant
+// 1500 x 1300 fields).
+struct FxTransport {
+    int64_t t;
+    int E;
+};
+template <bool kFlatY>
+__device__ __forceinline__ FxTransport fx_transport_any(FxC lx, FxC ly, const FxStencil &v)
 {
     uint32_t key = fx_max(fx_key(v.c), fx_key(v.x1));
     if (!kFlatY) key = fx_max(key, fx_key(v.y1));
-    if (kBase) key = fx_max(key, fx_key(v.base));
-    const int E = fx_imax((int)(key >> 21), G);
-    ok = !fx_out_of_range(E);
+    const int E = (int)(key >> 21);
     const int64_t c = fx_from(v.c, E);
-    FxAcc a = {0, 0}, l = {0, 0};
-    fx_mac(a, c, k.self);
-    if (kBase) fx_mac(a, fx_from(v.base, E), k.base);
+    FxAcc l = {0, 0};
 #pragma unroll 1
     for (int axis = 0; axis < (kFlatY ? 1 : 2); ++axis) {
         const double u2 = axis ? v.y2 : v.x2, u1 = axis ? v.y1 : v.x1, d1 = axis ? v.yd : v.xd;
         fx_mac(l, fx_nnd2(fx_clamped(u2, E), fx_from(u1, E), c, fx_clamped(d1, E)), axis ? ly : lx);
     }
+    return {fx_sum<61>(l), E};
+}
+// ... and the update with it: relaxation and base at the top exponent of their terms,
+// rounded to double, then the transport.  ok: in range.
+template <bool kBase>
+__device__ __forceinline__ double fx_relax_any(const FxCoef &k, const FxStencil &v, int64_t h, int G,
+                                               const FxTransport &t, bool &ok)
+{
+    uint32_t key = fx_key(v.c);
+    if (kBase) key = fx_max(key, fx_key(v.base));
+    const int E = fx_imax((int)(key >> 21), G);
+    FxAcc a = {0, 0};
+    fx_mac(a, fx_from(v.c, E), k.self);
+    if (kBase) fx_mac(a, fx_from(v.base, E), k.base);
     const double o = fx_to(fx_sum<61>(a) + fx_shift(h, E - G + (kGroupLead - kLead)), E);
-    // o may lie some binades above E
-    const int F = fx_imax(E, (int)(fx_key(o) >> 21));
-    return fx_to(fx_from(o, F) + fx_shift(fx_sum<61>(l), F - E), F);
+    const int F = fx_imax(t.E, (int)(fx_key(o) >> 21));
+    ok = !fx_out_of_range(E) && !fx_out_of_range(F);
+    return fx_to(fx_from(o, F) + fx_shift(t.t, F - t.E), F);
 }
 
 // Operands of one sign and exponent: no conversion; the sum is in 64ths of c's unit in
@@ -299,11 +312,126 @@ __device__ __noinline__ void fx_rest_of_group(const Cell cell, const EqBlocks &B
         const int i = 4 * g + j;
         const FxStencil v = cell.template stencil<kFlatY>(i, dirx(i), diry(i), kBase ? cell.base(i) : 0.0);
         bool ok;
-        const double o = fx_update_any<kFlatY, kBase>(k, l.lx[g], l.ly[g], v, h.member(j), h.G, ok);
+        const double o = fx_relax_any<kBase>(k, v, h.member(j), h.G, fx_transport_any<kFlatY>(l.lx[g], l.ly[g], v), ok);
         if (ok) cell.put(i, o);
         else slow |= 1u << j;
     }
     if (slow) fx_double_group<Cell, kBase, kFlatY>(cell, B, m, d, g, slow, flag);
+}
+
+// ---- a cell on 16 threads ----
+
+// Shared memory of 32 cells whose velocities are on 16 warps.
+struct FxCells16 {
+    uint32_t key[kNV][32];
+    int64_t q[kNV][32];
+    double moment[4][32];
+    EqFactors factors[32];
+    int64_t h[kNV][32];
+    int G[4][32];
+};
+
+// The velocity of warp w of 16: first the four that a 1-D grid does not move, whose warps
+// (one on each SM sub-partition) also form the cell's equilibrium.
+__device__ __forceinline__ int cell16_velocity(int w)
+{
+    return w < 4 ? (w < 2 ? 1 + 2 * w : 5 + 2 * w) : (w < 8 ? (w < 6 ? 2 * (w - 4) : 2 * w - 4) : (w < 12 ? w - 4 : w));
+}
+
+// One stage of the lane's cell for the velocity i of warp w: on a grid of a few hundred or
+// thousand cells the time of a stage is the chain of one thread (about 4 cycles per
+// integer instruction and 64 per FP64 one, the rate of each SM sub-partition), which is
+// shortest with one velocity per thread.  Four warps form one moment each, one of them
+// the factors while the others take the transport (of a 1-D grid; on 2-D grids the warp of
+// the factors takes its own later), and four one group each; five block
+// barriers, which every thread of the block reaches, separate the exchanges through
+// shared memory.  (Repeating the moments and factors on the four group warps saves two
+// barriers but lengthens the chain: 4.6 against 4.2 us on 500 cells.)  The values are
+// those of the one-thread form.  v: the cell's value, its neighbours (the cell itself
+// along an axis without component) and base.  `lead`: the warp that forms the
+// factors, below 4.  Returns whether `out` is the result; otherwise the cell is outside
+// the integer path (fx_double_group).
+template <bool kFlatY, bool kBase>
+__device__ __forceinline__ bool fx_cell16(const StageArgs &a, FxCells16 &s, int w, int lead, int i, const FxStencil &v,
+                                          unsigned *flag, double &out)
+{
+    const int lane = threadIdx.x & 31, g = i >> 2;
+    s.key[i][lane] = fx_key(v.c);
+    __syncthreads();
+    uint32_t key = 0;
+#pragma unroll
+    for (int k = 0; k < kNV; ++k) key = fx_max(key, s.key[k][lane]);
+    const int top = (int)(key >> 21);
+    const bool cell_ok = !fx_out_of_range(top);
+    s.q[i][lane] = fx_from(v.c, top);
+    __syncthreads();
+    if (w < 4) {                          // moment w: rho, j_x, j_y, E
+        FxSum m = kFxHalfUnit;
+        int64_t r = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            int64_t q[4], s0, sx, sy;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) q[j] = s.q[4 * k + j][lane];
+            fx_group_sums(k, q, s0, sx, sy);
+            r += s0;
+            fx_mul(m, w == 1 ? sx : (w == 2 ? sy : s0), w == 3 ? a.fx.m.w[k] : a.fx.m.c[k]);
+        }
+        s.moment[w][lane] = w == 0 ? fx_to(r, top) : fx_to(fx_sum59(m), top + (w == 3 ? a.fx.m.wexp : a.fx.m.cexp));
+    }
+    __syncthreads();
+    const uint32_t hc = f64_hi(v.c);
+    uint32_t diff = (f64_hi(v.x2) ^ hc) | (f64_hi(v.x1) ^ hc) | (f64_hi(v.xd) ^ hc);
+    if (!kFlatY) diff |= (f64_hi(v.y2) ^ hc) | (f64_hi(v.y1) ^ hc) | (f64_hi(v.yd) ^ hc);
+    if (kBase) diff |= f64_hi(v.base) ^ hc;
+    const bool same = (diff & 0xfff00000u) == 0;
+    FxTransport t = {0, 0};
+    auto transport = [&]() {
+        if (same) {
+            FxSum l = {0, 0, 0};
+            fx_mul(l, fx_nnd2(fx_raw(v.x2), fx_raw(v.x1), fx_raw(v.c), fx_raw(v.xd)), a.fx.l.klx[g]);
+            if (!kFlatY) fx_mul(l, fx_nnd2(fx_raw(v.y2), fx_raw(v.y1), fx_raw(v.c), fx_raw(v.yd)), a.fx.l.kly[g]);
+            t.t = fx_sum_units(l);
+        } else {
+            t = fx_transport_any<kFlatY>(a.fx.l.lx[g], a.fx.l.ly[g], v);
+        }
+    };
+    if (w == lead)
+        s.factors[lane] = eq_factors(a.m, s.moment[0][lane], s.moment[1][lane], s.moment[2][lane], s.moment[3][lane],
+                                     flag);
+    else if (!kFlatY || w >= 4)           // the first four of a 1-D grid have none
+        transport();
+    __syncthreads();
+    if (w < 4) {                          // group w
+        const FxGroup e = fx_group(a.eq, s.factors[lane], w);
+        s.h[4 * w][lane] = e.h0;
+        s.h[4 * w + 1][lane] = e.h1;
+        s.h[4 * w + 2][lane] = e.h2;
+        s.h[4 * w + 3][lane] = e.h3;
+        s.G[w][lane] = e.G;
+    }
+    if (!kFlatY && w == lead) transport();
+    __syncthreads();
+    const int64_t h = s.h[i][lane];
+    const int G = s.G[g][lane];
+    bool ok = same;
+    if (same) {                           // fx_update() with the transport at hand
+        const int E = (int)((hc << 1) >> 21), n = E - G;
+        const int64_t C = fx_raw(v.c), sg = (int64_t)((int32_t)hc >> 31);
+        const int64_t M = (C & 0xfffffffffffffll) | 0x10000000000000ll;
+        FxSum r = kFxHalf;
+        fx_mul(r, M, a.fx.k.krelax);
+        if (kBase) fx_mul(r, fx_raw(v.base) - C, a.fx.k.kbase);
+        const int64_t m = (h ^ sg) - sg;
+        const int64_t O = C + fx_round64ths(fx_sum64ths(r) + fx_shift(m, n + (kGroupLead - kLead)), C) + t.t;
+        out = fx_bits((uint32_t)(O >> 32), (uint32_t)O);
+        ok = (((uint32_t)(O >> 32) ^ hc) & 0xfff00000u) == 0 && n >= -2 && !fx_out_of_range(E);
+    }
+    if (!ok) {
+        if (same || (kFlatY && w < 4)) t = fx_transport_any<kFlatY>(a.fx.l.lx[g], a.fx.l.ly[g], v);
+        out = fx_relax_any<kBase>(a.fx.k, v, h, G, t, ok);
+    }
+    return ok && cell_ok;
 }
 
 }  // namespace cdbm
