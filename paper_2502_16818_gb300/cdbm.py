@@ -411,7 +411,8 @@ class Solver:
             a = np.ascontiguousarray(np.broadcast_to(np.asarray(a, dtype=np.float64),
                                                      (self.ny, self.nx)))
             return a, a.ctypes.data
-        a = a.to(torch.float64).contiguous()
+        if a.dtype is not torch.float64 or not a.is_contiguous():
+            a = a.to(torch.float64).contiguous()
         return a, a.data_ptr()
 
     def init(self, rho, ux, uy, T):
@@ -523,7 +524,9 @@ class BatchSolver:
 
     def macros(self):
         """(rho, ux, uy, T) as concatenated float64 numpy arrays."""
-        out = [np.zeros(self.total) for _ in range(4)]
+        # written once by the host: into pages that nothing has touched yet, the device's
+        # copy takes 60 instead of 5 ms for 2.2 M cells
+        out = [np.full(self.total, 0.0) for _ in range(4)]
         cdbm_batch_macros(self.b, *(a.ctypes.data for a in out))
         return tuple(out)
 

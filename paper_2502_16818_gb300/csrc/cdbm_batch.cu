@@ -801,32 +801,46 @@ cdbm_status cdbm_batch_init(cdbm_batch *b, const double *rho, const double *ux, 
     if (!rho || !ux || !uy || !T) return bset_err(b, CDBM_EINVAL, "cdbm_batch_init: NULL field");
     const size_t n = (size_t)b->P;
     const double *src[4] = {rho, ux, uy, T};
-    std::vector<double> host[4];
+    const bool single = single_storage(b->precision);
+    std::vector<double> copy[4];
+    const double *host[4] = {nullptr, nullptr, nullptr, nullptr};    // readable by the host where needed
     const double *dev[4];
     // the second buffer (16 planes of the storage type) stages host fields: 4 double planes fit
     double *stage = (double *)b->f1;
     for (int k = 0; k < 4; ++k) {
-        host[k].resize(n);
-        if (bcuda(b, cudaMemcpy(host[k].data(), src[k], sizeof(double) * n, cudaMemcpyDefault), "batch fields read"))
-            return b->err;
         if (is_device_ptr(src[k])) {
             dev[k] = src[k];
+            if (k == 2 || (single && (k == 0 || k == 3))) {
+                copy[k].resize(n);
+                if (bcuda(b, cudaMemcpy(copy[k].data(), src[k], sizeof(double) * n, cudaMemcpyDefault), "batch fields read"))
+                    return b->err;
+                host[k] = copy[k].data();
+            }
         } else {
             if (bcuda(b, cudaMemcpyAsync(stage + k * n, src[k], sizeof(double) * n, cudaMemcpyHostToDevice,
                                          b->stream), "batch fields upload"))
                 return b->err;
             dev[k] = stage + k * n;
+            host[k] = src[k];
         }
     }
     // u_y = 0 everywhere: every tube's state is y-symmetric and stays so
     bool sym = true;
-    for (size_t c = 0; c < n && sym; ++c) sym = host[2][c] == 0.0;
+    for (size_t c = 0; c < n && sym; c += 4096) {
+        uint64_t any = 0;                  // the bits but the sign: +0 and -0 only
+        for (size_t j = c, e = std::min(n, c + 4096); j < e; ++j) {
+            uint64_t bits;
+            memcpy(&bits, host[2] + j, sizeof bits);
+            any |= bits << 1;
+        }
+        sym = any == 0;
+    }
     if (sym != b->sym) {
         b->sym = sym;
         drop_batch_graph(b);
     }
-    // per-tube reference state (FP32-bulk): means of rho and T over the tube
-    for (int t = 0; t < b->ntubes; ++t) {
+    // per-tube reference state of a single-precision state: means of rho and T over the tube
+    for (int t = 0; t < b->ntubes && single; ++t) {
         TubeInfo &ti = b->info[t];
         const ClassConsts &C = b->args.cls[ti.cls];
         double sr = 0.0, sT = 0.0;
@@ -838,9 +852,7 @@ cdbm_status cdbm_batch_init(cdbm_batch *b, const double *rho, const double *ux, 
         ti.rhoF = ti.EF = 0.0;
         for (int g = 0; g < 4; ++g) {
             const double *S = C.unit.S + 4 * g;
-            ti.Fg[g] = single_storage(b->precision)
-                           ? S[0] * r0 + S[1] * K * P0 + S[3] * 2.0 * (K + 2.0) * P0 * T0
-                           : 0.0;
+            ti.Fg[g] = S[0] * r0 + S[1] * K * P0 + S[3] * 2.0 * (K + 2.0) * P0 * T0;
             ti.rhoF += 4.0 * ti.Fg[g];
             ti.EF += 4.0 * ti.Fg[g] * C.m.w[g];
         }
