@@ -184,7 +184,7 @@ __device__ __forceinline__ void tube_group_fx(const TubeCell<kSym> &cell, const 
                                               int grp, const FxGroup h, bool cell_ok, unsigned *flag)
 {
     constexpr bool kBase = kStage == 1;
-    const FxK lx = C.l[kStage].klx[grp];
+    const FxC lx = C.l[kStage].klx[grp];
     unsigned rest = 0;
     auto pass = [&](int j, auto transport) {
         constexpr bool kX = decltype(transport)::value;

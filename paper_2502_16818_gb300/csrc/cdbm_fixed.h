@@ -159,14 +159,13 @@ CDBM_FX_HD int64_t fx_nnd2(int64_t u2, int64_t u1, int64_t c, int64_t d1)
 // these are the differences of the magnitudes in units in the last place.
 CDBM_FX_HD int64_t fx_raw(double v) { return (int64_t)((uint64_t)f64_hi(v) << 32 | f64_lo(v)); }
 
-// A constant of the run as b1 2^30 + b0 in units of 2^-60; b0x4 = 4 b0.
+// A constant of the run as b1 2^30 + b0 in units of 2^-59; b0x4 = 4 b0.
 struct FxK {
     int32_t b1, b0, b0x4;
 };
 
-// Sum of products x b, all four partial products kept.  No partial sum overflows for up
-// to four products of |x| < 2^56 and |b| <= 2 in units of 2^-60 (the stage coefficients)
-// nor for the moments: the four |x| add up to less than 2^63, |b| <= 1 in 2^-59.
+// Sum of products x b, all four partial products kept.  No partial sum overflows for the
+// moments: the four |x| add up to less than 2^63, |b| <= 1 in 2^-59.
 struct FxSum {
     int64_t r, mid, low;
 };
@@ -179,13 +178,26 @@ CDBM_FX_HD void fx_mul(FxSum &a, int64_t x, FxK b)
     a.mid += (int64_t)x0 * b.b1;
     a.low += (int64_t)x0 * b.b0;
 }
-// The sum in 1/64 of the units of x, rounded to nearest, of an FxSum that starts from
-// kFxHalf.
-constexpr FxSum kFxHalf = {0, 1 << 23, 0};
-CDBM_FX_HD int64_t fx_sum64ths(const FxSum &a)
+// The same with a constant as hi 2^32 + lo: the sum is r 2^64 + mid 2^32 + low, so that the
+// shift by 64 that the scale of the operands is chosen for below costs nothing (in units of
+// 2^-60 it took about ten instructions more per velocity: 0.99 against 0.96 ms per step of
+// 1500 x 1300 cells).  Two products
+// at most, lo of one of the constants above -2^31.
+CDBM_FX_HD void fx_mul(FxSum &a, int64_t x, FxC b)
 {
-    return (int64_t)((uint64_t)a.r << 8) + ((a.mid + (a.low >> 30)) >> 24);
+    const int32_t x0 = (int32_t)x;
+    const int32_t x1 = (int32_t)(x >> 32) + (int32_t)((uint32_t)x0 >> 31);
+    a.r += (int64_t)x1 * b.hi;
+    a.mid += (int64_t)x1 * b.lo;
+    a.mid += (int64_t)x0 * b.hi;
+    a.low += (int64_t)x0 * b.lo;
 }
+// The sum in 1/64 of the units of y, rounded to nearest, of an FxSum that starts from
+// kFxHalf and takes x = y 2^9 with constants in units of 2^-61 (|y| < 2^53; relaxation
+// |b| <= 2, base |b| <= 1/2).
+constexpr int kFxUp = 9;
+constexpr FxSum kFxHalf = {0, (int64_t)1 << 31, 0};
+CDBM_FX_HD int64_t fx_sum64ths(const FxSum &a) { return a.r + ((a.mid + (a.low >> 32)) >> 32); }
 // The sum in the units of x, rounded to nearest, for constants in units of 2^-59, of an
 // FxSum that starts from kFxHalfUnit.
 constexpr FxSum kFxHalfUnit = {0, 1 << 28, 0};
@@ -195,28 +207,30 @@ CDBM_FX_HD int64_t fx_sum59(const FxSum &a)
 }
 // 64ths rounded to the nearest unit so that C plus the result is even on a tie.
 CDBM_FX_HD int64_t fx_round64ths(int64_t t, int64_t C) { return (t + 31 + (((t >> 6) ^ C) & 1)) >> 6; }
-// The sum rounded to the nearest unit of x, a tie toward zero.
+// The sum rounded to the nearest unit of x, a tie toward zero, for constants in units of
+// 2^-64 (-1/2 <= b <= 0; two that add up to less than -1/2 by rounding only).
 CDBM_FX_HD int64_t fx_sum_units(const FxSum &a)
 {
-    const int64_t m = a.mid + (a.low >> 30);                  // the sum is r 2^62 + m 2^30, in 2^-60
-    const int64_t v = (int64_t)((uint64_t)a.r << 2) + (m >> 30);
-    const uint32_t tie = 0x1fffffffu + (uint32_t)((uint64_t)v >> 63);
-    return v + (int64_t)((((uint32_t)m & 0x3fffffffu) + tie) >> 30);
+    const int64_t m = a.mid + (a.low >> 32);
+    const int64_t v = a.r + (m >> 32);
+    const uint32_t tie = 0x7fffffffu + (uint32_t)((uint64_t)v >> 63);
+    return v + (int64_t)(((uint64_t)(uint32_t)m + tie) >> 32);
 }
 
-// v 2^bits (|v| <= 2) as a constant of fx_mac.
-inline FxC fx_const(double v, int bits)
+inline FxC fx_split(int64_t b)
 {
-    const int64_t b = std::llrint(std::ldexp(v, bits));
     FxC c;
     c.lo = (int32_t)(uint32_t)b;
-    c.hi = (int32_t)((b - c.lo) >> 32);
+    c.hi = (int32_t)((b >> 32) + (c.lo < 0));
     return c;
 }
+inline int64_t fx_int(FxC c) { return ((int64_t)c.hi << 32) + c.lo; }
+// v 2^bits (|v| <= 2) as a constant of fx_mac.
+inline FxC fx_const(double v, int bits) { return fx_split(std::llrint(std::ldexp(v, bits))); }
 
 inline FxK fx_k(FxC a)
 {
-    const int64_t b = (((int64_t)a.hi << 32) + a.lo) / 2;      // in twice the unit of a
+    const int64_t b = fx_int(a) / 2;                           // in twice the unit of a
     FxK k;
     k.b1 = (int32_t)((b + (1 << 29)) >> 30);
     k.b0 = (int32_t)(b - ((int64_t)k.b1 << 30));
@@ -239,16 +253,16 @@ struct FxModel {
     FxK c[4], w[4];
     int cexp, wexp;
 };
-// Stage coefficients, out = base base + self g + heq - sum l D: times 2^61 for any
-// operands, and base and self + base - 1 = -gamma h for operands of one exponent.
+// Stage coefficients, out = base base + self g + heq - sum l D, times 2^61; for operands of
+// one exponent self + base - 1 = -gamma h.
 struct FxCoef {
-    FxC self, base;
-    FxK kbase, krelax;
+    FxC self, base, relax;
 };
-// Transport coefficients as -l / 2 (fx_nnd2 gives 2 D), in both forms.
+// Transport coefficients -l / 2 (fx_nnd2 gives 2 D) times 2^61, and times 2^64 for operands
+// of one exponent.
 struct FxFlux {
     FxC lx[4], ly[4];
-    FxK klx[4], kly[4];
+    FxC klx[4], kly[4];
 };
 
 inline FxModel fx_model(const double c[4], const double w[4])
@@ -268,13 +282,11 @@ inline FxCoef fx_coef(double self, double base)
     k.self = fx_const(self, 61);
     k.base = fx_const(base, 61);
     // the same real numbers in both forms: self + base - 1 from the rounded constants
-    const int64_t one = (int64_t)1 << 61;
-    const int64_t r = ((int64_t)k.self.hi << 32) + k.self.lo + ((int64_t)k.base.hi << 32) + k.base.lo - one;
-    FxC relax;
-    relax.lo = (int32_t)(uint32_t)r;
-    relax.hi = (int32_t)((r - relax.lo) >> 32);
-    k.kbase = fx_k(k.base);
-    k.krelax = fx_k(relax);
+    k.relax = fx_split(fx_int(k.self) + fx_int(k.base) - ((int64_t)1 << 61));
+    if (k.relax.lo == INT32_MIN) {       // see fx_mul
+        k.self = fx_split(fx_int(k.self) + 1);
+        k.relax.lo += 1;
+    }
     return k;
 }
 // lx, ly: gamma dt c_g / dr; along an axis of one cell every difference is zero and l
@@ -282,11 +294,16 @@ inline FxCoef fx_coef(double self, double base)
 inline FxFlux fx_flux(const double lx[4], const double ly[4], bool along_x, bool along_y)
 {
     FxFlux f;
+    auto set = [](double l, FxC &c, FxC &k) {
+        int64_t b = std::llrint(std::ldexp(-0.5 * l, 61));
+        if (b < -((int64_t)1 << 60)) b = -((int64_t)1 << 60);    // l = 1 but for rounding
+        if ((uint32_t)((uint64_t)b << 3) == 0x80000000u) ++b;    // see fx_mul
+        c = fx_split(b);
+        k = fx_split((int64_t)((uint64_t)b << 3));
+    };
     for (int g = 0; g < 4; ++g) {
-        f.lx[g] = fx_const(along_x ? -0.5 * lx[g] : 0.0, 61);
-        f.ly[g] = fx_const(along_y ? -0.5 * ly[g] : 0.0, 61);
-        f.klx[g] = fx_k(f.lx[g]);
-        f.kly[g] = fx_k(f.ly[g]);
+        set(along_x ? lx[g] : 0.0, f.lx[g], f.klx[g]);
+        set(along_y ? ly[g] : 0.0, f.ly[g], f.kly[g]);
     }
     return f;
 }

@@ -204,7 +204,7 @@ __device__ __forceinline__ void fx_grid_group(const double *g, const double *bas
             v.x1 = St::get(gp + (up ? (neg ? st.rp1 : st.rm1) : st.row), up ? st.c : (neg ? st.p1 : st.m1));
             v.xd = St::get(gp + (up ? (neg ? st.rm1 : st.rp1) : st.row), up ? st.c : (neg ? st.m1 : st.p1));
         }
-        const FxK kx = !kDiag && !kFlatY && (j & 1) ? a.fx.l.kly[grp] : a.fx.l.klx[grp];
+        const FxC kx = !kDiag && !kFlatY && (j & 1) ? a.fx.l.kly[grp] : a.fx.l.klx[grp];
         double o;
         const bool ok = fx_update<kX, kY, kBase>(a.fx.k, kx, a.fx.l.kly[grp], v, h.member(j), h.G, o);
         if (live && ok && cell_ok) *(double *)((char *)(out + plane + st.row) + st.c) = o;
@@ -224,10 +224,12 @@ __device__ __forceinline__ void fx_grid_group(const double *g, const double *bas
                                                   a.fx.l, {a.a_self, a.a_base, a.lx, a.ly}, grp, rest, cell_ok, h, flag);
 }
 
-// Stage in double precision, one cell per thread (cdbm_stage_fx.cuh).  Bound by the
-// issue of about 4100 integer instructions per cell and stage (against 246 / 262 FP64
-// instructions of 64 cycles each); 64 registers for 32 warps per SM, which hide the
-// latency of its dependent chains (7.1 ms per 4096^2 step; 7.6 at 24 warps, 8.2 at 16).
+// Stage in double precision, one cell per thread (cdbm_stage_fx.cuh).  Bound by the ALU
+// pipe, which takes about 3200 of some 6000 instructions per cell and stage (ncu: 66-73 %
+// busy, the FP64 pipe 48-53 %, issue 60-64 %; against 246 / 262 FP64 instructions of 64
+// cycles each before); 64 registers for 32 warps per SM, which hide the latency of its
+// dependent chains (24 warps 7 % slower, 16 warps 15 %).  6.9 ms per 4096^2 step (15.8 all
+// in FP64), 0.96 ms per 1500 x 1300.
 constexpr int kFxMinBlocks = 8;
 template <bool kBase, bool kFlatY, bool kWide>
 __global__ void __launch_bounds__(kStageThreads, kFxMinBlocks)

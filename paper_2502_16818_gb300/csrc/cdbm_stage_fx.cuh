@@ -162,7 +162,10 @@ struct FxGroup {
     __device__ __forceinline__ int64_t member(int j) const { return (j & 2) ? ((j & 1) ? h3 : h2) : ((j & 1) ? h1 : h0); }
 };
 
-// Group g.  kSym: of a y-symmetric state, whose y-odd components and diagonal quadrupole
+// Group g.  The products with the blocks stay in FP64: as integer dot products at one
+// exponent per cell they leave 30 of the 68 FP64 instructions, but the stage is not bound
+// by that pipe any more (1.28 against 1.02 ms per step of 1500 x 1300 cells).
+// kSym: of a y-symmetric state, whose y-odd components and diagonal quadrupole
 // are zero.
 template <bool kSym = false>
 __device__ __forceinline__ FxGroup fx_group(const EqBlocks &B, const EqFactors &q, int g)
@@ -246,7 +249,7 @@ __device__ __forceinline__ double fx_relax_any(const FxCoef &k, const FxStencil 
 // the last place and is added to c's bits.  false: not that case, or the result leaves
 // the binade.
 template <bool kX, bool kY, bool kBase>
-__device__ __forceinline__ bool fx_update(const FxCoef &k, FxK lx, FxK ly, const FxStencil &v, int64_t h, int G,
+__device__ __forceinline__ bool fx_update(const FxCoef &k, FxC lx, FxC ly, const FxStencil &v, int64_t h, int G,
                                           double &out)
 {
     const uint32_t hc = f64_hi(v.c);
@@ -258,8 +261,8 @@ __device__ __forceinline__ bool fx_update(const FxCoef &k, FxK lx, FxK ly, const
     const int64_t C = fx_raw(v.c), s = (int64_t)((int32_t)hc >> 31);
     const int64_t M = (C & 0xfffffffffffffll) | 0x10000000000000ll;
     FxSum a = kFxHalf, l = {0, 0, 0};
-    fx_mul(a, M, k.krelax);
-    if (kBase) fx_mul(a, fx_raw(v.base) - C, k.kbase);
+    fx_mul(a, M << kFxUp, k.relax);
+    if (kBase) fx_mul(a, (int64_t)((uint64_t)(fx_raw(v.base) - C) << kFxUp), k.base);
     if (kX) fx_mul(l, fx_nnd2(fx_raw(v.x2), fx_raw(v.x1), C, fx_raw(v.xd)), lx);
     if (kY) fx_mul(l, fx_nnd2(fx_raw(v.y2), fx_raw(v.y1), C, fx_raw(v.yd)), ly);
     const int64_t m = (h ^ s) - s;                   // the sums are those of the magnitudes
@@ -420,8 +423,8 @@ __device__ __forceinline__ bool fx_cell16(const StageArgs &a, FxCells16 &s, int 
         const int64_t C = fx_raw(v.c), sg = (int64_t)((int32_t)hc >> 31);
         const int64_t M = (C & 0xfffffffffffffll) | 0x10000000000000ll;
         FxSum r = kFxHalf;
-        fx_mul(r, M, a.fx.k.krelax);
-        if (kBase) fx_mul(r, fx_raw(v.base) - C, a.fx.k.kbase);
+        fx_mul(r, M << kFxUp, a.fx.k.relax);
+        if (kBase) fx_mul(r, (int64_t)((uint64_t)(fx_raw(v.base) - C) << kFxUp), a.fx.k.base);
         const int64_t m = (h ^ sg) - sg;
         const int64_t O = C + fx_round64ths(fx_sum64ths(r) + fx_shift(m, n + (kGroupLead - kLead)), C) + t.t;
         out = fx_bits((uint32_t)(O >> 32), (uint32_t)O);

@@ -79,8 +79,8 @@ int main()
         ++used;
         const int64_t C = fx_raw(s[0]), M = (C & 0xfffffffffffffll) | 0x10000000000000ll;
         FxSum r = kFxHalf, t = {0, 0, 0};
-        fx_mul(r, M, c.krelax);
-        fx_mul(r, fx_raw(s[7]) - C, c.kbase);
+        fx_mul(r, M << kFxUp, c.relax);
+        fx_mul(r, (fx_raw(s[7]) - C) * (1 << kFxUp), c.base);
         fx_mul(t, fx_nnd2(fx_raw(s[1]), fx_raw(s[2]), C, fx_raw(s[3])), f.klx[0]);
         fx_mul(t, fx_nnd2(fx_raw(s[4]), fx_raw(s[5]), C, fx_raw(s[6])), f.kly[0]);
         // the increment alone, in units in the last place of the cell's value
@@ -92,10 +92,11 @@ int main()
     std::printf("any %.3f\nfast %.3f\nused %ld\n", any, fast, used > 50000 ? 0l : used);
     // ties of the transport sum go toward zero
     bad = 0;
+    const double half[4] = {1, 1, 1, 1};
     for (int64_t v = -9; v <= 9; ++v) {
         FxSum s = {0, 0, 0};
-        fx_mul(s, v, fx_k(fx_const(0.5, 61)));
-        if (fx_sum_units(s) != v / 2) ++bad;
+        fx_mul(s, v, fx_flux(half, half, true, true).klx[0]);   // -v / 2 of fx_nnd2's 2 D
+        if (fx_sum_units(s) != -v / 2) ++bad;
     }
     std::printf("ties %ld\n", bad);
 }
