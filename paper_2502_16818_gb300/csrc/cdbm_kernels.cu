@@ -1252,6 +1252,12 @@ StageLaunch stage_launch_config(const StageArgs &a, bool with_base, int sm_count
             R = r;
         }
     }
+    // FP32_BULK waits on the FP64 pipe, which the differences carried from row to row do not
+    // relieve, while longer runs leave the last wave of blocks nearly empty: one row per block
+    // takes 9.7 against 11.2 ms per 40 steps of 700 x 650 cells, 19.4 against 21.0 per 20 of
+    // 1500 x 1300, 36.3 against 36.9 per 4 of 4096^2 (4 rows 11.2, 20.4, 37.4; the one-cell
+    // kernel 9.9, 20.6, 37.6).
+    if (!pair) R = 1;
     if (march) {
         L.func = pair ? stage_march2_func(with_base, (a.nx & 1) == 0, prec == CDBM_FP32_DEV)
                       : stage_func<kEqDouble>(true, with_base, false);
