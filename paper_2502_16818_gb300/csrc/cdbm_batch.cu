@@ -331,6 +331,10 @@ __global__ void __launch_bounds__(kThreads, batch_min_blocks(!kSingle<TS>, kThre
                                                          const __grid_constant__ BatchArgs a, unsigned *flag)
 {
     __shared__ TubeConsts tc;          // FP64 only
+    // in registers: read from the parameters in each step they cost a tube of the deviation
+    // state a tenth of its time (16 tubes, 30 steps with init and read-out: 1.16 against 1.02
+    // ms; 1024 tubes, 200 steps: 60.2 against 58.2)
+    const float as0 = a.a_self_f[0], ab0 = a.a_base_f[0], as1 = a.a_self_f[1], ab1 = a.a_base_f[1];
     for (int w = work_off[blockIdx.x]; w < work_off[blockIdx.x + 1]; ++w) {
         const TubeInfo &t = tubes[work[w]];
         const ClassConsts &C = a.cls[t.cls];
@@ -357,9 +361,9 @@ __global__ void __launch_bounds__(kThreads, batch_min_blocks(!kSingle<TS>, kThre
                 __syncthreads();
                 tube_stage2<1, kSym>(f1t, ft, ft, a.P, t, C, a.a_self_f2[1], a.a_base_f2[1], flag);
             } else {
-                tube_stage<0, kEq, kSym>(ft, nullptr, f1t, a.P, t, C, a.a_self_f[0], a.a_base_f[0], flag);
+                tube_stage<0, kEq, kSym>(ft, nullptr, f1t, a.P, t, C, as0, ab0, flag);
                 __syncthreads();
-                tube_stage<1, kEq, kSym>(f1t, ft, ft, a.P, t, C, a.a_self_f[1], a.a_base_f[1], flag);
+                tube_stage<1, kEq, kSym>(f1t, ft, ft, a.P, t, C, as1, ab1, flag);
             }
             __syncthreads();
         }
