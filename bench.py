@@ -34,15 +34,14 @@ sys.path.insert(0, ROOT)
 METRIC = "cell-updates/s and HBM GB/s vs FP64 plain on same GB300 at stated L2 error"
 UNIT = "cell-updates/s"
 
-# FP64-pipe work of the stage kernels per cell; the rest of a stage (sums, transport,
-# update) runs on the integer pipes.  Instructions per stage: ncu
-# sm__inst_executed_pipe_fp64 per warp of 32 cells where no cell leaves the integer path:
-# 68.  Flops, counted from the kernel source with an FMA as two flops: 30 for the factors
-# and 20 per velocity group.  Bytes
-# per cell-step: stage 1 reads f^n and writes f1 (128 + 128 B); stage 2 reads f1 and
+# FP64-pipe work of the stage kernels per cell; the group sums and the transport
+# differences run on the integer pipes.  Instructions: ncu sm__inst_executed_pipe_fp64 per
+# warp of 32 cells (stage 1: 141, stage 2: 157).  Flops, counted from the kernel source
+# with an FMA as two flops: 24 for the moments, 30 for the factors of the equilibrium, 118
+# for the four groups, 80 (stage 2: 112) for the update.  Bytes per cell-step: stage 1 reads f^n and writes f1 (128 + 128 B); stage 2 reads f1 and
 # f^n and writes f^n+1 (384 B).
-FP64_INSTR_PER_CELL_STEP = 136
-FP64_FLOPS_PER_CELL_STEP = 220
+FP64_INSTR_PER_CELL_STEP = 298
+FP64_FLOPS_PER_CELL_STEP = 536
 BYTES_PER_CELL_STEP = 640
 FP64_LANES_PER_CLK_PER_SM = 2       # 1.25 TFLOP/s nominal FP64 / (2 flops x 152 SMs x 2.07 GHz)
 BYTES_PER_CELL_STEP_FP32 = 320      # the same buffers in single precision
@@ -56,11 +55,11 @@ BYTES_PER_CELL_STEP_ADJ_BWD = 640 + 384 + 512
 # the stage kernels; valid only while the code of the kernel sources (comments
 # stripped) hashes to TRAFFIC_SHA.
 # Captured at 1024^2 (134 MB per plane set, above L2) and scaled by 16 cells-fold.
-TRAFFIC_SHA = "df6f489c4de42fde"
-TRAFFIC_BYTES_PER_LAUNCH = 5.609e9
+TRAFFIC_SHA = "4ec522ff2ff730c8"
+TRAFFIC_BYTES_PER_LAUNCH = 4.948e9
 
 
-STAGE_SOURCES = ("cdbm_device.cuh", "cdbm_fixed.h", "cdbm_stage_fx.cuh", "cdbm_kernels.cu", "cdbm_internal.h")
+STAGE_SOURCES = ("cdbm_device.cuh", "cdbm_exact.h", "cdbm_stage_exact.cuh", "cdbm_stage_double.cu", "cdbm_internal.h")
 
 
 def _code_only(text):
@@ -355,7 +354,7 @@ def run_cdbm(a, rank, world, local_rank):
     probe = fp64_peak(torch, cdbm, stream, local_rank)
     roofline = {"bound": "alu", "achieved": achieved_tflops, "peak": peak_tflops, "unit": "TFLOP/s",
                 "frac": achieved_tflops / peak_tflops, "traffic": traffic,
-                "kernel": "stage_fx_kernel (RK stages 1 and 2, mean per launch; the FP64 part of its work)",
+                "kernel": "stage_double_kernel (RK stages 1 and 2, mean per launch; the FP64 part of its work)",
                 "peak_source": "FP64 pipe: 2 lanes/clk/SM x 152 SMs x 2070 MHz x 2 flops (recipe nominal 1.25 TFLOP/s)",
                 "peak_measured": probe["tflops"], "frac_of_measured_peak": achieved_tflops / probe["tflops"],
                 "peak_measured_source": "%s, %d x %d threads x 8 chains x %d FMAs, best of %d, this run"
@@ -659,9 +658,8 @@ def aux_kernels(s, w, stream, torch, cdbm, state_bytes, with_init, reps=10):
     32 B), Delta* (reads the planes, writes 12 doubles: 96 B; it rebuilds the
     central moments of every cell from its raw moments) and the conserved sums
     (reads the planes; a synchronous call that returns 4
-    doubles).  On the FP64 state they take 88 (Delta*), 10 (macros) and 22 (sums) FP64
-    instructions per cell; macros runs near the memory's rate, the other two near the
-    FP64 pipe's.  state_bytes:
+    doubles).  On the FP64 state Delta* takes some 135 FP64 instructions per cell for the
+    vortex' velocity set, macros 27 and the sums 22, near the FP64 pipe's rate.  state_bytes:
     bytes per stored value (8 for FP64, 4 for the single-precision states)."""
     cells = w.nx * w.ny
     planes = 16 * state_bytes

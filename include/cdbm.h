@@ -159,7 +159,7 @@ cdbm_status cdbm_step(cdbm_ctx *ctx, int nsteps);
 
 /* Enables (default) or disables the small-grid paths of cdbm_step: on 1-D grids the
  * persistent cluster kernel, and for CDBM_FP64 the stage kernels that split each cell
- * over 16 or two threads (grids of up to about 67000 cells).  Disabled, those grids step
+ * over 16 or two threads (grids of up to about 39000 cells).  Disabled, those grids step
  * with the one-cell-per-thread stage kernel like any other, with the same results bit
  * for bit. */
 cdbm_status cdbm_set_small_grid_path(cdbm_ctx *ctx, int enable);

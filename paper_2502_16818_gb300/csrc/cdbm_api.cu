@@ -68,7 +68,6 @@ struct cdbm_ctx {
     double Fg[4];                 // FP32-bulk reference equilibrium per group (0 for FP64)
     StageArgs stage[2];
     StageLaunch launch[2];
-    StageLaunch adj_launch[2];    // the same stages in FP64 throughout, for the adjoint's run
     RkStage rks[2];
     FieldArgs fields;
 
@@ -496,7 +495,6 @@ cdbm_status cdbm_create(const cdbm_grid *grid, const cdbm_vset *vset, double I, 
     build_stages(c);
     c->fields.eq = c->eq_unit;
     c->fields.m = c->mc;
-    c->fields.fx = fx_model(c->mc.c, c->mc.w);
     for (int i = 0; i < kNV; ++i) {
         const double s = vset->v[i >> 2];
         c->fields.vx[i] = dirx(i) * s;
@@ -665,9 +663,7 @@ cdbm_status cdbm_macros(cdbm_ctx *c, double *rho, double *ux, double *uy, double
         any_host |= host[k];
         dev[k] = host[k] ? (double *)c->f1 + k * c->plane : dst[k];
     }
-    // the fields of a recorded run are the start of its adjoint: in FP64, as the run
-    const bool recorded = c->adj_steps > 0 && c->step_count == c->adj_end;
-    if (cuda_check(c, launch_macros(c->fields, c->f, c->precision, recorded, dev[0], dev[1], dev[2], dev[3], c->stream),
+    if (cuda_check(c, launch_macros(c->fields, c->f, c->precision, dev[0], dev[1], dev[2], dev[3], c->stream),
                    "macros launch"))
         return c->err;
     for (int k = 0; k < 4; ++k)
@@ -820,8 +816,6 @@ cdbm_status cdbm_adjoint_forward(cdbm_ctx *c, int nsteps, int every)
     if (c->err) return c->err;
     if (adjoint_supported(c, "cdbm_adjoint_forward")) return c->err;
     if (nsteps < 1 || every < 1) return set_err(c, CDBM_EINVAL, "cdbm_adjoint_forward: nsteps, every >= 1");
-    for (int s = 0; s < 2; ++s)
-        c->adj_launch[s] = double_stage_launch_config(c->stage[s], s == 1, c->sm_count, c->march_enabled, c->small_enabled);
     if (!c->state_set) return set_err(c, CDBM_EINVAL, "cdbm_adjoint_forward: state not initialised");
     free_ckpt(c);
     const size_t fb = sizeof(double) * kNV * c->plane;
@@ -838,14 +832,7 @@ cdbm_status cdbm_adjoint_forward(cdbm_ctx *c, int nsteps, int every)
         if (cuda_check(c, cudaMemcpyAsync(c->ckpt[k], c->f, fb, cudaMemcpyDeviceToDevice, c->stream), "checkpoint"))
             return c->err;
         const int n = (k + 1) * every <= nsteps ? every : nsteps - k * every;
-        for (int s = 0; s < n; ++s) {
-            cudaError_t e = launch_stage(c->adj_launch[0], c->f, nullptr, c->f1, c->stage[0], c->flag, c->stream);
-            if (e == cudaSuccess)
-                e = launch_stage(c->adj_launch[1], c->f1, c->f, c->f, c->stage[1], c->flag, c->stream);
-            if (cuda_check(c, e, "adjoint forward")) return c->err;
-        }
-        c->t += n * c->dt;
-        c->step_count += n;
+        if (cdbm_step(c, n)) return c->err;
     }
     c->adj_steps = nsteps;
     c->adj_every = every;
@@ -909,15 +896,15 @@ cdbm_status cdbm_adjoint_backward(cdbm_ctx *c, const double *fbar, double *grad_
         for (int j = 0; j < len && !st; ++j) {
             if (!keep1 && j + 1 == len) break;
             double *g1 = keep1 ? seg1[j] : G1;
-            cudaError_t e = launch_stage(c->adj_launch[0], seg[j], nullptr, g1, c->stage[0], c->flag, c->stream);
+            cudaError_t e = launch_stage(c->launch[0], seg[j], nullptr, g1, c->stage[0], c->flag, c->stream);
             if (e == cudaSuccess && j + 1 < len)
-                e = launch_stage(c->adj_launch[1], g1, seg[j], seg[j + 1], c->stage[1], c->flag, c->stream);
+                e = launch_stage(c->launch[1], g1, seg[j], seg[j + 1], c->stage[1], c->flag, c->stream);
             st = cuda_check(c, e, "adjoint recompute");
         }
         for (int j = len - 1; j >= 0 && !st; --j) {
             const double *g1 = keep1 ? seg1[j] : G1;
             cudaError_t e = keep1 ? cudaSuccess
-                                  : launch_stage(c->adj_launch[0], seg[j], nullptr, G1, c->stage[0], c->flag, c->stream);
+                                  : launch_stage(c->launch[0], seg[j], nullptr, G1, c->stage[0], c->flag, c->stream);
             if (e == cudaSuccess)   // stage 2: f^{n+1} = f^n/2 + f1/2 + dt/2 L(f1)
                 e = launch_adjoint_stage(g1, B, nullptr, 0.0, B1, c->stage[1], 0.5 * h, inv_tau, c->adj_limiter, acc,
                                          c->stream);

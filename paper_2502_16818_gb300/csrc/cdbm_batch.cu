@@ -21,7 +21,7 @@
 #include <vector>
 
 #include "cdbm_stage.cuh"
-#include "cdbm_stage_fx.cuh"
+#include "cdbm_stage_exact.cuh"
 #include "cdbm_internal.h"
 
 using namespace cdbm;
@@ -37,7 +37,6 @@ struct TubeInfo {
     double lx[2][4];                  // per stage: gamma dt c_g / dx_t
     float lx_f[2][4];
     float2 lx_f2[2][4];               // lx_f twice (two-column df64 stage)
-    FxFlux fx[2];                     // per stage: lx in fixed point (CDBM_FP64)
     double sF[2][4];                  // per stage: gamma h F_g (FP32-bulk reference)
     double Fg[4];                     // reference equilibrium per group
     double rhoF, EF;                  // its conserved moments
@@ -53,7 +52,6 @@ struct ClassConsts {
     DFModel dfm;
     DFBlocksT<float2> dfeq2[2];       // the same with each value twice
     DFModelT<float2> dfm2;
-    FxModel fx;                       // fixed-point model constants (CDBM_FP64)
     DevProj dp[2];                    // per stage: conservation projection (CDBM_FP32_DEV)
 };
 
@@ -62,7 +60,6 @@ struct BatchArgs {
     double a_self[2], a_base[2];
     float a_self_f[2], a_base_f[2];
     float2 a_self_f2[2], a_base_f2[2];
-    FxCoef fx[2];                     // fixed-point stage coefficients (CDBM_FP64)
     long long P;                      // total cells: stride between velocity planes
 };
 
@@ -146,67 +143,35 @@ __device__ __forceinline__ void tube_stage(const float *g, const float *base, fl
     }
 }
 
-// Access to one cell of a tube for fx_rest_of_group(): zero-gradient ends; with kSym a
-// result goes to its plane and to that of its mirror image.
-template <bool kSym>
-struct TubeCell {
-    const double *g, *b;
-    double *out;
-    long long P;
-    int nx, x;
-    template <bool kFlatY>
-    __device__ __forceinline__ FxStencil stencil(int i, int dx, int, double base) const
-    {
-        auto at = [&](int j) { return g[i * P + (j < 0 ? 0 : (j >= nx ? nx - 1 : j))]; };
-        return {at(x), at(x - 2 * dx), at(x - dx), at(x + dx), 0, 0, 0, base};
-    }
-    __device__ __forceinline__ double base(int i) const { return b[i * P + x]; }
-    __device__ __forceinline__ void put(int i, double v) const
-    {
-        out[i * P + x] = v;
-        if (kSym && sym_partner(i) >= 0) out[sym_partner(i) * P + x] = v;
-    }
-};
-
 // The constants of the tube a block works on, in shared memory: indexed per tube in the
 // kernel's parameters they cost several times as much to read.
 struct TubeConsts {
     EqBlocks eq[2];
     ModelConsts m;
-    FxModel fx;
-    FxFlux l[2];
     double lx[2][4];
 };
 
 // The members of group grp of one cell of a tube (kSym: the distinct ones), one per pass.
+// xs: the columns two and one to the left, one and two to the right.
 template <bool kDiag, int kStage, bool kSym>
-__device__ __forceinline__ void tube_group_fx(const TubeCell<kSym> &cell, const int xs[4], const TubeConsts &C, const FxCoef &k, double a_self, double a_base,
-                                              int grp, const FxGroup h, bool cell_ok, unsigned *flag)
+__device__ __forceinline__ void tube_group(const double *g, const double *base, double *out, long long P, int x,
+                                           const int xs[4], double lx, double a_self, double a_base, int grp,
+                                           const EqGroup h)
 {
     constexpr bool kBase = kStage == 1;
-    const FxC lx = C.l[kStage].klx[grp];
-    unsigned rest = 0;
     auto pass = [&](int j, auto transport) {
-        constexpr bool kX = decltype(transport)::value;
-        const double *gp = cell.g + (4 * grp + j) * cell.P;
-        FxStencil v = {};
-        if (kBase) v.base = cell.b[(4 * grp + j) * cell.P + cell.x];
-        v.c = gp[cell.x];
-        if constexpr (kX) {
+        const long long plane = (4 * grp + j) * P;
+        const double *gp = g + plane;
+        const double c = gp[x];
+        double o = fma(a_self, c, h.member(j));
+        if (kBase) o = fma(a_base, base[plane + x], o);
+        if constexpr (decltype(transport)::value) {
             const bool west = kDiag ? j == 1 || j == 2 : j == 2;
-            v.x2 = gp[west ? xs[3] : xs[0]];
-            v.x1 = gp[west ? xs[2] : xs[1]];
-            v.xd = gp[west ? xs[1] : xs[2]];
+            o = fma(-lx, nnd_exact(gp[west ? xs[3] : xs[0]], gp[west ? xs[2] : xs[1]], c, gp[west ? xs[1] : xs[2]]), o);
         }
-        double o;
-        const bool ok = fx_update<kX, false, kBase>(k, lx, lx, v, h.member(j), h.G, o);
-        if (ok && cell_ok) {
-            cell.out[(4 * grp + j) * cell.P + cell.x] = o;
-            // mirror images: S of N; SE of NE, SW of NW
-            if (kSym && (kDiag || j == 1)) cell.out[(4 * grp + (kDiag ? 3 - j : 3)) * cell.P + cell.x] = o;
-        } else {
-            rest |= 1u << j;
-        }
+        out[plane + x] = o;
+        // mirror images: S of N; SE of NE, SW of NW
+        if (kSym && (kDiag || j == 1)) out[(4 * grp + (kDiag ? 3 - j : 3)) * P + x] = o;
     };
     if constexpr (kDiag) {
 #pragma unroll 1
@@ -217,31 +182,38 @@ __device__ __forceinline__ void tube_group_fx(const TubeCell<kSym> &cell, const 
 #pragma unroll 1
         for (int j = 1; j < (kSym ? 2 : 4); j += 2) pass(j, std::false_type{});     // N, S: no transport
     }
-    if (rest)
-        fx_rest_of_group<TubeCell<kSym>, kBase, true>(cell, C.eq[kStage], C.m, k, C.l[kStage],
-                                                      {a_self, a_base, C.lx[kStage], C.lx[kStage]}, grp, rest, cell_ok,
-                                                      h, flag);
 }
 
-// The FP64 stage of one tube (cdbm_stage_fx.cuh), one cell per thread.
-template <int kStage, bool kSym>
-__device__ __forceinline__ void tube_stage_fx(const double *g, const double *base, double *out, long long P,
-                                              int nx, const TubeConsts &C, const FxCoef &k, double a_self,
-                                              double a_base, unsigned *flag)
+// The FP64 stage of one tube (cdbm_stage_exact.cuh), one cell per thread.
+template <int kStage, bool kSym, bool kRounded>
+__device__ __forceinline__ void tube_cells_double(const double *g, const double *base, double *out, long long P, int nx,
+                                                  const TubeConsts &C, double a_self, double a_base, unsigned *flag)
 {
     for (int x = threadIdx.x; x < nx; x += blockDim.x) {
         const int xs[4] = {x >= 2 ? x - 2 : 0, x >= 1 ? x - 1 : 0, x + 1 < nx ? x + 1 : nx - 1, x + 2 < nx ? x + 2 : nx - 1};
-        const TubeCell<kSym> cell = {g, base, out, P, nx, x};
-        const FxCons m = fx_conserved(C.fx, [=](int i) { return g[(kSym ? mirror_y(i) : i) * P + x]; });
+        double f[kNV];
+#pragma unroll
+        for (int i = 0; i < kNV; ++i) f[i] = g[(kSym ? mirror_y(i) : i) * P + x];
+        const Cons m = moments_exact(C.m, f);
         const EqFactors q = kSym ? eq_factors_sym(C.m, m.rho, m.jx, m.E, flag) : eq_factors(C.m, m.rho, m.jx, m.jy, m.E, flag);
+        const EqBlocks &B = C.eq[kStage];
+        const double *lx = C.lx[kStage];
 #pragma unroll 1
         for (int p = 0; p < 4; p += 2) {
-            tube_group_fx<false, kStage, kSym>(cell, xs, C, k, a_self, a_base, p, fx_group<kSym>(C.eq[kStage], q, p),
-                                               m.ok, flag);
-            tube_group_fx<true, kStage, kSym>(cell, xs, C, k, a_self, a_base, p + 1,
-                                              fx_group<kSym>(C.eq[kStage], q, p + 1), m.ok, flag);
+            tube_group<false, kStage, kSym>(g, base, out, P, x, xs, lx[p], a_self, a_base, p, eq_group<false, kSym>(B, q, p, kRounded));
+            tube_group<true, kStage, kSym>(g, base, out, P, x, xs, lx[p + 1], a_self, a_base, p + 1,
+                                           eq_group<true, kSym>(B, q, p + 1, kRounded));
         }
     }
+}
+
+// ... with the rounding of the same tube alone.
+template <int kStage, bool kSym>
+__device__ __forceinline__ void tube_stage_double(const double *g, const double *base, double *out, long long P, int nx,
+                                                  const TubeConsts &C, double a_self, double a_base, unsigned *flag)
+{
+    if (nx <= kRoundedTube) tube_cells_double<kStage, kSym, true>(g, base, out, P, nx, C, a_self, a_base, flag);
+    else tube_cells_double<kStage, kSym, false>(g, base, out, P, nx, C, a_self, a_base, flag);
 }
 
 // The df64 stage of one tube with two cells per thread: each thread takes the
@@ -305,10 +277,10 @@ __device__ __forceinline__ void tube_stage2(const float *g, const float *base, f
 }
 
 // Register budget (resident threads per SM the registers must allow).
-// FP64 (fixed-point form): 1024 for blocks of 256 threads (64 registers; 3.25e9
-// cell-updates/s on the 1024-tube ensemble at 4 blocks per SM, against 3.12e9 at a
-// budget of 512 or 640), 512 for narrower ones, whose tiles keep fewer warps (2.91e9 at
-// 128 x 4, against 2.69e9 at 1024).
+// FP64: 512 (90 registers in the symmetric form, no spills): 0.81 ms per step of the
+// 1024-tube ensemble at 128 x 4 threads per SM, 0.84 at 128 x 3 (1.12 and 1.14 with all
+// operations on the FP64 pipe).  Blocks of 256 threads 1024, for their tile of 4 blocks
+// (0.83 ms; 0.97-0.99 at a budget of 640 or 768, which 3 blocks do not notice: 0.80-0.82).
 // FP32_BULK: 384 (168 registers at 128 threads), 512 in the symmetric form, which keeps
 // less live state (116 registers, 3.05e9 against 2.90e9).  Two-column df64: 384, 640 in
 // the symmetric form (96 registers; 1.13e10 against 1.07e10; 768 spilled 380 bytes).  The
@@ -342,20 +314,18 @@ __global__ void __launch_bounds__(kThreads, batch_min_blocks(!kSingle<TS>, kThre
             // every thread of the block has passed the last barrier of the tube before
             for (int s = threadIdx.x; s < 2; s += blockDim.x) {
                 tc.eq[s] = C.eq[s];
-                tc.l[s] = t.fx[s];
                 for (int g = 0; g < 4; ++g) tc.lx[s][g] = t.lx[s][g];
             }
             if (threadIdx.x == 32) tc.m = C.m;
-            if (threadIdx.x == 33) tc.fx = C.fx;
             __syncthreads();
         }
         TS *ft = f + t.offset;
         TS *f1t = f1 + t.offset;
         for (int s = 0; s < nsteps; ++s) {
             if constexpr (!kSingle<TS>) {
-                tube_stage_fx<0, kSym>(ft, nullptr, f1t, a.P, t.nx, tc, a.fx[0], a.a_self[0], a.a_base[0], flag);
+                tube_stage_double<0, kSym>(ft, nullptr, f1t, a.P, t.nx, tc, a.a_self[0], a.a_base[0], flag);
                 __syncthreads();
-                tube_stage_fx<1, kSym>(f1t, ft, ft, a.P, t.nx, tc, a.fx[1], a.a_self[1], a.a_base[1], flag);
+                tube_stage_double<1, kSym>(f1t, ft, ft, a.P, t.nx, tc, a.a_self[1], a.a_base[1], flag);
             } else if constexpr (kEq == kEqDF) {
                 tube_stage2<0, kSym>(ft, nullptr, f1t, a.P, t, C, a.a_self_f2[0], a.a_base_f2[0], flag);
                 __syncthreads();
@@ -407,15 +377,6 @@ __global__ void __launch_bounds__(128) batch_init_kernel(const BatchArgs a, cons
     }
 }
 
-// Conserved moments in FP64, for cells outside the fixed-point path.
-template <typename TS>
-__device__ __noinline__ Cons batch_conserved_any(const ModelConsts &m, const TS *own, long long P)
-{
-    double fc[kNV];
-    for (int i = 0; i < kNV; ++i) fc[i] = widen(own[i * P]);
-    return conserved(fc, m);
-}
-
 template <typename TS>
 __global__ void __launch_bounds__(128) batch_macros_kernel(const ClassConsts *__restrict__ cls, long long P, const TubeInfo *tubes,
                                                             const long long *offs, int ntubes, const TS *f,
@@ -428,10 +389,10 @@ __global__ void __launch_bounds__(128) batch_macros_kernel(const ClassConsts *__
         // the operations of the single-grid macros kernel: moments of the stored
         // values (plus the reference equilibrium's for a single-precision state)
         // and one reciprocal of rho
-        const TS *own = f + c;
-        const FxCons fm = fx_conserved(cls[t.cls].fx, [=](int i) { return __ldg(own + i * P); });
-        Cons q = {fm.rho, fm.jx, fm.jy, fm.E};
-        if (!fm.ok) q = batch_conserved_any(m, own, P);
+        TS fc[kNV];
+#pragma unroll
+        for (int i = 0; i < kNV; ++i) fc[i] = f[i * P + c];
+        Cons q = moments_exact(m, fc);
         if constexpr (kSingle<TS>) {
             q.rho += t.rhoF;
             q.E += t.EF;
@@ -701,7 +662,6 @@ cdbm_status cdbm_batch_create(int ntubes, const int *nx, const double *dx, const
     for (int s = 0; s < 2; ++s) {
         b->args.a_self[s] = beta[s] - gamma[s] * h;
         b->args.a_base[s] = alpha[s];
-        b->args.fx[s] = fx_coef(b->args.a_self[s], b->args.a_base[s]);
         b->args.a_self_f[s] = (float)b->args.a_self[s];
         b->args.a_base_f[s] = (float)b->args.a_base[s];
         b->args.a_self_f2[s] = make_float2(b->args.a_self_f[s], b->args.a_self_f[s]);
@@ -740,7 +700,6 @@ cdbm_status cdbm_batch_create(int ntubes, const int *nx, const double *dx, const
             }
             C.dfm = df_model(C.m);
             C.dfm2 = df_model_twice(C.dfm);
-            C.fx = fx_model(C.m.c, C.m.w);
             for (int s = 0; s < 2; ++s) C.dp[s] = dev_proj(C.m, gamma[s] * h);
         }
         TubeInfo &ti = b->info[t];
@@ -754,7 +713,6 @@ cdbm_status cdbm_batch_create(int ntubes, const int *nx, const double *dx, const
                 ti.lx_f[s][g] = (float)ti.lx[s][g];
                 ti.lx_f2[s][g] = make_float2(ti.lx_f[s][g], ti.lx_f[s][g]);
             }
-        for (int s = 0; s < 2; ++s) ti.fx[s] = fx_flux(ti.lx[s], ti.lx[s], nx[t] > 1, false);
         b->offs[t + 1] = b->offs[t] + nx[t];
     }
     b->P = b->offs[ntubes];

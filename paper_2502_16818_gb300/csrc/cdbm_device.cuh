@@ -1,8 +1,8 @@
-// Device building blocks of the CDBM kernels: velocity-set geometry, the
-// conserved moments, the factored equilibrium, the minmod limiter and the NND
-// transport difference.  Everything here is double precision; integer work
-// (limiter decisions, validity tests, neighbour indices) is kept off the FP64
-// pipe, which is the scarce unit on GB300.
+// Device building blocks of the CDBM kernels: velocity-set geometry, the conserved
+// moments, the factored equilibrium, the minmod limiter and the NND transport
+// difference, in double precision (the single-precision limiter and difference beside
+// them).  Integer work (limiter decisions, validity tests, neighbour indices) is kept off
+// the FP64 pipe, which is the scarce unit on GB300.
 #pragma once
 
 #include <cstdint>
@@ -270,6 +270,64 @@ __device__ __forceinline__ Prim primitives(const double f[kNV], const ModelConst
     s.T = s.p * r;
     if (!(positive_finite(s.q.rho) && positive_finite(s.p))) atomicOr(flag, kFlagNonPhys);
     return s;
+}
+
+// The factors of the equilibrium of one cell.
+struct EqFactors {
+    double rho, E, jx, jy, T, ru2, m1416, W4, d57, m6, u2, dlt;
+};
+
+__device__ __forceinline__ EqFactors eq_factors(const ModelConsts &m, double rho, double jx, double jy, double E,
+                                                unsigned *flag)
+{
+    EqFactors q;
+    const double r = rcp64(rho);
+    const double ux = jx * r, uy = jy * r;
+    const double jyuy = __dmul_rn(jy, uy), uy2 = __dmul_rn(uy, uy);
+    q.ru2 = fma(jx, ux, jyuy);
+    const double P = (E - q.ru2) * m.invK;
+    q.T = P * r;
+    if (!(positive_finite(rho) && positive_finite(P))) atomicOr(flag, kFlagNonPhys);
+    q.rho = rho;
+    q.E = E;
+    q.jx = jx;
+    q.jy = jy;
+    q.u2 = fma(ux, ux, uy2);
+    q.dlt = fma(ux, ux, -uy2);
+    q.m1416 = fma(q.T, fma(m.Kp6, q.ru2, __dmul_rn(m.twoKp2, P)), __dmul_rn(q.ru2, q.u2));
+    q.W4 = fma(m.Kp4, q.T, q.u2);
+    q.d57 = fma(jx, ux, -jyuy);
+    q.m6 = jx * uy;
+    // kept in registers: the compiler otherwise repeats FP64 instructions in the loop
+    // over the groups to save some
+    asm volatile("" : "+d"(q.T), "+d"(q.ru2), "+d"(q.m1416), "+d"(q.W4), "+d"(q.d57), "+d"(q.m6), "+d"(q.u2), "+d"(q.dlt));
+    return q;
+}
+
+// eq_factors() of a y-symmetric state (j_y = u_y = 0).
+__device__ __forceinline__ EqFactors eq_factors_sym(const ModelConsts &m, double rho, double jx, double E, unsigned *flag)
+{
+    EqFactors q;
+    const double r = rcp64(rho);
+    const double ux = jx * r;
+    q.ru2 = __dmul_rn(jx, ux);
+    const double P = (E - q.ru2) * m.invK;
+    q.T = P * r;
+    if (!(positive_finite(rho) && positive_finite(P))) atomicOr(flag, kFlagNonPhys);
+    q.rho = rho;
+    q.E = E;
+    q.jx = jx;
+    q.jy = 0.0;
+    q.u2 = __dmul_rn(ux, ux);
+    q.dlt = q.u2;
+    q.m1416 = fma(q.T, fma(m.Kp6, q.ru2, __dmul_rn(m.twoKp2, P)), __dmul_rn(q.ru2, q.u2));
+    q.W4 = fma(m.Kp4, q.T, q.u2);
+    q.d57 = q.ru2;
+    q.m6 = 0.0;
+    asm volatile("" : "+d"(q.T), "+d"(q.ru2), "+d"(q.m1416), "+d"(q.W4), "+d"(q.u2));
+    q.dlt = q.u2;
+    q.d57 = q.ru2;
+    return q;
 }
 
 // ---- y-symmetric states of 1-D grids ----

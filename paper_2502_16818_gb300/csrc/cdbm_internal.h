@@ -6,7 +6,6 @@
 #include <cstddef>
 
 #include "../../include/cdbm.h"
-#include "cdbm_fixed.h"
 
 namespace cdbm {
 
@@ -128,7 +127,6 @@ struct StageArgs {
     DevProj dp;                   // conservation projection (CDBM_FP32_DEV)
     float2 a_base_f2, a_self_f2;  // a_base_f, a_self_f, lx_f, ly_f twice
     float2 lx_f2[4], ly_f2[4];
-    FxStage fx;                   // fixed-point constants of the FP64 stage
     int nx, ny;
     int bc_x, bc_y;
 };
@@ -138,7 +136,6 @@ struct FieldArgs {
     ModelConsts m;
     double vx[kNV], vy[kNV], eta[kNV];
     double Fg[4];    // reference equilibrium per group (FP32-bulk state only)
-    FxModel fx;      // fixed-point model constants
     int nx, ny;
 };
 
@@ -164,8 +161,7 @@ char *thread_error_buffer();
 cudaError_t launch_init(const FieldArgs &a, const double *rho, const double *ux,
                         const double *uy, const double *T, void *f, int prec, unsigned *flag,
                         cudaStream_t s);
-// in_double: the sums of a CDBM_FP64 state in FP64 (the read-out of a recorded run).
-cudaError_t launch_macros(const FieldArgs &a, const void *f, int prec, bool in_double, double *rho, double *ux,
+cudaError_t launch_macros(const FieldArgs &a, const void *f, int prec, double *rho, double *ux,
                           double *uy, double *T, cudaStream_t s);
 cudaError_t launch_tne(const FieldArgs &a, const void *f, int prec, double *out, cudaStream_t s);
 cudaError_t launch_sums(const FieldArgs &a, const void *f, int prec, double *partials, int nblocks,
@@ -190,15 +186,9 @@ struct StageLaunch {
 StageLaunch stage_launch_config(const StageArgs &a, bool with_base, int sm_count, int prec,
                                 bool allow_march = true, bool allow_split = true);
 
-// The all-FP64 stage kernels (cdbm_stage_double.cu) of the run that the adjoint
-// differentiates.
-StageLaunch double_stage_launch_config(const StageArgs &a, bool with_base, int sm_count, bool allow_march,
-                                       bool allow_split);
+// The same for a CDBM_FP64 state (cdbm_stage_double.cu).
+StageLaunch double_stage_launch_config(const StageArgs &a, bool with_base, int sm_count, bool allow_split);
 
-// FP64 stage kernel for 1-D grids with each cell split over four threads
-// (cdbm_small1d.cu): kSplitFlatThreads threads per block, 4 nx threads in all.
-constexpr int kSplitFlatThreads = 128;
-void *split_flat_func(bool with_base);
 cudaError_t launch_stage(const StageLaunch &L, const void *g, const void *base, void *out,
                          const StageArgs &a, unsigned *flag, cudaStream_t s);
 
@@ -240,8 +230,6 @@ void fill_df_consts(StageArgs &a);
 // The conservation projection of a stage whose blocks are scaled by gh = gamma h.
 DevProj dev_proj(const ModelConsts &m, double gh);
 void fill_dev_proj(StageArgs &a, double gh);
-// Fills a.fx from the double constants of a (CDBM_FP64).
-void fill_fx_consts(StageArgs &a);
 // The same constants with each value twice, for the two-column (packed FP32x2) kernels.
 DFBlocksT<float2> df_blocks_twice(const DFBlocks &d);
 DFModelT<float2> df_model_twice(const DFModel &d);

@@ -1,19 +1,19 @@
-// CDBM kernels: initial equilibrium, the fused Runge-Kutta stage, macroscopic
-// fields, nonequilibrium moments and conserved sums.  The distribution buffers
-// are stored in double (CDBM_FP64) or single (CDBM_FP32_BULK, CDBM_FP32_DF64,
-// CDBM_FP32_DEV) precision, selected by the template parameter TS; the conserved
-// sums and the equilibrium of a stage are computed in double, in double-float
-// arithmetic on the FP32 pipe for CDBM_FP32_DF64, or in single precision on the
-// moment deviations for CDBM_FP32_DEV (template parameter kEq).
+// CDBM kernels: initial equilibrium, the fused Runge-Kutta stage of the single-precision
+// states (CDBM_FP32_BULK, CDBM_FP32_DF64, CDBM_FP32_DEV; CDBM_FP64 in
+// cdbm_stage_double.cu), macroscopic fields, nonequilibrium moments and conserved sums.
+// TS is the type a state is stored in.  The conserved sums and the equilibrium of a stage
+// are computed in double, in double-float arithmetic on the FP32 pipe for CDBM_FP32_DF64,
+// or in single precision on the moment deviations for CDBM_FP32_DEV (template parameter
+// kEq).
 //
 // Layout: f[16][ny][nx] (velocity plane outermost, x fastest).  A block covers a
 // run of columns along x, so centre loads and stores of a warp are coalesced rows
 // and the stencil neighbours (x +- 1, 2 and the rows y +- 1, 2) are served from
-// L1/L2 or shared memory.  stage_kernel gives each thread one cell; the
-// row-marching kernels give each thread one column (two for the df64 and deviation states) over a
-// run of rows.
+// L1/L2 or shared memory.  stage_kernel gives each thread one cell; the row-marching
+// kernels give each thread one column (two for the df64 and deviation states) over a run
+// of rows.
 #include "cdbm_stage.cuh"
-#include "cdbm_stage_fx.cuh"
+#include "cdbm_stage_exact.cuh"
 
 namespace cdbm {
 
@@ -37,8 +37,7 @@ constexpr int stage_min_blocks(int eq) { return eq != kEqDouble ? CDBM_STAGE_MIN
 // f_eq of the fields.  Bound by the FP64 pipe: 86 instructions (2.60 ms for 4096^2 cells),
 // 102 for a single-precision state (118 before the narrowing left the pipe, 3.87 -> 3.26
 // ms with the means of rho and T).  Rebuilding the members in fixed point took 62 and
-// 1.99 ms, but the initial state is also the adjoint's, whose dL/dtau must not change
-// (cdbm_stage_double.cu).
+// 1.99 ms, but rounds differently, and the time step amplifies that (cdbm_exact.h).
 template <typename TS>
 __global__ void __launch_bounds__(128) init_kernel(const FieldArgs a, const double *__restrict__ rho,
                                                     const double *__restrict__ ux,
@@ -114,227 +113,6 @@ __global__ void __launch_bounds__(kStageThreads, stage_min_blocks(kEq))
             }
             out[i * P + c] = o;
         }
-    }
-}
-
-// Row pointers and offsets of a cell's stencil.  The row pointers are uniform over a
-// block, the offsets in a row 32 bits wide (kWide: 64 bits, for rows of 2^29 cells and
-// more), which saves the 64-bit address arithmetic of about 100 loads per cell.
-template <bool kWide>
-struct GridStencil {
-    using Off = std::conditional_t<kWide, size_t, unsigned>;
-    Off c, m2, m1, p1, p2;
-    size_t row, rm2, rm1, rp1, rp2;
-    __device__ __forceinline__ GridStencil(int x, int nx, int bc)
-        : c((Off)8 * x), m2((Off)8 * neighbour_near(x - 2, nx, bc)), m1((Off)8 * neighbour_near(x - 1, nx, bc)),
-          p1((Off)8 * neighbour_near(x + 1, nx, bc)), p2((Off)8 * neighbour_near(x + 2, nx, bc))
-    {
-    }
-    template <bool kFlatY>
-    __device__ __forceinline__ void at_row(int y, int nx, int ny, int bc)
-    {
-        row = (size_t)y * nx;
-        if (!kFlatY) {
-            rm2 = (size_t)neighbour_near(y - 2, ny, bc) * nx;
-            rm1 = (size_t)neighbour_near(y - 1, ny, bc) * nx;
-            rp1 = (size_t)neighbour_near(y + 1, ny, bc) * nx;
-            rp2 = (size_t)neighbour_near(y + 2, ny, bc) * nx;
-        }
-    }
-    static __device__ __forceinline__ double get(const double *p, Off o) { return __ldg((const double *)((const char *)p + o)); }
-};
-
-// Access to one cell of a grid for fx_rest_of_group().
-struct GridCell {
-    const double *g, *b;
-    double *out;
-    int nx, ny, bc_x, bc_y, x, y;
-    __device__ __forceinline__ size_t at(int i) const { return (size_t)i * nx * ny + (size_t)y * nx + x; }
-    // any direction signs, 0 included
-    template <bool kFlatY>
-    __device__ __forceinline__ FxStencil stencil(int i, int dx, int dy, double base) const
-    {
-        const double *gp = g + (size_t)i * nx * ny, *gr = gp + (size_t)y * nx;
-        FxStencil v = {gr[x], gr[neighbour_near(x - 2 * dx, nx, bc_x)], gr[neighbour_near(x - dx, nx, bc_x)],
-                       gr[neighbour_near(x + dx, nx, bc_x)], 0, 0, 0, base};
-        if (!kFlatY) {
-            v.y2 = gp[(size_t)neighbour_near(y - 2 * dy, ny, bc_y) * nx + x];
-            v.y1 = gp[(size_t)neighbour_near(y - dy, ny, bc_y) * nx + x];
-            v.yd = gp[(size_t)neighbour_near(y + dy, ny, bc_y) * nx + x];
-        }
-        return v;
-    }
-    __device__ __forceinline__ double base(int i) const { return b[at(i)]; }
-    __device__ __forceinline__ void put(int i, double v) const { out[at(i)] = v; }
-};
-
-// The four members of group grp of one cell: loads, update and stores, one member per
-// pass.  The passes differ in the offsets of the neighbours only and share their code:
-// unrolled, the members' independent chains overlap (6.9 ms per 4096^2 step at 12
-// warps per SM, 7.0 as here at 32), but the code outgrows the instruction cache as soon
-// as other paths run beside it (1500 x 1300 piecewise-constant fields: 1.9 against
-// 1.27 ms).
-template <int kUnroll, bool kDiag, bool kFlatY, bool kBase, bool kWide>
-__device__ __forceinline__ void fx_grid_group(const double *g, const double *base, double *out, const StageArgs &a,
-                                              const GridStencil<kWide> &st, size_t P, int x, int y, int grp,
-                                              const FxGroup h, bool cell_ok, bool live, unsigned *flag)
-{
-    using St = GridStencil<kWide>;
-    unsigned rest = 0;
-    auto pass = [&](int j, auto transport) {
-        constexpr bool kX = decltype(transport)::value, kY = kDiag && !kFlatY && kX;
-        const size_t plane = (4 * grp + j) * P;
-        const double *gp = g + plane, *gr = gp + st.row;
-        FxStencil v = {};
-        if (kBase) v.base = *(const double *)((const char *)(base + plane + st.row) + st.c);
-        v.c = St::get(gr, st.c);
-        if constexpr (kX && (kDiag || kFlatY)) {
-            const bool west = kDiag ? j == 1 || j == 2 : j == 2;
-            v.x2 = St::get(gr, west ? st.p2 : st.m2);
-            v.x1 = St::get(gr, west ? st.p1 : st.m1);
-            v.xd = St::get(gr, west ? st.m1 : st.p1);
-            if constexpr (kY) {
-                v.y2 = St::get(gp + (j < 2 ? st.rm2 : st.rp2), st.c);
-                v.y1 = St::get(gp + (j < 2 ? st.rm1 : st.rp1), st.c);
-                v.yd = St::get(gp + (j < 2 ? st.rp1 : st.rm1), st.c);
-            }
-        } else if constexpr (kX) {     // E, W along x; N, S along y
-            const bool up = j & 1, neg = j >= 2;
-            v.x2 = St::get(gp + (up ? (neg ? st.rp2 : st.rm2) : st.row), up ? st.c : (neg ? st.p2 : st.m2));
-            v.x1 = St::get(gp + (up ? (neg ? st.rp1 : st.rm1) : st.row), up ? st.c : (neg ? st.p1 : st.m1));
-            v.xd = St::get(gp + (up ? (neg ? st.rm1 : st.rp1) : st.row), up ? st.c : (neg ? st.m1 : st.p1));
-        }
-        const FxC kx = !kDiag && !kFlatY && (j & 1) ? a.fx.l.kly[grp] : a.fx.l.klx[grp];
-        double o;
-        const bool ok = fx_update<kX, kY, kBase>(a.fx.k, kx, a.fx.l.kly[grp], v, h.member(j), h.G, o);
-        if (live && ok && cell_ok) *(double *)((char *)(out + plane + st.row) + st.c) = o;
-        else rest |= 1u << j;
-    };
-    if constexpr (!kDiag && kFlatY) {
-#pragma unroll kUnroll
-        for (int j = 0; j < 4; j += 2) pass(j, std::true_type{});
-#pragma unroll kUnroll
-        for (int j = 1; j < 4; j += 2) pass(j, std::false_type{});    // N, S of a 1-D grid: no transport
-    } else {
-#pragma unroll kUnroll
-        for (int j = 0; j < 4; ++j) pass(j, std::true_type{});
-    }
-    if (rest && live)
-        fx_rest_of_group<GridCell, kBase, kFlatY>({g, base, out, a.nx, a.ny, a.bc_x, a.bc_y, x, y}, a.eq, a.m, a.fx.k,
-                                                  a.fx.l, {a.a_self, a.a_base, a.lx, a.ly}, grp, rest, cell_ok, h, flag);
-}
-
-// Stage in double precision, one cell per thread (cdbm_stage_fx.cuh).  Bound by the ALU
-// pipe, which takes about 3200 of some 6000 instructions per cell and stage (ncu: 66-73 %
-// busy, the FP64 pipe 48-53 %, issue 60-64 %; against 246 / 262 FP64 instructions of 64
-// cycles each before); 64 registers for 32 warps per SM, which hide the latency of its
-// dependent chains (24 warps 7 % slower, 16 warps 15 %).  6.9 ms per 4096^2 step (15.8 all
-// in FP64), 0.96 ms per 1500 x 1300.
-constexpr int kFxMinBlocks = 8;
-template <bool kBase, bool kFlatY, bool kWide>
-__global__ void __launch_bounds__(kStageThreads, kFxMinBlocks)
-    stage_fx_kernel(const double *__restrict__ g, const double *base, double *out, const __grid_constant__ StageArgs a,
-                    unsigned *flag)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= a.nx) return;
-    const size_t P = (size_t)a.nx * a.ny;
-    GridStencil<kWide> st(x, a.nx, a.bc_x);
-    for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
-        st.template at_row<kFlatY>(y, a.nx, a.ny, a.bc_y);
-        const double *own = g + st.row + x;
-        const FxCons m = fx_conserved(a.fx.m, [=](int i) { return __ldg(own + i * P); });
-        const EqFactors q = eq_factors(a.m, m.rho, m.jx, m.jy, m.E, flag);
-#pragma unroll 1
-        for (int p = 0; p < 4; p += 2) {
-            fx_grid_group<1, false, kFlatY, kBase>(g, base, out, a, st, P, x, y, p, fx_group(a.eq, q, p), m.ok, true, flag);
-            fx_grid_group<1, true, kFlatY, kBase>(g, base, out, a, st, P, x, y, p + 1, fx_group(a.eq, q, p + 1), m.ok, true,
-                                               flag);
-        }
-    }
-}
-
-// The same stage with a cell on two threads: on a grid of some ten thousand cells the time
-// of a stage is the chain of one thread, which this shortens.  Two warps of a block have
-// two velocity groups of 32 cells each; they exchange the groups' largest exponents and
-// sums through shared memory, and each forms the moments and the factors of the
-// equilibrium.  The values are those of stage_fx_kernel.  With few warps per SM the
-// members' passes are unrolled so that their chains overlap.
-template <bool kBase, bool kFlatY>
-__global__ void __launch_bounds__(128, 4)
-    stage_fx_split_kernel(const double *__restrict__ g, const double *base, double *out,
-                          const __grid_constant__ StageArgs a, unsigned *flag)
-{
-    __shared__ uint32_t keys[2][64];
-    __shared__ int64_t sums[4][3][64];
-    const int warp = threadIdx.x >> 5;
-    const int way = warp & 1, at = (warp >> 1) * 32 + (threadIdx.x & 31);
-    const int x0 = blockIdx.x * 64 + at;
-    const bool live = x0 < a.nx;
-    const int x = live ? x0 : a.nx - 1;              // idle lanes mirror the last cell
-    const size_t P = (size_t)a.nx * a.ny;
-    GridStencil<true> st(x, a.nx, a.bc_x);
-    for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
-        st.template at_row<kFlatY>(y, a.nx, a.ny, a.bc_y);
-        const double *own = g + (size_t)(8 * way) * P + st.row + x;
-        double f[8];
-        uint32_t key = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            f[j] = __ldg(own + j * P);
-            key = fx_max(key, fx_key(f[j]));
-        }
-        keys[way][at] = key;
-        __syncthreads();
-        const int top = (int)(fx_max(keys[0][at], keys[1][at]) >> 21);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int grp = 2 * way + k;
-            int64_t q4[4], s0, sx, sy;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) q4[j] = fx_from(f[4 * k + j], top);
-            fx_group_sums(grp, q4, s0, sx, sy);
-            sums[grp][0][at] = s0;
-            sums[grp][1][at] = sx;
-            sums[grp][2][at] = sy;
-        }
-        __syncthreads();
-        FxMoments mo = kFxNoMoments;
-#pragma unroll
-        for (int h = 0; h < 4; ++h) fx_add_sums(a.fx.m, h, sums[h][0][at], sums[h][1][at], sums[h][2][at], mo);
-        const FxCons m = fx_round_moments(a.fx.m, mo, top);
-        const EqFactors q = eq_factors(a.m, m.rho, m.jx, m.jy, m.E, flag);
-        const int grp = 2 * way;
-        fx_grid_group<4, false, kFlatY, kBase>(g, base, out, a, st, P, x, y, grp, fx_group(a.eq, q, grp), m.ok, live, flag);
-        fx_grid_group<4, true, kFlatY, kBase>(g, base, out, a, st, P, x, y, grp + 1, fx_group(a.eq, q, grp + 1), m.ok, live,
-                                              flag);
-        // the next row writes keys[] only after every warp has passed the second barrier
-    }
-}
-
-// The same stage with a cell on 16 threads (fx_cell16): 512 threads per 32 cells of a row.
-template <bool kBase, bool kFlatY>
-__global__ void __launch_bounds__(512, 2)
-    stage_fx_cell16_kernel(const double *__restrict__ g, const double *base, double *out,
-                           const __grid_constant__ StageArgs a, unsigned *flag)
-{
-    __shared__ FxCells16 s;
-    const int w = threadIdx.x >> 5, i = cell16_velocity(w);
-    const int x0 = blockIdx.x * 32 + (int)(threadIdx.x & 31);
-    const bool live = x0 < a.nx;
-    const int x = live ? x0 : a.nx - 1;              // idle lanes mirror the last cell
-    for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
-        const GridCell cell = {g, base, out, a.nx, a.ny, a.bc_x, a.bc_y, x, y};
-        const FxStencil v = cell.stencil<kFlatY>(i, dirx(i), kFlatY ? 0 : diry(i), kBase ? cell.base(i) : 0.0);
-        double o;
-        const bool ok = fx_cell16<kFlatY, kBase>(a, s, w, 0, i, v, flag, o);
-        if (live) {
-            if (ok) cell.put(i, o);
-            else
-                fx_double_group<GridCell, kBase, kFlatY>(cell, a.eq, a.m, {a.a_self, a.a_base, a.lx, a.ly}, i >> 2,
-                                                         1u << (i & 3), flag);
-        }
-        // the next row's first write to what this row still reads (s.h) follows two barriers
     }
 }
 
@@ -719,19 +497,9 @@ RefMoments ref_moments(const FieldArgs &a, bool single)
 __device__ __forceinline__ double stored(double v) { return v; }
 __device__ __forceinline__ double stored(float v) { return widen_f32(v); }
 
-// The conserved moments of a stored cell: in fixed point (cdbm_stage_fx.cuh), or in FP64
-// where its exponents are outside that path.  10 instead of 51 FP64 instructions took
-// the fields of 4096^2 cells from 1.61 to 0.51 ms (0.40 ms at the memory's rate).
+// The conserved moments with the group sums on the integer pipes (cdbm_exact.h): 27 instead
+// of 51 FP64 instructions per cell.
 template <typename TS>
-__device__ __noinline__ Cons conserved_any(const FieldArgs &a, const TS *own, size_t P)
-{
-    double fc[kNV];
-    for (int i = 0; i < kNV; ++i) fc[i] = stored(own[i * P]);
-    return conserved(fc, a.m);
-}
-
-// kDouble: all in FP64, for the read-out of a recorded run (cdbm_stage_double.cu).
-template <typename TS, bool kDouble>
 __global__ void __launch_bounds__(128) macros_kernel(const __grid_constant__ FieldArgs a, const RefMoments F,
                                                      const TS *__restrict__ f, double *rho, double *ux, double *uy,
                                                      double *T)
@@ -739,18 +507,10 @@ __global__ void __launch_bounds__(128) macros_kernel(const __grid_constant__ Fie
     const size_t P = (size_t)a.nx * a.ny;
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < P;
          c += (size_t)gridDim.x * blockDim.x) {
-        const TS *own = f + c;
-        Cons q;
-        if constexpr (kDouble) {
-            double fc[kNV];
+        TS fc[kNV];
 #pragma unroll
-            for (int i = 0; i < kNV; ++i) fc[i] = stored(__ldg(own + i * P));
-            q = conserved(fc, a.m);
-        } else {
-            const FxCons m = fx_conserved(a.fx, [=](int i) { return __ldg(own + i * P); });
-            q = {m.rho, m.jx, m.jy, m.E};
-            if (!m.ok) q = conserved_any(a, own, P);
-        }
+        for (int i = 0; i < kNV; ++i) fc[i] = __ldg(f + i * P + c);
+        Cons q = moments_exact(a.m, fc);
         if constexpr (kSingle<TS>) {
             q.rho += F.rho;
             q.E += F.E;
@@ -784,6 +544,17 @@ TneSet tne_set(const double v[4])
     t.e = fx_exponent(v, 4);
     for (int g = 0; g < 4; ++g) t.k[g] = fx_k(fx_const(std::ldexp(v[g], -t.e), 60));
     return t;
+}
+
+__device__ __forceinline__ bool fx_out_of_range(int E) { return (unsigned)(E - kExpLo) >= (unsigned)kExpSpan; }
+
+// Group sums of the fixed-point members E N W S or NE NW SW SE of group g.
+__device__ __forceinline__ void fx_group_sums(int g, const int64_t q[4], int64_t &s0, int64_t &sx, int64_t &sy)
+{
+    s0 = (q[0] + q[2]) + (q[1] + q[3]);
+    const int64_t d = q[0] - q[2], b = q[1] - q[3];
+    sx = (g & 1) == 0 ? d : d - b;
+    sy = (g & 1) == 0 ? b : d + b;
 }
 
 // The raw moments of a cell up to the fourth order (rows of Eq. 6 at u = 0).
@@ -1088,28 +859,6 @@ void *stage_march2_func(bool with_base, bool vec, bool dev)
     return dev ? stage_march2_func_t<kEqF32>(with_base, vec) : stage_march2_func_t<kEqDF>(with_base, vec);
 }
 
-void *fx_func(bool with_base, bool flat, bool wide)
-{
-    if (wide) {
-        if (with_base) return flat ? (void *)stage_fx_kernel<true, true, true> : (void *)stage_fx_kernel<true, false, true>;
-        return flat ? (void *)stage_fx_kernel<false, true, true> : (void *)stage_fx_kernel<false, false, true>;
-    }
-    if (with_base) return flat ? (void *)stage_fx_kernel<true, true, false> : (void *)stage_fx_kernel<true, false, false>;
-    return flat ? (void *)stage_fx_kernel<false, true, false> : (void *)stage_fx_kernel<false, false, false>;
-}
-
-void *fx_split_func(bool with_base, bool flat)
-{
-    if (with_base) return flat ? (void *)stage_fx_split_kernel<true, true> : (void *)stage_fx_split_kernel<true, false>;
-    return flat ? (void *)stage_fx_split_kernel<false, true> : (void *)stage_fx_split_kernel<false, false>;
-}
-
-void *fx_cell16_func(bool with_base, bool flat)
-{
-    if (with_base) return flat ? (void *)stage_fx_cell16_kernel<true, true> : (void *)stage_fx_cell16_kernel<true, false>;
-    return flat ? (void *)stage_fx_cell16_kernel<false, true> : (void *)stage_fx_cell16_kernel<false, false>;
-}
-
 template <int kEq>
 void *stage_func(bool march, bool with_base, bool flat)
 {
@@ -1133,17 +882,15 @@ cudaError_t launch_init(const FieldArgs &a, const double *rho, const double *ux,
     return cudaGetLastError();
 }
 
-cudaError_t launch_macros(const FieldArgs &a, const void *f, int prec, bool in_double, double *rho, double *ux,
+cudaError_t launch_macros(const FieldArgs &a, const void *f, int prec, double *rho, double *ux,
                           double *uy, double *T, cudaStream_t s)
 {
     const unsigned nb = grid_for((size_t)a.nx * a.ny, 128);
     const RefMoments F = ref_moments(a, single_storage(prec));
     if (single_storage(prec))
-        macros_kernel<float, false><<<nb, 128, 0, s>>>(a, F, (const float *)f, rho, ux, uy, T);
-    else if (in_double)
-        macros_kernel<double, true><<<nb, 128, 0, s>>>(a, F, (const double *)f, rho, ux, uy, T);
+        macros_kernel<float><<<nb, 128, 0, s>>>(a, F, (const float *)f, rho, ux, uy, T);
     else
-        macros_kernel<double, false><<<nb, 128, 0, s>>>(a, F, (const double *)f, rho, ux, uy, T);
+        macros_kernel<double><<<nb, 128, 0, s>>>(a, F, (const double *)f, rho, ux, uy, T);
     return cudaGetLastError();
 }
 
@@ -1203,35 +950,10 @@ cudaError_t launch_field_means(const double *rho, const double *T, size_t n, dou
 StageLaunch stage_launch_config(const StageArgs &a, bool with_base, int sm_count, int prec, bool allow_march,
                                 bool allow_split)
 {
+    if (prec == CDBM_FP64) return double_stage_launch_config(a, with_base, sm_count, allow_split);
     StageLaunch L;
     const bool flat = (a.ny == 1);
     const size_t cells = (size_t)a.nx * a.ny;
-    if (prec == CDBM_FP64) {
-        const unsigned rows = a.ny < 65535 ? a.ny : 65535;
-        // While the grid leaves most of the SMs' threads idle, the time is the chain of
-        // one thread, and the cell is split over 16 or two.  us per stage with 16 threads
-        // per cell, two and one: 5.6 / 12.7 / 24.5 at 64^2, 12.8 / 14.9 / 24.4 at 128^2,
-        // 22.9 / 21.3 / 28.1 at 192^2, 29.8 / 33.3 / 35.7 at 220^2, 37.6 / 35.0 / 37.5 at
-        // 256^2, 42.3 (two) / 39.8 at 270^2; tubes of 2000 cells 4.5 / 9.9 / 20, of 20000
-        // 11.3 / 13.0 / 20, of 30000 15.0 / 13.3 / 20.
-        if (allow_split && cells <= (size_t)sm_count * 440) {
-            const bool many = cells <= (size_t)sm_count * (flat ? 170 : 318);
-            const unsigned per = many ? 32 : 64;
-            L.func = many ? fx_cell16_func(with_base, flat) : fx_split_func(with_base, flat);
-            L.block = dim3(many ? 512 : 128, 1, 1);
-            L.grid = dim3((unsigned)(((size_t)a.nx + per - 1) / per), rows, 1);
-            return L;
-        }
-        // the widest block whose padding past the row's end is least
-        unsigned w = kStageThreads;
-        auto pad = [&](unsigned t) { return ((size_t)a.nx + t - 1) / t * t; };
-        for (unsigned t = kStageThreads / 2; t >= 32; t /= 2)
-            if (pad(t) < pad(w)) w = t;
-        L.func = fx_func(with_base, flat, a.nx >= (1 << 29));
-        L.block = dim3(w, 1, 1);
-        L.grid = dim3((unsigned)(pad(w) / w), rows, 1);
-        return L;
-    }
     // The df64 and single-precision deviation equilibria march two columns per thread
     // (stage_march2_kernel).
     const bool pair = prec == CDBM_FP32_DF64 || prec == CDBM_FP32_DEV;
@@ -1371,7 +1093,6 @@ DFShiftT<float2> df_shift_twice(const DFShift &d)
 
 void fill_df_consts(StageArgs &a)
 {
-    fill_fx_consts(a);
     a.d.b = df_blocks(a.eq);
     a.d.m = df_model(a.m);
     a.d.r = df_shift(a.sF, a.rhoF, a.EF);
@@ -1385,13 +1106,6 @@ void fill_df_consts(StageArgs &a)
         a.lx_f2[g] = make_float2(a.lx_f[g], a.lx_f[g]);
         a.ly_f2[g] = make_float2(a.ly_f[g], a.ly_f[g]);
     }
-}
-
-void fill_fx_consts(StageArgs &a)
-{
-    a.fx.m = fx_model(a.m.c, a.m.w);
-    a.fx.k = fx_coef(a.a_self, a.a_base);
-    a.fx.l = fx_flux(a.lx, a.ly, a.nx > 1, a.ny > 1);
 }
 
 DevProj dev_proj(const ModelConsts &m, double gh)

@@ -145,7 +145,6 @@ extern "C" cdbm_status cdbm_step_noalloc(const cdbm_grid *grid, const cdbm_vset 
         a[s].ny = grid->ny;
         a[s].bc_x = grid->bc_x;
         a[s].bc_y = grid->bc_y;
-        fill_fx_consts(a[s]);
         L[s] = stage_launch_config(a[s], s == 1, sm_count, CDBM_FP64);
     }
 

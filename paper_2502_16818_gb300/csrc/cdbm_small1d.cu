@@ -10,13 +10,12 @@
 // are separated by the cluster barrier, a hardware barrier over the co-scheduled
 // CTAs (no software spin-wait).  In single precision the per-cell arithmetic is
 // that of the flat stage kernel in the same order, so the result is the same bit for
-// bit; the df64 variant splits a cell over two threads (split_stage_df) and the FP64
-// variant over four (split_stage).  The FP64 four-thread split also runs as an
-// ordinary stage launch for tubes too long for one cluster (stage_split_flat_kernel).
+// bit; the df64 variant splits a cell over two threads (split_stage_df), the FP64 variant
+// over 16 (cell16 of cdbm_stage_exact.cuh, the arithmetic of its stage launches).
 #include <cooperative_groups.h>
 
 #include "cdbm_stage.cuh"
-#include "cdbm_stage_fx.cuh"
+#include "cdbm_stage_exact.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -126,137 +125,11 @@ __global__ void __launch_bounds__(256) small1d_kernel(float *f, int nsteps, cons
     }
 }
 
-// The arithmetic of one cell's group g in the four-thread split: from the group's four values q, its base
-// values bs and x stencil values, the four updated values o.  The four threads of a
-// cell are lanes 4c .. 4c + 3 of one warp.
-__device__ __forceinline__ void split_cell(const StageArgs &a, int g, const double q[4], const double bs[4],
-                                           const double up2[4], const double up1[4], const double dn1[4],
-                                           bool with_base, bool live, unsigned *flag, double o[4])
-{
-    const int t = threadIdx.x;
-    // group components, as conserved()
-    double c0, cx, cy;
-    if ((g & 1) == 0) {
-        cx = q[0] - q[2];
-        cy = q[1] - q[3];
-        c0 = (q[0] + q[2]) + (q[1] + q[3]);
-    } else {
-        const double e = q[0] + q[3], w = q[1] + q[2];
-        cx = e - w;
-        cy = (q[0] + q[1]) - (q[2] + q[3]);
-        c0 = e + w;
-    }
-    const int lane0 = (t & 31) & ~3;
-    double S0[4], SX[4], SY[4];
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-        S0[h] = __shfl_sync(0xffffffffu, c0, lane0 + h);
-        SX[h] = __shfl_sync(0xffffffffu, cx, lane0 + h);
-        SY[h] = __shfl_sync(0xffffffffu, cy, lane0 + h);
-    }
-    const ModelConsts &m = a.m;
-    Prim s;
-    s.q.rho = (S0[0] + S0[1]) + (S0[2] + S0[3]);
-    s.q.jx = fma(m.c[3], SX[3], fma(m.c[2], SX[2], fma(m.c[1], SX[1], m.c[0] * SX[0])));
-    s.q.jy = fma(m.c[3], SY[3], fma(m.c[2], SY[2], fma(m.c[1], SY[1], m.c[0] * SY[0])));
-    s.q.E = fma(m.w[3], S0[3], fma(m.w[2], S0[2], fma(m.w[1], S0[1], m.w[0] * S0[0])));
-    const double r = rcp64(s.q.rho);
-    s.ux = s.q.jx * r;
-    s.uy = s.q.jy * r;
-    s.jyuy = s.q.jy * s.uy;
-    s.ru2 = fma(s.q.jx, s.ux, s.jyuy);
-    s.p = (s.q.E - s.ru2) * m.invK;
-    s.T = s.p * r;
-    if (live && g == 0 && !(positive_finite(s.q.rho) && positive_finite(s.p))) atomicOr(flag, kFlagNonPhys);
-    // this group's part of equilibrium()
-    const EqBlocks &B = a.eq;
-    const double ux2 = s.ux * s.ux, uy2 = s.uy * s.uy, u2 = ux2 + uy2, dlt = ux2 - uy2;
-    const double m1416 = fma(s.T, fma(m.Kp6, s.ru2, m.twoKp2 * s.p), s.ru2 * u2);
-    const double W4 = fma(m.Kp4, s.T, u2);
-    const double d57 = fma(s.q.jx, s.ux, -s.jyuy);
-    const double m6 = s.q.jx * s.uy;
-    const double *S = B.S + 4 * g;
-    const double e0 = fma(S[3], m1416, fma(S[2], s.ru2, fma(S[1], s.q.E, S[0] * s.q.rho)));
-    const double qv = (g & 1) == 0 ? d57 * fma(B.B1[g + 1], W4, B.B1[g])       // g = 0: a, g = 2: c
-                                   : m6 * fma(B.B2[g], W4, B.B2[g - 1]);       // g = 1: b, g = 3: d
-    double heq[4];
-    equilibrium_group(B, g, e0, qv, s.q.jx, s.q.jy, s.T, u2, dlt, heq);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int i = 4 * g + j;
-        o[j] = fma(a.a_self, q[j], heq[j]);
-        if (with_base) o[j] = fma(a.a_base, bs[j], o[j]);
-        if (dirx(i) != 0) o[j] = fma(-a.lx[g], nnd(up2[j], up1[j], q[j], dn1[j]), o[j]);
-    }
-}
-
-// One FP64 stage of a 1-D grid as an ordinary launch with each cell split over four
-// threads (split_cell), for tubes too long for the cluster kernel.  With one thread
-// per cell a tube of a few thousand cells leaves about a warp per SM, and the chain
-// of dependent FP64 instructions of one cell, not the launch, sets the time of a
-// stage; four threads per cell shorten that chain.  Threads past the last cell
-// mirror it (they take part in the shuffles) and store nothing.
-template <bool kBase>
-__global__ void __launch_bounds__(kSplitFlatThreads) stage_split_flat_kernel(const double *__restrict__ g,
-                                                                             const double *base, double *out,
-                                                                             const StageArgs a, unsigned *flag)
-{
-    const int t = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    const int gq = t & 3;                             // velocity group of this thread
-    const int x0 = t >> 2;
-    const int nx = a.nx;
-    const bool live = x0 < nx;
-    const int x = live ? x0 : nx - 1;
-    const size_t P = (size_t)nx;                      // ny = 1
-    double q[4], bs[4], up2[4], up1[4], dn1[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        q[j] = g[(4 * gq + j) * P + x];
-        bs[j] = kBase ? base[(4 * gq + j) * P + x] : 0.0;
-    }
-    const int xm2 = neighbour_near(x - 2, nx, a.bc_x), xm1 = neighbour_near(x - 1, nx, a.bc_x);
-    const int xp1 = neighbour_near(x + 1, nx, a.bc_x), xp2 = neighbour_near(x + 2, nx, a.bc_x);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int i = 4 * gq + j;
-        const int sx = dirx(i);
-        const double *p = g + i * P;
-        up2[j] = sx == 0 ? 0.0 : p[sx > 0 ? xm2 : xp2];
-        up1[j] = sx == 0 ? 0.0 : p[sx > 0 ? xm1 : xp1];
-        dn1[j] = sx == 0 ? 0.0 : p[sx > 0 ? xp1 : xm1];
-    }
-    double o[4];
-    split_cell(a, gq, q, bs, up2, up1, dn1, kBase, live, flag, o);
-    if (live) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) out[(4 * gq + j) * P + x] = o[j];
-    }
-}
-
-// Access to one cell of the cluster's state for fx_double_group().
-struct ClusterCell {
-    const double *src, *b;
-    double *dst;
-    int chunk, rank, nx, bc, x;
-    __device__ double at(int i, int gx) const
-    {
-        return cluster_value(cg::this_cluster(), src, chunk, rank, i, gx);
-    }
-    template <bool kFlatY>
-    __device__ FxStencil stencil(int i, int dx, int, double base) const
-    {
-        return {at(i, x), at(i, neighbour_near(x - 2 * dx, nx, bc)), at(i, neighbour_near(x - dx, nx, bc)),
-                at(i, neighbour_near(x + dx, nx, bc)), 0, 0, 0, base};
-    }
-    __device__ double base(int i) const { return b[i * chunk + (x - rank * chunk)]; }
-    __device__ void put(int i, double v) const { dst[i * chunk + (x - rank * chunk)] = v; }
-};
-
-// FP64 stage in the cluster, a cell on 16 threads (fx_cell16): warp w of the CTA has
+// FP64 stage in the cluster, a cell on 16 threads (cell16): warp w of the CTA has
 // the velocity cell16_velocity(w mod 16) of the cells 32 (w / 16) .. + 31 of the CTA's chunk.
 template <bool kBase>
 __device__ __forceinline__ void cluster_stage16(const cg::cluster_group &cl, const double *src, const double *base,
-                                                double *dst, const StageArgs &a, FxCells16 *s, int chunk, int rank, int x0,
+                                                double *dst, const StageArgs &a, Cells16 *s, int chunk, int rank, int x0,
                                                 int len, unsigned *flag)
 {
     const int w = threadIdx.x >> 5, i = cell16_velocity(w & 15), set = w >> 4, nx = a.nx;
@@ -265,7 +138,7 @@ __device__ __forceinline__ void cluster_stage16(const cg::cluster_group &cl, con
     const int lx = live ? l0 : len - 1;               // idle lanes mirror the last cell
     const int gx = x0 + lx;
     const double c = src[i * chunk + lx];
-    FxStencil v = {c, c, c, c, 0, 0, 0, kBase ? base[i * chunk + lx] : 0.0};
+    Stencil v = {c, c, c, c, 0, 0, 0, kBase ? base[i * chunk + lx] : 0.0};
     const int d = dirx(i);
     if (d != 0) {
         if (lx >= 2 && lx + 2 < len) {
@@ -279,22 +152,17 @@ __device__ __forceinline__ void cluster_stage16(const cg::cluster_group &cl, con
             v.xd = cluster_value(cl, src, chunk, rank, i, neighbour_near(gx + d, nx, a.bc_x));
         }
     }
-    double o;
-    const bool ok = fx_cell16<true, kBase>(a, s[set], w & 15, set, i, v, flag, o);
-    if (!live) return;
-    if (ok) dst[i * chunk + lx] = o;
-    else
-        fx_double_group<ClusterCell, kBase, true>({src, base, dst, chunk, rank, nx, a.bc_x, gx}, a.eq, a.m,
-                                                  {a.a_self, a.a_base, a.lx, a.ly}, i >> 2, 1u << (i & 3), flag);
+    const double o = cell16<true, kBase, true>(a, s[set], w & 15, set, i, v, flag);
+    if (live) dst[i * chunk + lx] = o;
 }
 
-__global__ void __launch_bounds__(1024) small1d_fx_kernel(double *f, int nsteps, const __grid_constant__ StageArgs a0,
+__global__ void __launch_bounds__(1024) small1d_double_kernel(double *f, int nsteps, const __grid_constant__ StageArgs a0,
                                                           const __grid_constant__ StageArgs a1, unsigned *flag, int chunk)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *s0 = reinterpret_cast<double *>(smem_raw);
     double *s1 = s0 + kNV * chunk;
-    FxCells16 *cells = reinterpret_cast<FxCells16 *>(s1 + kNV * chunk);
+    Cells16 *cells = reinterpret_cast<Cells16 *>(s1 + kNV * chunk);
     const cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const int nx = a0.nx;
@@ -431,15 +299,10 @@ void *small1d_func_of(int prec, int chunk)
         return chunk <= kSplitDfMaxChunk ? (void *)small1d_split_df_kernel : small1d_func<kEqDF>();
     if (prec == CDBM_FP32_DEV) return small1d_func<kEqF32>();
     if (prec == CDBM_FP32_BULK) return small1d_func<kEqDouble>();
-    return (void *)small1d_fx_kernel;
+    return (void *)small1d_double_kernel;
 }
 
 }  // namespace
-
-void *split_flat_func(bool with_base)
-{
-    return with_base ? (void *)stage_split_flat_kernel<true> : (void *)stage_split_flat_kernel<false>;
-}
 
 Small1D small1d_config(const StageArgs &a, int prec)
 {
@@ -458,7 +321,7 @@ Small1D small1d_config(const StageArgs &a, int prec)
     cluster = (a.nx + chunk - 1) / chunk;            // no empty CTAs
     const int sets = (chunk + 31) / 32;               // FP64: 32 cells on 16 warps each
     const size_t smem = 2 * kNV * (size_t)chunk * storage_bytes(prec) +
-                        (prec == CDBM_FP64 ? sets * sizeof(FxCells16) : 0);
+                        (prec == CDBM_FP64 ? sets * sizeof(Cells16) : 0);
     // df64: two threads per cell (split_stage_df, up to kSplitDfMaxChunk cells), all cells
     // of the CTA in one pass
     const int per_cell = prec == CDBM_FP32_DF64 && chunk <= kSplitDfMaxChunk ? 2 : 1;

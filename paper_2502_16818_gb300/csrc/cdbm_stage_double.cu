@@ -1,295 +1,242 @@
-// Runge-Kutta stage kernels of the double-precision state entirely in FP64, for the run
-// that the adjoint differentiates (cdbm_adjoint_forward and the recomputation of its
-// segments).  cdbm_step takes the fixed-point kernels (cdbm_stage_fx.cuh), which agree to
-// rounding and are twice as fast; but dL/dtau sums o . (f - f_eq) over the run, where
-// f - f_eq is 1e-5 of f and the sum cancels over the cells, so it carries the rounding of
-// every stage at 1e-9 to 1e-6 of its value.  Recorded gradients stay reproducible to the
-// bit only with the rounding they were recorded with.
-#include "cdbm_device.cuh"
+// Runge-Kutta stage kernels of the double-precision state on a grid: a cell per thread, on
+// two threads or on 16, all with the same values bit for bit (cdbm_stage_exact.cuh).
+#include "cdbm_stage_exact.cuh"
 
 namespace cdbm {
 
 namespace {
 
 constexpr int kThreads = 128;
-constexpr int kMinBlocks = 3;     // resident blocks per SM the register budget must allow (168 registers)
 
-__device__ __forceinline__ void stage_equilibrium(const StageArgs &a, const double f[kNV], double heq[kNV], unsigned *flag)
-{
-    const Prim s = primitives<false>(f, a.m, 0.0, 0.0, flag);
-    equilibrium<false>(a.eq, a.m, s.q.rho, s.q.E, s.q.jx, s.q.jy, s.ux, s.uy, s.ru2, s.jyuy, s.p, s.T, heq);
-}
-
-// out = a_base base + a_self g + gamma h f_eq(g) - sum_r l_r D_r(g) for one cell:
-// macros -> equilibrium -> BGK -> NND transport of all 16 velocities -> update.
-template <bool kBase, bool kFlatY>
-__global__ void __launch_bounds__(kThreads, kMinBlocks)
-    stage_kernel(const double *__restrict__ g, const double *base, double *out, const StageArgs a, unsigned *flag)
-{
-    const int nx = a.nx, ny = a.ny;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= nx) return;
-    const size_t P = (size_t)nx * ny;
-    const int xm2 = neighbour_near(x - 2, nx, a.bc_x), xm1 = neighbour_near(x - 1, nx, a.bc_x);
-    const int xp1 = neighbour_near(x + 1, nx, a.bc_x), xp2 = neighbour_near(x + 2, nx, a.bc_x);
-    for (int y = blockIdx.y; y < ny; y += gridDim.y) {
-        const size_t row = (size_t)y * nx;
-        const size_t c = row + x;
-        size_t rm2 = 0, rm1 = 0, rp1 = 0, rp2 = 0;
+// Row pointers and offsets of a cell's stencil.  The row pointers are uniform over a
+// block, the offsets in a row 32 bits wide (kWide: 64 bits, for rows of 2^29 cells and
+// more), which saves the 64-bit address arithmetic of about 100 loads per cell.
+template <bool kWide>
+struct GridStencil {
+    using Off = std::conditional_t<kWide, size_t, unsigned>;
+    Off c, m2, m1, p1, p2;
+    size_t row, rm2, rm1, rp1, rp2;
+    __device__ __forceinline__ GridStencil(int x, int nx, int bc)
+        : c((Off)8 * x), m2((Off)8 * neighbour_near(x - 2, nx, bc)), m1((Off)8 * neighbour_near(x - 1, nx, bc)),
+          p1((Off)8 * neighbour_near(x + 1, nx, bc)), p2((Off)8 * neighbour_near(x + 2, nx, bc))
+    {
+    }
+    template <bool kFlatY>
+    __device__ __forceinline__ void at_row(int y, int nx, int ny, int bc)
+    {
+        row = (size_t)y * nx;
         if (!kFlatY) {
-            rm2 = (size_t)neighbour_near(y - 2, ny, a.bc_y) * nx + x;
-            rm1 = (size_t)neighbour_near(y - 1, ny, a.bc_y) * nx + x;
-            rp1 = (size_t)neighbour_near(y + 1, ny, a.bc_y) * nx + x;
-            rp2 = (size_t)neighbour_near(y + 2, ny, a.bc_y) * nx + x;
+            rm2 = (size_t)neighbour_near(y - 2, ny, bc) * nx;
+            rm1 = (size_t)neighbour_near(y - 1, ny, bc) * nx;
+            rp1 = (size_t)neighbour_near(y + 1, ny, bc) * nx;
+            rp2 = (size_t)neighbour_near(y + 2, ny, bc) * nx;
         }
-        double fs[kNV];
-#pragma unroll
-        for (int i = 0; i < kNV; ++i) fs[i] = __ldg(g + i * P + c);
-        double heq[kNV];
-        stage_equilibrium(a, fs, heq, flag);
+    }
+    static __device__ __forceinline__ double get(const double *p, Off o) { return __ldg((const double *)((const char *)p + o)); }
+};
 
-#pragma unroll
-        for (int i = 0; i < kNV; ++i) {
-            const int grp = i >> 2;
-            const double *gp = g + i * P;
-            double o = fma(a.a_self, fs[i], heq[i]);
-            if (kBase) o = fma(a.a_base, base[i * P + c], o);
-            if (dirx(i) != 0) {
-                const double u2 = __ldg(gp + row + (dirx(i) > 0 ? xm2 : xp2));
-                const double u1 = __ldg(gp + row + (dirx(i) > 0 ? xm1 : xp1));
-                const double d1 = __ldg(gp + row + (dirx(i) > 0 ? xp1 : xm1));
-                o = fma(-a.lx[grp], nnd(u2, u1, fs[i], d1), o);
-            }
-            if (!kFlatY && diry(i) != 0) {
-                const double u2 = __ldg(gp + (diry(i) > 0 ? rm2 : rp2));
-                const double u1 = __ldg(gp + (diry(i) > 0 ? rm1 : rp1));
-                const double d1 = __ldg(gp + (diry(i) > 0 ? rp1 : rm1));
-                o = fma(-a.ly[grp], nnd(u2, u1, fs[i], d1), o);
-            }
-            out[i * P + c] = o;
+// The four members of group grp of one cell: loads, update and stores, one member per
+// pass.  The passes differ in the offsets of the neighbours only and share their code:
+// unrolled, the members' independent chains overlap, but the code outgrows the instruction
+// cache as soon as other paths run beside it.
+template <int kUnroll, bool kDiag, bool kFlatY, bool kBase, bool kWide>
+__device__ __forceinline__ void grid_group(const double *g, const double *base, double *out, const StageArgs &a,
+                                           const GridStencil<kWide> &st, size_t P, int grp, const EqGroup h, bool live)
+{
+    using St = GridStencil<kWide>;
+    auto pass = [&](int j, auto transport) {
+        constexpr bool kX = decltype(transport)::value;
+        const size_t plane = (4 * grp + j) * P;
+        const double *gp = g + plane, *gr = gp + st.row;
+        const double c = St::get(gr, st.c);
+        double o = fma(a.a_self, c, h.member(j));
+        if (kBase) o = fma(a.a_base, *(const double *)((const char *)(base + plane + st.row) + st.c), o);
+        if constexpr (kX && (kDiag || kFlatY)) {
+            const bool west = kDiag ? j == 1 || j == 2 : j == 2;
+            o = fma(-a.lx[grp], nnd_exact(St::get(gr, west ? st.p2 : st.m2), St::get(gr, west ? st.p1 : st.m1), c,
+                                          St::get(gr, west ? st.m1 : st.p1)), o);
+            if constexpr (kDiag && !kFlatY)
+                o = fma(-a.ly[grp], nnd_exact(St::get(gp + (j < 2 ? st.rm2 : st.rp2), st.c),
+                                              St::get(gp + (j < 2 ? st.rm1 : st.rp1), st.c), c,
+                                              St::get(gp + (j < 2 ? st.rp1 : st.rm1), st.c)), o);
+        } else if constexpr (kX) {     // E, W along x; N, S along y
+            const bool up = j & 1, neg = j >= 2;
+            const double u2 = St::get(gp + (up ? (neg ? st.rp2 : st.rm2) : st.row), up ? st.c : (neg ? st.p2 : st.m2));
+            const double u1 = St::get(gp + (up ? (neg ? st.rp1 : st.rm1) : st.row), up ? st.c : (neg ? st.p1 : st.m1));
+            const double d1 = St::get(gp + (up ? (neg ? st.rm1 : st.rp1) : st.row), up ? st.c : (neg ? st.m1 : st.p1));
+            o = fma(-(up ? a.ly[grp] : a.lx[grp]), nnd_exact(u2, u1, c, d1), o);
         }
+        if (live) *(double *)((char *)(out + plane + st.row) + st.c) = o;
+    };
+    if constexpr (!kDiag && kFlatY) {
+#pragma unroll kUnroll
+        for (int j = 0; j < 4; j += 2) pass(j, std::true_type{});
+#pragma unroll kUnroll
+        for (int j = 1; j < 4; j += 2) pass(j, std::false_type{});    // N, S of a 1-D grid: no transport
+    } else {
+#pragma unroll kUnroll
+        for (int j = 0; j < 4; ++j) pass(j, std::true_type{});
     }
 }
 
-// Same stage for 2-D grids with the y-direction differences shared along a run of
-// rows.  A block covers kThreads columns and a run of R = ceil(ny / gridDim.y)
-// rows; each thread marches up its column.  For a velocity with y-sign s the
-// upwind-ordered difference U_y = f_y - f_{y-s} and N_y = minmod(U_{y+s}, U_y) give
-// the transport difference U_y + (N_y - N_{y-s}) / 2, which is the nnd() expression
-// with a = U_y, b = U_{y-s}, e = U_{y+s}.  Each row computes one new U and one new N
-// per velocity and carries them to the next row in shared memory, so a y-term costs
-// 4 instead of 6 arithmetic instructions, with the same operations as stage_kernel.
-constexpr int kNY = 12;                             // velocities with a y-component
-constexpr size_t kMarchRowBytes = 2 * 12 * (kThreads + 2) * sizeof(double);   // FP64 x row buffers
-__host__ __device__ constexpr int yvel(int k)       // k-th velocity with diry != 0
-{
-    return k < 2 ? 1 + 2 * k : (k < 6 ? k + 2 : (k < 8 ? 9 + 2 * (k - 6) : k + 4));
-}
-
-template <bool kBase>
+// Stage in double precision, one cell per thread.  Bound by the FP64 pipe (146 / 162
+// instructions of 64 cycles in the two stages); with all sums and differences on that pipe
+// it took 246 / 262 at best, rows marched and differences shared.  4.59 ms per 4096^2 stage
+// of the vortex (7.91 before), 0.557 per 1500 x 1300 of smooth fields (1.02).  64 registers
+// for 32 warps per SM, which hide the latency of the integer chains (20 warps: 4.59-4.72 and
+// 0.563-0.576, 16: 4.75 and 0.564).
+constexpr int kMinBlocks = 8;
+template <bool kBase, bool kFlatY, bool kRounded, bool kWide>
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
-    stage_march_kernel(const double *__restrict__ g, const double *base, double *out, const StageArgs a, unsigned *flag)
+    stage_double_kernel(const double *__restrict__ g, const double *base, double *out, const __grid_constant__ StageArgs a,
+                        unsigned *flag)
 {
-    // The x differences are shared as well: each thread computes
-    // U_x = f_x - f_{x-s} of its cell once per velocity and reads U_{x+s}, U_{x-s} of
-    // its neighbours from a row buffer (double-buffered in dynamic shared memory, so
-    // one block barrier per row; the edge threads add the halo values), so an x-term
-    // costs 4 FP64 instructions plus a share of the halo instead of 6.  The operands and operations are those of nnd(), so the
-    // result is the same bit for bit.
-    constexpr int kNXV = 12;                          // velocities with an x component
-    __shared__ double carry_u[kNY][kThreads];
-    __shared__ double carry_n[kNY][kThreads];
-    extern __shared__ __align__(16) unsigned char march_dyn[];   // [2][kNXV][kThreads + 2] double
-    double(*const row_buf)[kThreads + 2] = reinterpret_cast<double(*)[kThreads + 2]>(march_dyn);
-    const int nx = a.nx, ny = a.ny;
-    const int tid = threadIdx.x;
-    const int x = blockIdx.x * blockDim.x + tid;
-    const bool active = x < nx;
-    const int R = (ny + gridDim.y - 1) / gridDim.y;
-    const int y0 = blockIdx.y * R;
-    const int y1 = y0 + R < ny ? y0 + R : ny;
-    if (y0 >= y1) return;                             // the same for the whole block
-    const int last = (nx - (int)(blockIdx.x * blockDim.x) < (int)blockDim.x
-                          ? nx - (int)(blockIdx.x * blockDim.x) : (int)blockDim.x) - 1;   // last active thread
-    const size_t P = (size_t)nx * ny;
-    const int xc = active ? x : nx - 1;               // inactive threads only pass the barriers
-    const int xm2 = neighbour_near(xc - 2, nx, a.bc_x), xm1 = neighbour_near(xc - 1, nx, a.bc_x);
-    const int xp1 = neighbour_near(xc + 1, nx, a.bc_x), xp2 = neighbour_near(xc + 2, nx, a.bc_x);
-
-    // prologue: U_{y0} and N_{y0 - 1} for s = +1, N_{y0} for s = -1
-    if (active) {
-        const size_t r0 = (size_t)y0 * nx + x;
-        const size_t rm1 = (size_t)neighbour_near(y0 - 1, ny, a.bc_y) * nx + x;
-        const size_t rm2 = (size_t)neighbour_near(y0 - 2, ny, a.bc_y) * nx + x;
-        const size_t rp1 = (size_t)neighbour_near(y0 + 1, ny, a.bc_y) * nx + x;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= a.nx) return;
+    const size_t P = (size_t)a.nx * a.ny;
+    GridStencil<kWide> st(x, a.nx, a.bc_x);
+    for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
+        st.template at_row<kFlatY>(y, a.nx, a.ny, a.bc_y);
+        const double *own = g + st.row + x;
+        double f[kNV];
 #pragma unroll
-        for (int k = 0; k < kNY; ++k) {
-            const int i = yvel(k);
-            const double *gp = g + i * P;
-            const double f0 = __ldg(gp + r0), fm1 = __ldg(gp + rm1);
-            if (diry(i) > 0) {
-                const double u = f0 - fm1;                    // U_{y0}
-                const double um = fm1 - __ldg(gp + rm2);      // U_{y0-1}
-                carry_u[k][tid] = u;
-                carry_n[k][tid] = minmod(u, um);          // N_{y0-1}
-            } else {
-                const double u = f0 - __ldg(gp + rp1);        // U_{y0}
-                const double um = fm1 - f0;                   // U_{y0-1}
-                carry_u[k][tid] = u;
-                carry_n[k][tid] = minmod(um, u);          // N_{y0}
-            }
-        }
-    }
-
-    for (int y = y0; y < y1; ++y) {
-        const size_t row = (size_t)y * nx;
-        const size_t c = row + xc;
-        // row y writes buffer y & 1; its readers have passed the next row's barrier
-        // before row y + 2 writes the same buffer again
-        double(*const row_u)[kThreads + 2] = row_buf + (y & 1) * kNXV;
-        double fs[kNV], o[kNV];
-        if (active) {
-#pragma unroll
-            for (int i = 0; i < kNV; ++i) fs[i] = __ldg(g + i * P + c);
-            double heq[kNV];
-            stage_equilibrium(a, fs, heq, flag);
-            int k = 0;
-#pragma unroll
-            for (int i = 0; i < kNV; ++i) {
-                o[i] = fma(a.a_self, fs[i], heq[i]);
-                if (kBase) o[i] = fma(a.a_base, base[i * P + c], o[i]);
-                if (dirx(i) != 0) {
-                    const double *gp = g + i * P + row;
-                    const double u1 = __ldg(gp + (dirx(i) > 0 ? xm1 : xp1));
-                    row_u[k][tid + 1] = fs[i] - u1;            // U at x: the upwind-ordered a of nnd()
-                    ++k;
-                }
-            }
-        }
-        {
-            // Halo of the row buffer: U_{x-1} left of the block and U_{x+1} right of it (the
-            // e or b of nnd() of the edge cells).  One branch taken by the edge threads only,
-            // so the other warps do not issue these instructions.
-            if (active && tid == 0) {
-                int k = 0;
-#pragma unroll
-                for (int i = 0; i < kNV; ++i) {
-                    if (dirx(i) == 0) continue;
-                    const double *gp = g + i * P + row;
-                    row_u[k][0] = dirx(i) > 0 ? __ldg(gp + xm1) - __ldg(gp + xm2) : __ldg(gp + xm1) - fs[i];
-                    ++k;
-                }
-            }
-            if (active && tid == last) {
-                int k = 0;
-#pragma unroll
-                for (int i = 0; i < kNV; ++i) {
-                    if (dirx(i) == 0) continue;
-                    const double *gp = g + i * P + row;
-                    row_u[k][last + 2] = dirx(i) > 0 ? __ldg(gp + xp1) - fs[i] : __ldg(gp + xp1) - __ldg(gp + xp2);
-                    ++k;
-                }
-            }
-            __syncthreads();
-            if (active) {
-                int k = 0;
-#pragma unroll
-                for (int i = 0; i < kNV; ++i) {
-                    if (dirx(i) == 0) continue;
-                    const int s = dirx(i);
-                    const double av = row_u[k][tid + 1];              // c - u1
-                    const double bv = row_u[k][tid + 1 + s];          // d1 - c
-                    const double ev = row_u[k][tid + 1 - s];          // u1 - u2
-                    const double t = minmod(bv, av) - minmod(av, ev);
-                    o[i] = fma(-a.lx[i >> 2], fma(0.5, t, av), o[i]);
-                    ++k;
-                }
-            }
-        }
-        if (active) {
-            const size_t rp1 = (size_t)neighbour_near(y + 1, ny, a.bc_y) * nx + x;
-            const size_t rp2 = (size_t)neighbour_near(y + 2, ny, a.bc_y) * nx + x;
-#pragma unroll
-            for (int k = 0; k < kNY; ++k) {
-                const int i = yvel(k);
-                const double *gp = g + i * P;
-                const double u = carry_u[k][tid];
-                const double n = carry_n[k][tid];
-                double t;
-                if (diry(i) > 0) {
-                    const double un = __ldg(gp + rp1) - fs[i];                  // U_{y+1}
-                    const double nn = minmod(un, u);                            // N_y
-                    t = nn - n;                                             // N_y - N_{y-1}
-                    carry_u[k][tid] = un;
-                    carry_n[k][tid] = nn;
-                } else {
-                    const double un = __ldg(gp + rp1) - __ldg(gp + rp2);        // U_{y+1}
-                    const double nn = minmod(u, un);                            // N_{y+1}
-                    t = n - nn;                                             // N_y - N_{y+1}
-                    carry_u[k][tid] = un;
-                    carry_n[k][tid] = nn;
-                }
-                o[i] = fma(-a.ly[i >> 2], fma(0.5, t, u), o[i]);
-            }
-#pragma unroll
-            for (int i = 0; i < kNV; ++i) out[i * P + c] = o[i];
+        for (int i = 0; i < kNV; ++i) f[i] = __ldg(own + i * P);
+        const Cons m = moments_exact(a.m, f);
+        const EqFactors q = eq_factors(a.m, m.rho, m.jx, m.jy, m.E, flag);
+#pragma unroll 1
+        for (int p = 0; p < 4; p += 2) {
+            grid_group<1, false, kFlatY, kBase>(g, base, out, a, st, P, p, eq_group<false>(a.eq, q, p, kRounded), true);
+            grid_group<1, true, kFlatY, kBase>(g, base, out, a, st, P, p + 1, eq_group<true>(a.eq, q, p + 1, kRounded), true);
         }
     }
 }
 
-template <bool kBase>
-void *stage_func(bool march, bool flat)
+// The same stage with a cell on two threads: on a grid of some ten thousand cells the time
+// of a stage is the chain of one thread, which this shortens.  Two warps of a block have
+// two velocity groups of 32 cells each; they exchange the groups' sums through shared
+// memory, and each forms the moments and the factors of the equilibrium.  With few warps
+// per SM the members' passes are unrolled so that their chains overlap.
+template <bool kBase, bool kFlatY, bool kRounded>
+__global__ void __launch_bounds__(128, 4)
+    stage_double_split_kernel(const double *__restrict__ g, const double *base, double *out,
+                              const __grid_constant__ StageArgs a, unsigned *flag)
 {
-    if (march) return (void *)stage_march_kernel<kBase>;
-    return flat ? (void *)stage_kernel<kBase, true> : (void *)stage_kernel<kBase, false>;
+    // by parity of the row: a warp that has passed the next row's barrier writes the other
+    // half, and the half it reads is written again only after one more barrier
+    __shared__ double sums[2][4][3][64];
+    const int warp = threadIdx.x >> 5;
+    const int way = warp & 1, at = (warp >> 1) * 32 + (threadIdx.x & 31);
+    const int x0 = blockIdx.x * 64 + at;
+    const bool live = x0 < a.nx;
+    const int x = live ? x0 : a.nx - 1;              // idle lanes mirror the last cell
+    const size_t P = (size_t)a.nx * a.ny;
+    GridStencil<true> st(x, a.nx, a.bc_x);
+    int b = 0;
+    for (int y = blockIdx.y; y < a.ny; y += gridDim.y, b ^= 1) {
+        st.template at_row<kFlatY>(y, a.nx, a.ny, a.bc_y);
+        const double *own = g + (size_t)(8 * way) * P + st.row + x;
+        const int grp = 2 * way;
+        double f[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) f[j] = __ldg(own + j * P);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const GroupSums s = ex_group_sums(k, f + 4 * k);
+            sums[b][grp + k][0][at] = s.s0;
+            sums[b][grp + k][1][at] = s.sx;
+            sums[b][grp + k][2][at] = s.sy;
+        }
+        __syncthreads();
+        double s0[4], sx[4], sy[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            s0[h] = sums[b][h][0][at];
+            sx[h] = sums[b][h][1][at];
+            sy[h] = sums[b][h][2][at];
+        }
+        const Cons m = group_moments(a.m, s0, sx, sy);
+        const EqFactors q = eq_factors(a.m, m.rho, m.jx, m.jy, m.E, flag);
+        grid_group<4, false, kFlatY, kBase>(g, base, out, a, st, P, grp, eq_group<false>(a.eq, q, grp, kRounded), live);
+        grid_group<4, true, kFlatY, kBase>(g, base, out, a, st, P, grp + 1, eq_group<true>(a.eq, q, grp + 1, kRounded), live);
+    }
+}
+
+// The same stage with a cell on 16 threads (cell16): 512 threads per 32 cells of a row.
+template <bool kBase, bool kFlatY, bool kRounded>
+__global__ void __launch_bounds__(512, 2)
+    stage_double_cell16_kernel(const double *__restrict__ g, const double *base, double *out,
+                               const __grid_constant__ StageArgs a, unsigned *flag)
+{
+    __shared__ Cells16 s;
+    const int w = threadIdx.x >> 5, i = cell16_velocity(w);
+    const int x0 = blockIdx.x * 32 + (int)(threadIdx.x & 31);
+    const bool live = x0 < a.nx;
+    const int x = live ? x0 : a.nx - 1;              // idle lanes mirror the last cell
+    const int dx = dirx(i), dy = kFlatY ? 0 : diry(i);
+    const size_t P = (size_t)a.nx * a.ny;
+    const int xm2 = neighbour_near(x - 2 * dx, a.nx, a.bc_x), xm1 = neighbour_near(x - dx, a.nx, a.bc_x),
+              xp1 = neighbour_near(x + dx, a.nx, a.bc_x);
+    for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
+        const double *gp = g + i * P, *gr = gp + (size_t)y * a.nx;
+        const size_t c = i * P + (size_t)y * a.nx + x;
+        Stencil v = {gr[x], gr[xm2], gr[xm1], gr[xp1], 0, 0, 0, kBase ? base[c] : 0.0};
+        if (!kFlatY) {
+            v.y2 = gp[(size_t)neighbour_near(y - 2 * dy, a.ny, a.bc_y) * a.nx + x];
+            v.y1 = gp[(size_t)neighbour_near(y - dy, a.ny, a.bc_y) * a.nx + x];
+            v.yd = gp[(size_t)neighbour_near(y + dy, a.ny, a.bc_y) * a.nx + x];
+        }
+        const double o = cell16<kFlatY, kBase, kRounded>(a, s, w, 0, i, v, flag);
+        if (live) out[c] = o;
+        // the next row's writes to what this row still reads (s.h) follow four barriers
+    }
+}
+
+template <bool kBase, bool kFlatY, bool kRounded>
+void *stage_func(int ways, bool wide)
+{
+    if (ways == 16) return (void *)stage_double_cell16_kernel<kBase, kFlatY, kRounded>;
+    if (ways == 2) return (void *)stage_double_split_kernel<kBase, kFlatY, kRounded>;
+    if constexpr (!kRounded) {
+        if (wide) return (void *)stage_double_kernel<kBase, kFlatY, false, true>;
+    }
+    return (void *)stage_double_kernel<kBase, kFlatY, kRounded, false>;
+}
+
+template <bool kBase>
+void *stage_func(int ways, bool flat, bool rounded, bool wide)
+{
+    if (!flat) return stage_func<kBase, false, false>(ways, wide);
+    return rounded ? stage_func<kBase, true, true>(ways, wide) : stage_func<kBase, true, false>(ways, wide);
 }
 
 }  // namespace
 
-StageLaunch double_stage_launch_config(const StageArgs &a, bool with_base, int sm_count, bool allow_march,
-                                       bool allow_split)
+StageLaunch double_stage_launch_config(const StageArgs &a, bool with_base, int sm_count, bool allow_split)
 {
     StageLaunch L;
-    const bool flat = a.ny == 1;
-    const size_t cells = (size_t)a.nx * a.ny;
-    if (allow_split && flat && a.nx <= 8192) {
-        // short tubes: four threads per cell shorten the dependent chain of a stage (8.8
-        // against 10.0 us at 8192 cells, 16.3 against 10.7 us at 16384)
-        L.func = split_flat_func(with_base);
-        L.block = dim3(kSplitFlatThreads, 1, 1);
-        L.grid = dim3((unsigned)((4 * (size_t)a.nx + kSplitFlatThreads - 1) / kSplitFlatThreads), 1, 1);
-        return L;
+    const bool flat = a.ny == 1, rounded = flat && a.nx <= kRoundedTube;
+    auto pad = [&](unsigned t) { return ((size_t)a.nx + t - 1) / t * t; };
+    // While the grid leaves most of the SMs' threads idle, the time is the chain of one
+    // thread, and the cell is split over 16 threads or two; the lanes past a row's end count
+    // as cells.  us per stage with 16 threads per cell, two and one: 5.4 / 10.6 / 17.5 at
+    // 64^2, 16.5 / 19.8 / 23.0 at 160^2, 19.6 / 19.5 / 22.9 at 168^2, 21.7 / 20.0 / 23.4 at
+    // 192^2, 26.0 / 33.1 / 24.6 at 200^2; tubes of 4000 cells 4.3 / 7.0 / 12.2, of 22000
+    // 11.9 / 11.9 / 15.5, of 36000 17.3 / 15.0 / 16.1, of 40000 19.2 / 18.1 / 17.2; 3 x 4096
+    // cells 70 / 111 / 54, 33 x 700 26.3 / 29.9 / 23.0, 63 x 420 17.5 / 17.0 / 20.5.
+    int ways = 1;
+    if (allow_split && pad(32) * a.ny <= (size_t)sm_count * 180) ways = 16;
+    else if (allow_split && pad(64) * a.ny <= (size_t)sm_count * 255) ways = 2;
+    unsigned w = ways == 16 ? 32 : 64;
+    if (ways == 1) {
+        // the widest block whose padding past the row's end is least
+        w = kThreads;
+        for (unsigned t = kThreads / 2; t >= 32; t /= 2)
+            if (pad(t) < pad(w)) w = t;
     }
-    const unsigned xblocks = (unsigned)((a.nx + kThreads - 1) / kThreads);
-    // Row-marching kernel when runs of at least 8 rows still give two full waves of
-    // blocks; runs grow to 32 rows while at least 8 waves remain; on smaller grids runs of
-    // 4 or 2 rows if they give two waves.
-    const size_t wave = (size_t)sm_count * kMinBlocks;
-    int R = 8;
-    while (R < 32 && (size_t)xblocks * ((a.ny + 2 * R - 1) / (2 * R)) >= 8 * wave) R *= 2;
-    bool march = allow_march && !flat && a.ny >= 16 && (size_t)xblocks * ((a.ny + 7) / 8) >= 2 * wave;
-    for (int r = 4; allow_march && !march && !flat && a.ny >= 16 && r >= 2; r /= 2) {
-        if ((size_t)xblocks * ((a.ny + r - 1) / r) >= 2 * wave) {
-            march = true;
-            R = r;
-        }
-    }
-    L.func = with_base ? stage_func<true>(march, flat) : stage_func<false>(march, flat);
-    if (march) {
-        // the double-buffered x row buffer
-        L.smem = kMarchRowBytes;
-        if (cudaFuncSetAttribute(L.func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem) != cudaSuccess)
-            cudaGetLastError();   // the launch then reports the error
-        L.block = dim3(kThreads, 1, 1);
-        const unsigned yblocks = (unsigned)((a.ny + R - 1) / R);
-        L.grid = dim3(xblocks, yblocks < 65535 ? yblocks : 65535, 1);
-        return L;
-    }
-    // Small grids: narrower blocks so that more SMs share the cells.
-    int threads = kThreads;
-    while (threads > 32 && cells < (size_t)sm_count * threads * 2) threads >>= 1;
-    L.block = dim3(threads, 1, 1);
-    L.grid = dim3((a.nx + threads - 1) / threads, a.ny < 65535 ? a.ny : 65535, 1);
+    const bool wide = a.nx >= (1 << 29);
+    L.func = with_base ? stage_func<true>(ways, flat, rounded, wide) : stage_func<false>(ways, flat, rounded, wide);
+    L.block = dim3(ways == 16 ? 512 : ways * w, 1, 1);
+    L.grid = dim3((unsigned)(pad(w) / w), a.ny < 65535 ? a.ny : 65535, 1);
     return L;
 }
 
