@@ -529,8 +529,9 @@ __global__ void __launch_bounds__(128) macros_kernel(const __grid_constant__ Fie
 
 // Powers of the group speed component c_g (v = (+-c_g, 0), (0, +-c_g) on the axis
 // groups, (+-c_g, +-c_g) on the diagonal ones) and of W_g = |v|^2 + eta_g^2, each set
-// relative to a power of two.
+// also in fixed point relative to a power of two.
 struct TneSet {
+    double v[4];
     FxK k[4];
     int e;
 };
@@ -542,19 +543,28 @@ TneSet tne_set(const double v[4])
 {
     TneSet t;
     t.e = fx_exponent(v, 4);
-    for (int g = 0; g < 4; ++g) t.k[g] = fx_k(fx_const(std::ldexp(v[g], -t.e), 60));
+    for (int g = 0; g < 4; ++g) {
+        t.v[g] = v[g];
+        t.k[g] = fx_k(fx_const(std::ldexp(v[g], -t.e), 60));
+    }
     return t;
 }
 
-__device__ __forceinline__ bool fx_out_of_range(int E) { return (unsigned)(E - kExpLo) >= (unsigned)kExpSpan; }
-
-// Group sums of the fixed-point members E N W S or NE NW SW SE of group g.
-__device__ __forceinline__ void fx_group_sums(int g, const int64_t q[4], int64_t &s0, int64_t &sx, int64_t &sy)
+// Whether the fixed-point dot products with a set are no less exact than the FP64 ones
+// whatever the cell holds.  Relative to the largest value f and constant k of the sum,
+// each of the 16 fixed-point products is off by at most 2^-59 f k (a value below 2^-6 f is
+// rounded at 2^-59 f; one above is exact, and its constant off by 2^-60 of a power of two
+// below 2 k); the FP64 sum rounds its terms up to six times, 6 x 2^-53 k_min f at least.
+// So k <= 24 k_min, less a little.  (Of the velocity sets in use, the sound wave's; the
+// vortex' and the tubes' W c^2 spread further.)
+bool tne_fixed(const TneSet &t)
 {
-    s0 = (q[0] + q[2]) + (q[1] + q[3]);
-    const int64_t d = q[0] - q[2], b = q[1] - q[3];
-    sx = (g & 1) == 0 ? d : d - b;
-    sy = (g & 1) == 0 ? b : d + b;
+    double lo = t.v[0], hi = t.v[0];
+    for (int g = 1; g < 4; ++g) {
+        lo = t.v[g] < lo ? t.v[g] : lo;
+        hi = t.v[g] > hi ? t.v[g] : hi;
+    }
+    return hi <= 23.0 * lo;
 }
 
 // The raw moments of a cell up to the fourth order (rows of Eq. 6 at u = 0).
@@ -562,31 +572,116 @@ struct RawMoments {
     double rho, jx, jy, E, Rxx, Ryy, Rxy, Rwx, Rwy, Rxxx, Ryyy, Rxxy, Rxyy, Rwxx, Rwyy, Rwxy;
 };
 
-// ... in FP64, for cells outside the integer path.
+// ... with the dot products in FP64.
 template <typename TS>
-__device__ __noinline__ RawMoments raw_moments_any(const FieldArgs &a, const TS *own, size_t P)
+__device__ __forceinline__ RawMoments raw_moments(const TneConsts &t, const TS f[kNV])
 {
-    RawMoments r = {};
-    for (int i = 0; i < kNV; ++i) {
-        const double v = stored(own[i * P]), x = a.vx[i], y = a.vy[i], w = a.m.w[i >> 2];
-        r.rho += v;
-        r.jx = fma(x, v, r.jx);
-        r.jy = fma(y, v, r.jy);
-        r.E = fma(w, v, r.E);
-        r.Rxx = fma(x * x, v, r.Rxx);
-        r.Ryy = fma(y * y, v, r.Ryy);
-        r.Rxy = fma(x * y, v, r.Rxy);
-        r.Rwx = fma(w * x, v, r.Rwx);
-        r.Rwy = fma(w * y, v, r.Rwy);
-        r.Rxxx = fma(x * x * x, v, r.Rxxx);
-        r.Ryyy = fma(y * y * y, v, r.Ryyy);
-        r.Rxxy = fma(x * x * y, v, r.Rxxy);
-        r.Rxyy = fma(x * y * y, v, r.Rxyy);
-        r.Rwxx = fma(w * x * x, v, r.Rwxx);
-        r.Rwyy = fma(w * y * y, v, r.Rwyy);
-        r.Rwxy = fma(w * x * y, v, r.Rwxy);
+    double s0[4], sx[4], sy[4], ex[2], ey[2], sxy[2];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        const GroupSums s = ex_group_sums(g & 1, f + 4 * g);
+        s0[g] = s.s0;
+        sx[g] = s.sx;
+        sy[g] = s.sy;
+        if ((g & 1) == 0) {
+            ex[g >> 1] = s.a;
+            ey[g >> 1] = s.b;
+        } else {
+            sxy[g >> 1] = s.a;
+        }
     }
-    return r;
+    auto dot = [](const TneSet &k, double x0, double x1, double x2, double x3) {
+        return fma(k.v[3], x3, fma(k.v[2], x2, fma(k.v[1], x1, k.v[0] * x0)));
+    };
+    auto dot2 = [](const TneSet &k, double x1, double x3) { return fma(k.v[3], x3, k.v[1] * x1); };
+    RawMoments m;
+    m.rho = (s0[0] + s0[1]) + (s0[2] + s0[3]);
+    m.jx = dot(t.c, sx[0], sx[1], sx[2], sx[3]);
+    m.jy = dot(t.c, sy[0], sy[1], sy[2], sy[3]);
+    m.E = dot(t.W, s0[0], s0[1], s0[2], s0[3]);
+    m.Rxx = dot(t.c2, ex[0], s0[1], ex[1], s0[3]);
+    m.Ryy = dot(t.c2, ey[0], s0[1], ey[1], s0[3]);
+    m.Rxy = dot2(t.c2, sxy[0], sxy[1]);
+    m.Rwx = dot(t.Wc, sx[0], sx[1], sx[2], sx[3]);
+    m.Rwy = dot(t.Wc, sy[0], sy[1], sy[2], sy[3]);
+    m.Rxxx = dot(t.c3, sx[0], sx[1], sx[2], sx[3]);
+    m.Ryyy = dot(t.c3, sy[0], sy[1], sy[2], sy[3]);
+    m.Rxxy = dot2(t.c3, sy[1], sy[3]);
+    m.Rxyy = dot2(t.c3, sx[1], sx[3]);
+    m.Rwxx = dot(t.Wc2, ex[0], s0[1], ex[1], s0[3]);
+    m.Rwyy = dot(t.Wc2, ey[0], s0[1], ey[1], s0[3]);
+    m.Rwxy = dot2(t.Wc2, sxy[0], sxy[1]);
+    return m;
+}
+
+// ... of a cell outside the fixed-point path.
+template <typename TS>
+__device__ __noinline__ RawMoments raw_moments_any(const TneConsts &t, const TS *own, size_t P)
+{
+    TS f[kNV];
+    for (int i = 0; i < kNV; ++i) f[i] = own[i * P];
+    return raw_moments(t, f);
+}
+
+// ... in fixed point: exact sums, each dot product with constants rounded once.  ok: in range.
+template <typename TS>
+__device__ __forceinline__ RawMoments raw_moments_fixed(const TneConsts &t, const TS f[kNV], bool &ok)
+{
+    uint32_t key = 0;
+#pragma unroll
+    for (int i = 0; i < kNV; ++i) key = fx_max(key, fx_key(f[i]));
+    const int field = (int)(key >> (kSingle<TS> ? 24 : 21));
+    const int top = kSingle<TS> ? field + (1023 - 127) : field;
+    ok = kSingle<TS> ? field < 255 : (unsigned)(field - kExpLo) < (unsigned)kExpSpan;
+    int64_t s0[4], sx[4], sy[4], ex[2], ey[2], sxy[2];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        int64_t q[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) q[j] = fx_from(f[4 * g + j], field);
+        const int64_t d = q[0] - q[2], b = q[1] - q[3], x = q[0] + q[2], y = q[1] + q[3];
+        s0[g] = x + y;
+        sx[g] = (g & 1) == 0 ? d : d - b;
+        sy[g] = (g & 1) == 0 ? b : d + b;
+        if ((g & 1) == 0) {
+            ex[g >> 1] = x;
+            ey[g >> 1] = y;
+        } else {
+            sxy[g >> 1] = x - y;
+        }
+    }
+    auto dot = [&](const TneSet &k, int64_t x0, int64_t x1, int64_t x2, int64_t x3) {
+        FxSum m = kFxHalfUnit;
+        fx_mul(m, x0, k.k[0]);
+        fx_mul(m, x1, k.k[1]);
+        fx_mul(m, x2, k.k[2]);
+        fx_mul(m, x3, k.k[3]);
+        return fx_to(fx_sum59(m), top + k.e);
+    };
+    auto dot2 = [&](const TneSet &k, int64_t x1, int64_t x3) {      // the diagonal groups
+        FxSum m = kFxHalfUnit;
+        fx_mul(m, x1, k.k[1]);
+        fx_mul(m, x3, k.k[3]);
+        return fx_to(fx_sum59(m), top + k.e);
+    };
+    RawMoments m;
+    m.rho = fx_to((s0[0] + s0[1]) + (s0[2] + s0[3]), top);
+    m.jx = dot(t.c, sx[0], sx[1], sx[2], sx[3]);
+    m.jy = dot(t.c, sy[0], sy[1], sy[2], sy[3]);
+    m.E = dot(t.W, s0[0], s0[1], s0[2], s0[3]);
+    m.Rxx = dot(t.c2, ex[0], s0[1], ex[1], s0[3]);
+    m.Ryy = dot(t.c2, ey[0], s0[1], ey[1], s0[3]);
+    m.Rxy = dot2(t.c2, sxy[0], sxy[1]);
+    m.Rwx = dot(t.Wc, sx[0], sx[1], sx[2], sx[3]);
+    m.Rwy = dot(t.Wc, sy[0], sy[1], sy[2], sy[3]);
+    m.Rxxx = dot(t.c3, sx[0], sx[1], sx[2], sx[3]);
+    m.Ryyy = dot(t.c3, sy[0], sy[1], sy[2], sy[3]);
+    m.Rxxy = dot2(t.c3, sy[1], sy[3]);
+    m.Rxyy = dot2(t.c3, sx[1], sx[3]);
+    m.Rwxx = dot(t.Wc2, ex[0], s0[1], ex[1], s0[3]);
+    m.Rwyy = dot(t.Wc2, ey[0], s0[1], ey[1], s0[3]);
+    m.Rwxy = dot2(t.Wc2, sxy[0], sxy[1]);
+    return m;
 }
 
 // Rows 5..16 of M(u) (Eq. 6) applied to f - f_eq: Delta* of Eqs. (8)-(11).  f_eq is
@@ -596,75 +691,26 @@ __device__ __noinline__ RawMoments raw_moments_any(const FieldArgs &a, const TS 
 // fourth).  The central moments follow from the raw moments R_k = sum_i f_i row_k(v_i)
 // by the binomial expansion of (v - u) with j = rho u; the raw moments of a group
 // come from its members' sum, x and y differences, the x and y pair sums (axis
-// groups) and the xy parity (diagonal groups).  The raw moments are formed in fixed
-// point (exact sums, each dot product with constants rounded once), which leaves 88 of
-// 167 FP64 instructions: 5.14 -> 2.46 ms for 4096^2 cells.
-template <typename TS>
+// groups) and the xy parity (diagonal groups).  kFixed: the raw moments in fixed
+// point, which leaves 88 of 167 FP64 instructions: 2.46 ms for 4096^2 cells, against 4.24
+// with FP64 dot products of integer group sums (5.14 with all on the FP64 pipe).
+template <typename TS, bool kFixed>
 __global__ void __launch_bounds__(128) tne_kernel(const __grid_constant__ FieldArgs a, const __grid_constant__ TneConsts t,
                                                   const RefMoments F, const TS *__restrict__ f, double *__restrict__ out)
 {
     const size_t P = (size_t)a.nx * a.ny;
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < P;
          c += (size_t)gridDim.x * blockDim.x) {
-        const TS *own = f + c;
         TS fc[kNV];
-        uint32_t key = 0;
 #pragma unroll
-        for (int i = 0; i < kNV; ++i) fc[i] = __ldg(own + i * P);
-#pragma unroll
-        for (int i = 0; i < kNV; ++i) key = fx_max(key, fx_key(fc[i]));
-        const int field = (int)(key >> (kSingle<TS> ? 24 : 21));
-        const int top = kSingle<TS> ? field + (1023 - 127) : field;
-        // group components: s0 sum, sx / sy odd in x / y, ex / ey the x / y pairs
-        // (axis), sxy odd in x and y (diagonal)
-        int64_t s0[4], sx[4], sy[4], ex[2], ey[2], sxy[2];
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            int64_t q[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) q[j] = fx_from(fc[4 * g + j], field);
-            fx_group_sums(g, q, s0[g], sx[g], sy[g]);
-            if ((g & 1) == 0) {
-                ex[g >> 1] = q[0] + q[2];
-                ey[g >> 1] = q[1] + q[3];
-            } else {
-                sxy[g >> 1] = (q[0] + q[2]) - (q[1] + q[3]);
-            }
-        }
-        auto dot4 = [&](const TneSet &k, int64_t x0, int64_t x1, int64_t x2, int64_t x3) {
-            FxSum m = kFxHalfUnit;
-            fx_mul(m, x0, k.k[0]);
-            fx_mul(m, x1, k.k[1]);
-            fx_mul(m, x2, k.k[2]);
-            fx_mul(m, x3, k.k[3]);
-            return fx_to(fx_sum59(m), top + k.e);
-        };
-        auto dot2 = [&](const TneSet &k, int64_t x1, int64_t x3) {      // the diagonal groups
-            FxSum m = kFxHalfUnit;
-            fx_mul(m, x1, k.k[1]);
-            fx_mul(m, x3, k.k[3]);
-            return fx_to(fx_sum59(m), top + k.e);
-        };
+        for (int i = 0; i < kNV; ++i) fc[i] = __ldg(f + i * P + c);
         RawMoments m;
-        if (!(kSingle<TS> ? field == 255 : fx_out_of_range(field))) {
-            m.rho = fx_to((s0[0] + s0[1]) + (s0[2] + s0[3]), top);
-            m.jx = dot4(t.c, sx[0], sx[1], sx[2], sx[3]);
-            m.jy = dot4(t.c, sy[0], sy[1], sy[2], sy[3]);
-            m.E = dot4(t.W, s0[0], s0[1], s0[2], s0[3]);
-            m.Rxx = dot4(t.c2, ex[0], s0[1], ex[1], s0[3]);
-            m.Ryy = dot4(t.c2, ey[0], s0[1], ey[1], s0[3]);
-            m.Rxy = dot2(t.c2, sxy[0], sxy[1]);
-            m.Rwx = dot4(t.Wc, sx[0], sx[1], sx[2], sx[3]);
-            m.Rwy = dot4(t.Wc, sy[0], sy[1], sy[2], sy[3]);
-            m.Rxxx = dot4(t.c3, sx[0], sx[1], sx[2], sx[3]);
-            m.Ryyy = dot4(t.c3, sy[0], sy[1], sy[2], sy[3]);
-            m.Rxxy = dot2(t.c3, sy[1], sy[3]);
-            m.Rxyy = dot2(t.c3, sx[1], sx[3]);
-            m.Rwxx = dot4(t.Wc2, ex[0], s0[1], ex[1], s0[3]);
-            m.Rwyy = dot4(t.Wc2, ey[0], s0[1], ey[1], s0[3]);
-            m.Rwxy = dot2(t.Wc2, sxy[0], sxy[1]);
+        if constexpr (kFixed) {
+            bool ok;
+            m = raw_moments_fixed(t, fc, ok);
+            if (!ok) m = raw_moments_any(t, f + c, P);
         } else {
-            m = raw_moments_any(a, own, P);
+            m = raw_moments(t, fc);
         }
         if constexpr (kSingle<TS>) {    // the reference equilibrium's even moments
             m.rho += F.rho;
@@ -906,10 +952,15 @@ cudaError_t launch_tne(const FieldArgs &a, const void *f, int prec, double *out,
     const TneConsts t = {tne_set(a.m.c), tne_set(c2), tne_set(c3), tne_set(a.m.w), tne_set(wc), tne_set(wc2)};
     const unsigned nb = grid_for((size_t)a.nx * a.ny, 128);
     const RefMoments F = ref_moments(a, single_storage(prec));
-    if (single_storage(prec))
-        tne_kernel<float><<<nb, 128, 0, s>>>(a, t, F, (const float *)f, out);
-    else
-        tne_kernel<double><<<nb, 128, 0, s>>>(a, t, F, (const double *)f, out);
+    const bool fixed = tne_fixed(t.c) && tne_fixed(t.c2) && tne_fixed(t.c3) && tne_fixed(t.W) && tne_fixed(t.Wc) &&
+                       tne_fixed(t.Wc2);
+    if (single_storage(prec)) {
+        auto k = fixed ? tne_kernel<float, true> : tne_kernel<float, false>;
+        k<<<nb, 128, 0, s>>>(a, t, F, (const float *)f, out);
+    } else {
+        auto k = fixed ? tne_kernel<double, true> : tne_kernel<double, false>;
+        k<<<nb, 128, 0, s>>>(a, t, F, (const double *)f, out);
+    }
     return cudaGetLastError();
 }
 
