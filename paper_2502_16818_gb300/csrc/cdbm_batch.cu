@@ -521,6 +521,19 @@ bool is_device_ptr(const void *p)
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Work of stream s from here on runs after all work already queued on the legacy default
+// stream and on the streams that synchronise with it.
+cudaError_t wait_for_default_stream(cudaStream_t s)
+{
+    cudaEvent_t e;
+    cudaError_t r = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
+    if (r != cudaSuccess) return r;
+    r = cudaEventRecord(e, cudaStreamLegacy);
+    if (r == cudaSuccess) r = cudaStreamWaitEvent(s, e, 0);
+    cudaEventDestroy(e);
+    return r;
+}
+
 void drop_batch_graph(cdbm_batch *b)
 {
     if (b->graph) {
@@ -769,6 +782,9 @@ cdbm_status cdbm_batch_init(cdbm_batch *b, const double *rho, const double *ux, 
     const double *dev[4];
     // the second buffer (16 planes of the storage type) stages host fields: 4 double planes fit
     double *stage = (double *)b->f1;
+    bool any_dev = false;
+    for (int k = 0; k < 4; ++k) any_dev |= is_device_ptr(src[k]);
+    if (any_dev && bcuda(b, wait_for_default_stream(b->stream), "batch fields wait")) return b->err;
     for (int k = 0; k < 4; ++k) {
         if (is_device_ptr(src[k])) {
             dev[k] = src[k];
