@@ -111,11 +111,11 @@ __device__ __forceinline__ void tube_stage(const float *g, const float *base, fl
         } else {
             double f[kNV];
 #pragma unroll
-            for (int i = 0; i < kNV; ++i) f[i] = widen(fs[i]);
+            for (int i = 0; i < kNV; ++i) f[i] = widen_f32(fs[i]);
             double h[kNV];
             if constexpr (kSym) {
-                const Prim s = primitives_sym<true>(f, C.m, t.rhoF, t.EF, flag);
-                equilibrium_sym<true>(C.eq[kStage], C.m, s.q.rho, s.q.E, s.q.jx, s.ux, s.ru2, s.p, s.T, h,
+                const Prim s = primitives_sym(f, C.m, t.rhoF, t.EF, flag);
+                equilibrium_sym(C.eq[kStage], C.m, s.q.rho, s.q.E, s.q.jx, s.ux, s.ru2, s.p, s.T, h,
                                              t.sF[kStage]);
             } else {
                 const Prim s = primitives<true>(f, C.m, t.rhoF, t.EF, flag);
@@ -123,7 +123,7 @@ __device__ __forceinline__ void tube_stage(const float *g, const float *base, fl
                                          s.jyuy, s.p, s.T, h, t.sF[kStage]);
             }
 #pragma unroll
-            for (int i = 0; i < kNV; ++i) heq[i] = narrow<float>(h[i]);
+            for (int i = 0; i < kNV; ++i) heq[i] = narrow_f64(h[i]);
         }
 #pragma unroll
         for (int i = 0; i < kNV; ++i) {

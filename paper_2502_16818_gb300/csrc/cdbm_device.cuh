@@ -228,19 +228,6 @@ __device__ __forceinline__ void equilibrium_of(const EqBlocks &B, const ModelCon
 template <typename TS>
 constexpr bool kSingle = std::is_same<TS, float>::value;
 
-__device__ __forceinline__ double fma_t(double x, double y, double z) { return fma(x, y, z); }
-
-// Storage value to double and double to storage value; the single-precision
-// conversions run on the integer pipes (cdbm_convert.h).
-__device__ __forceinline__ double widen(double v) { return v; }
-__device__ __forceinline__ double widen(float v) { return widen_f32(v); }
-template <typename TS>
-__device__ __forceinline__ TS narrow(double v)
-{
-    if constexpr (kSingle<TS>) return narrow_f64(v); else return v;
-}
-__device__ __forceinline__ float fma_t(float x, float y, float z) { return fmaf(x, y, z); }
-
 // Per-cell macroscopic quantities of a stage: conserved moments (in double), then
 // u, P = rho T and T through the refined reciprocal of rho.  With kShift, f holds
 // g = f - F and the reference moments rhoF, EF are added.
@@ -383,17 +370,14 @@ __device__ __forceinline__ Cons conserved_sym(const double f[kNV], const ModelCo
     return r;
 }
 
-// primitives<kShift>() on a symmetric state (u_y = 0, rho u^2 = j_x u_x).
-template <bool kShift>
+// primitives<true>() on a symmetric state (u_y = 0, rho u^2 = j_x u_x).
 __device__ __forceinline__ Prim primitives_sym(const double f[kNV], const ModelConsts &m, double rhoF, double EF,
                                                unsigned *flag)
 {
     Prim s;
     s.q = conserved_sym(f, m);
-    if (kShift) {
-        s.q.rho += rhoF;
-        s.q.E += EF;
-    }
+    s.q.rho += rhoF;
+    s.q.E += EF;
     const double r = rcp64(s.q.rho);
     s.r = r;
     s.ux = s.q.jx * r;
@@ -406,13 +390,12 @@ __device__ __forceinline__ Prim primitives_sym(const double f[kNV], const ModelC
     return s;
 }
 
-// equilibrium<kShift>() on a symmetric state: u_y = j_y = 0, so rho u^2 = m5 - m7 =
+// equilibrium<true>() on a symmetric state: u_y = j_y = 0, so rho u^2 = m5 - m7 =
 // j_x u_x, m6 = m15 = 0 (no diagonal quadrupole), u^2 = u_x^2 - u_y^2 = u_x^2, and
 // the y-odd members equal their mirror images.  out receives all 16 values.
-template <bool kShift = false>
 __device__ __forceinline__ void equilibrium_sym(const EqBlocks &B, const ModelConsts &m, double rho, double E,
                                                 double jx, double ux, double ru2, double P, double T,
-                                                double out[kNV], const double *s0_shift = nullptr)
+                                                double out[kNV], const double *s0_shift)
 {
     const double u2 = ux * ux;
     const double m1416 = fma(T, fma(m.Kp6, ru2, m.twoKp2 * P), ru2 * u2);
@@ -422,10 +405,7 @@ __device__ __forceinline__ void equilibrium_sym(const EqBlocks &B, const ModelCo
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
         const double *S = B.S + 4 * g;
-        if (kShift)
-            s0[g] = fma(S[3], m1416, fma(S[2], ru2, fma(S[1], E, fma(S[0], rho, -s0_shift[g]))));
-        else
-            s0[g] = fma(S[3], m1416, fma(S[2], ru2, fma(S[1], E, S[0] * rho)));
+        s0[g] = fma(S[3], m1416, fma(S[2], ru2, fma(S[1], E, fma(S[0], rho, -s0_shift[g]))));
     }
     const double dq[2] = {d57 * fma(B.B1[1], W4, B.B1[0]), d57 * fma(B.B1[3], W4, B.B1[2])};
 #pragma unroll

@@ -1,9 +1,8 @@
-// 64-bit block fixed-point arithmetic for the double-precision stage.
+// 64-bit block fixed-point arithmetic for sums that need not round as FP64 does: the raw
+// moments of Delta* and the group sums of single-precision values.
 //
 // On GB300 one FP64 instruction occupies its pipe for 64 cycles per SM sub-partition
-// (2 lanes/clk/SM, measured), a 32-bit integer instruction for 1 to 2.  The stage's
-// sums, differences and products by constants of the run (conserved moments, NND
-// transport, Runge-Kutta update) therefore run on the integer pipes: the doubles of a
+// (2 lanes/clk/SM, measured), a 32-bit integer instruction for 1 to 2.  So the doubles of a
 // sum are brought to the largest exponent among them as 64-bit integers, added and
 // multiplied exactly or to a few units of 2^-58 of that largest value, and the result
 // is rounded to double once.  The FP64 form rounds after every operation, at 2^-53 of
@@ -115,10 +114,71 @@ CDBM_FX_HD double fx_to(int64_t v, int E)
     return fx_bits(hi | ((uint32_t)(s >> 32) & 0x80000000u), (uint32_t)q);
 }
 
-// A constant of the run as hi 2^32 + lo (lo signed), in units of 2^-61 or 2^-60.
+// A constant of the run as hi 2^32 + lo (lo signed).
 struct FxC {
     int32_t hi, lo;
 };
+
+// A constant of the run as b1 2^30 + b0 in units of 2^-59; b0x4 = 4 b0.
+struct FxK {
+    int32_t b1, b0, b0x4;
+};
+
+// Sum of products x b, all four partial products kept.  No partial sum overflows for the
+// moments: the four |x| add up to less than 2^63, |b| <= 1 in 2^-59.
+struct FxSum {
+    int64_t r, mid, low;
+};
+CDBM_FX_HD void fx_mul(FxSum &a, int64_t x, FxK b)
+{
+    const int32_t x0 = (int32_t)x;
+    const int32_t x1 = (int32_t)(x >> 32) + (int32_t)((uint32_t)x0 >> 31);
+    a.r += (int64_t)x1 * b.b1;
+    a.mid += (int64_t)x1 * b.b0x4;
+    a.mid += (int64_t)x0 * b.b1;
+    a.low += (int64_t)x0 * b.b0;
+}
+// The sum in the units of x, rounded to nearest, for constants in units of 2^-59, of an
+// FxSum that starts from kFxHalfUnit.
+constexpr FxSum kFxHalfUnit = {0, 1 << 28, 0};
+CDBM_FX_HD int64_t fx_sum59(const FxSum &a)
+{
+    return (int64_t)((uint64_t)a.r << 3) + ((a.mid + (a.low >> 30)) >> 29);
+}
+inline FxC fx_split(int64_t b)
+{
+    FxC c;
+    c.lo = (int32_t)(uint32_t)b;
+    c.hi = (int32_t)((b >> 32) + (c.lo < 0));
+    return c;
+}
+inline int64_t fx_int(FxC c) { return ((int64_t)c.hi << 32) + c.lo; }
+// v 2^bits (|v| <= 2) as a constant.
+inline FxC fx_const(double v, int bits) { return fx_split(std::llrint(std::ldexp(v, bits))); }
+
+inline FxK fx_k(FxC a)
+{
+    const int64_t b = fx_int(a) / 2;                           // in twice the unit of a
+    FxK k;
+    k.b1 = (int32_t)((b + (1 << 29)) >> 30);
+    k.b0 = (int32_t)(b - ((int64_t)k.b1 << 30));
+    k.b0x4 = 4 * k.b0;
+    return k;
+}
+
+// Exponent of the smallest power of two that is at least the largest of v[0..n-1].
+inline int fx_exponent(const double *v, int n)
+{
+    double m = 0.0;
+    for (int k = 0; k < n; ++k) m = v[k] > m ? v[k] : m;
+    int e = 0;
+    const double f = std::frexp(m, &e);
+    return f == 0.5 ? e - 1 : e;
+}
+
+// ---- The update of a Runge-Kutta stage ----
+// No kernel takes it: it is about as exact as FP64 arithmetic but rounds otherwise, and the
+// time step amplifies that (cdbm_exact.h).  Kept under its host check.
 
 // Sum of products x b: r holds the high parts, mid the cross terms and the rounded high
 // word of the products of the two low halves.
@@ -149,7 +209,8 @@ CDBM_FX_HD int64_t fx_max64(int64_t a, int64_t b) { return a > b ? a : b; }
 // e = u1 - u2.  minmod(b, a) is b clamped to the interval between 0 and a.
 CDBM_FX_HD int64_t fx_nnd2(int64_t u2, int64_t u1, int64_t c, int64_t d1)
 {
-    const int64_t a = c - u1, b = d1 - c, e = u1 - u2;
+    const int64_t a = (int64_t)((uint64_t)c - (uint64_t)u1), b = (int64_t)((uint64_t)d1 - (uint64_t)c),
+                  e = (int64_t)((uint64_t)u1 - (uint64_t)u2);
     const int64_t s = a >> 63;
     const int64_t lo = a & s, hi = a & ~s;
     return a + a + fx_max64(fx_min64(b, hi), lo) - fx_max64(fx_min64(e, hi), lo);
@@ -159,30 +220,9 @@ CDBM_FX_HD int64_t fx_nnd2(int64_t u2, int64_t u1, int64_t c, int64_t d1)
 // these are the differences of the magnitudes in units in the last place.
 CDBM_FX_HD int64_t fx_raw(double v) { return (int64_t)((uint64_t)f64_hi(v) << 32 | f64_lo(v)); }
 
-// A constant of the run as b1 2^30 + b0 in units of 2^-59; b0x4 = 4 b0.
-struct FxK {
-    int32_t b1, b0, b0x4;
-};
-
-// Sum of products x b, all four partial products kept.  No partial sum overflows for the
-// moments: the four |x| add up to less than 2^63, |b| <= 1 in 2^-59.
-struct FxSum {
-    int64_t r, mid, low;
-};
-CDBM_FX_HD void fx_mul(FxSum &a, int64_t x, FxK b)
-{
-    const int32_t x0 = (int32_t)x;
-    const int32_t x1 = (int32_t)(x >> 32) + (int32_t)((uint32_t)x0 >> 31);
-    a.r += (int64_t)x1 * b.b1;
-    a.mid += (int64_t)x1 * b.b0x4;
-    a.mid += (int64_t)x0 * b.b1;
-    a.low += (int64_t)x0 * b.b0;
-}
-// The same with a constant as hi 2^32 + lo: the sum is r 2^64 + mid 2^32 + low, so that the
-// shift by 64 that the scale of the operands is chosen for below costs nothing (in units of
-// 2^-60 it took about ten instructions more per velocity: 0.99 against 0.96 ms per step of
-// 1500 x 1300 cells).  Two products
-// at most, lo of one of the constants above -2^31.
+// fx_mul() with a constant as hi 2^32 + lo: the sum is r 2^64 + mid 2^32 + low, so that the
+// shift by 64 that the scale of the operands is chosen for below costs nothing.  Two products at most, lo of
+// one of the constants above -2^31.
 CDBM_FX_HD void fx_mul(FxSum &a, int64_t x, FxC b)
 {
     const int32_t x0 = (int32_t)x;
@@ -198,13 +238,6 @@ CDBM_FX_HD void fx_mul(FxSum &a, int64_t x, FxC b)
 constexpr int kFxUp = 9;
 constexpr FxSum kFxHalf = {0, (int64_t)1 << 31, 0};
 CDBM_FX_HD int64_t fx_sum64ths(const FxSum &a) { return a.r + ((a.mid + (a.low >> 32)) >> 32); }
-// The sum in the units of x, rounded to nearest, for constants in units of 2^-59, of an
-// FxSum that starts from kFxHalfUnit.
-constexpr FxSum kFxHalfUnit = {0, 1 << 28, 0};
-CDBM_FX_HD int64_t fx_sum59(const FxSum &a)
-{
-    return (int64_t)((uint64_t)a.r << 3) + ((a.mid + (a.low >> 30)) >> 29);
-}
 // 64ths rounded to the nearest unit so that C plus the result is even on a tie.
 CDBM_FX_HD int64_t fx_round64ths(int64_t t, int64_t C) { return (t + 31 + (((t >> 6) ^ C) & 1)) >> 6; }
 // The sum rounded to the nearest unit of x, a tie toward zero, for constants in units of
@@ -217,42 +250,6 @@ CDBM_FX_HD int64_t fx_sum_units(const FxSum &a)
     return v + (int64_t)(((uint64_t)(uint32_t)m + tie) >> 32);
 }
 
-inline FxC fx_split(int64_t b)
-{
-    FxC c;
-    c.lo = (int32_t)(uint32_t)b;
-    c.hi = (int32_t)((b >> 32) + (c.lo < 0));
-    return c;
-}
-inline int64_t fx_int(FxC c) { return ((int64_t)c.hi << 32) + c.lo; }
-// v 2^bits (|v| <= 2) as a constant of fx_mac.
-inline FxC fx_const(double v, int bits) { return fx_split(std::llrint(std::ldexp(v, bits))); }
-
-inline FxK fx_k(FxC a)
-{
-    const int64_t b = fx_int(a) / 2;                           // in twice the unit of a
-    FxK k;
-    k.b1 = (int32_t)((b + (1 << 29)) >> 30);
-    k.b0 = (int32_t)(b - ((int64_t)k.b1 << 30));
-    k.b0x4 = 4 * k.b0;
-    return k;
-}
-
-// Exponent of the smallest power of two that is at least the largest of v[0..n-1].
-inline int fx_exponent(const double *v, int n)
-{
-    double m = 0.0;
-    for (int k = 0; k < n; ++k) m = v[k] > m ? v[k] : m;
-    int e = 0;
-    const double f = std::frexp(m, &e);
-    return f == 0.5 ? e - 1 : e;
-}
-
-// Group speeds and energies relative to a power of two.
-struct FxModel {
-    FxK c[4], w[4];
-    int cexp, wexp;
-};
 // Stage coefficients, out = base base + self g + heq - sum l D, times 2^61; for operands of
 // one exponent self + base - 1 = -gamma h.
 struct FxCoef {
@@ -265,17 +262,6 @@ struct FxFlux {
     FxC klx[4], kly[4];
 };
 
-inline FxModel fx_model(const double c[4], const double w[4])
-{
-    FxModel m;
-    m.cexp = fx_exponent(c, 4);
-    m.wexp = fx_exponent(w, 4);
-    for (int g = 0; g < 4; ++g) {
-        m.c[g] = fx_k(fx_const(std::ldexp(c[g], -m.cexp), 60));   // 2^-59
-        m.w[g] = fx_k(fx_const(std::ldexp(w[g], -m.wexp), 60));
-    }
-    return m;
-}
 inline FxCoef fx_coef(double self, double base)
 {
     FxCoef k;
@@ -307,11 +293,5 @@ inline FxFlux fx_flux(const double lx[4], const double ly[4], bool along_x, bool
     }
     return f;
 }
-
-struct FxStage {
-    FxModel m;
-    FxCoef k;
-    FxFlux l;
-};
 
 }  // namespace cdbm

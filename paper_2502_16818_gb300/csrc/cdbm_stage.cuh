@@ -24,12 +24,12 @@ __device__ __forceinline__ void stage_equilibrium(const StageArgs &a, const floa
     } else {
         double f[kNV];
 #pragma unroll
-        for (int i = 0; i < kNV; ++i) f[i] = widen(fs[i]);
+        for (int i = 0; i < kNV; ++i) f[i] = widen_f32(fs[i]);
         const Prim s = primitives<true>(f, a.m, a.rhoF, a.EF, flag);
         double h[kNV];
         equilibrium<true>(a.eq, a.m, s.q.rho, s.q.E, s.q.jx, s.q.jy, s.ux, s.uy, s.ru2, s.jyuy, s.p, s.T, h, a.sF);
 #pragma unroll
-        for (int i = 0; i < kNV; ++i) heq[i] = narrow<float>(h[i]);
+        for (int i = 0; i < kNV; ++i) heq[i] = narrow_f64(h[i]);
     }
 }
 

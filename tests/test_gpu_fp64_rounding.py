@@ -118,3 +118,27 @@ def test_batch_has_the_bits_of_single_tubes():
                 assert np.array_equal(x, y.cpu().numpy()[0]), (uy, k)
             s.close()
         b.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(131, 67), (500, 1), (3001, 1), (226, 220)])
+def test_adjoint_is_the_same_from_every_form(nx, ny):
+    """The recorded run is cdbm_step's, and its recomputed segments have its bits whatever
+    form takes them: ragged grids, tubes in the cluster and beyond."""
+    from paper_2502_16818_gb300 import Solver, cdbm
+    w = blocks(nx, ny, (0, 0))
+    got = []
+    for small in (1, 0):
+        s = Solver.from_workload(w)
+        cdbm.cdbm_set_small_grid_path(s.ctx, small)
+        s.init(w.rho, w.ux, w.uy, w.T)
+        s.step(7)
+        plain = s.state().clone()
+        s.init(w.rho, w.ux, w.uy, w.T)
+        cdbm.cdbm_adjoint_forward(s.ctx, 7, 3)
+        assert torch.equal(s.state(), plain)
+        fbar = torch.ones((16, ny, nx), dtype=torch.float64, device="cuda") * 0.25
+        grads = [torch.empty((ny, nx), dtype=torch.float64, device="cuda") for _ in range(4)]
+        tau = cdbm.cdbm_adjoint_backward(s.ctx, fbar.data_ptr(), *(g.data_ptr() for g in grads))
+        got.append((grads, tau))
+        s.close()
+    assert got[0][1] == got[1][1] and all(torch.equal(a, b) for a, b in zip(got[0][0], got[1][0]))
