@@ -10,6 +10,7 @@ uniform draws and constants alone (no libm), so they are the same on every host.
 
 The shapes reach every form of the stage: a cell on one, two and 16 threads, in the
 cluster, on 1-D and 2-D grids, with rows that are no multiple of a warp."""
+import ctypes
 import hashlib
 import os
 
@@ -142,3 +143,18 @@ def test_adjoint_is_the_same_from_every_form(nx, ny):
         got.append((grads, tau))
         s.close()
     assert got[0][1] == got[1][1] and all(torch.equal(a, b) for a, b in zip(got[0][0], got[1][0]))
+
+
+@pytest.mark.parametrize("nx,ny", [(37, 1), (500, 1), (3001, 1), (9001, 1), (131, 67)])
+def test_step_noalloc_has_the_bits_of_step(nx, ny):
+    from paper_2502_16818_gb300 import Solver, cdbm
+    w = blocks(nx, ny, (1, 0))
+    s = Solver.from_workload(w)
+    s.init(w.rho, w.ux, w.uy, w.T)
+    f = s.state().clone()
+    s.step(9)
+    grid = cdbm.cdbm_grid(w.nx, w.ny, w.dx, w.dy, w.bc_x, w.bc_y)
+    vset = cdbm.cdbm_vset((ctypes.c_double * 4)(*w.vg), (ctypes.c_double * 4)(*w.eg))
+    cdbm.cdbm_step_noalloc(grid, vset, w.I, w.tau, w.dt, f.data_ptr(), 9, torch.cuda.current_stream().cuda_stream)
+    assert torch.equal(f, s.state())
+    s.close()
