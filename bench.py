@@ -55,7 +55,7 @@ BYTES_PER_CELL_STEP_ADJ_BWD = 640 + 384 + 512
 # the stage kernels; valid only while the code of the kernel sources (comments
 # stripped) hashes to TRAFFIC_SHA.
 # Captured at 1024^2 (134 MB per plane set, above L2) and scaled by 16 cells-fold.
-TRAFFIC_SHA = "4ec522ff2ff730c8"
+TRAFFIC_SHA = "b7df2ade56823933"
 TRAFFIC_BYTES_PER_LAUNCH = 4.948e9
 
 

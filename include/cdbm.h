@@ -157,7 +157,8 @@ cdbm_status cdbm_init(cdbm_ctx *ctx, const double *rho, const double *ux, const 
  */
 cdbm_status cdbm_step(cdbm_ctx *ctx, int nsteps);
 
-/* Enables (default) or disables the small-grid paths of cdbm_step: on 1-D grids the
+/* Enables (default) or disables the small-grid paths of cdbm_step (and of the run that
+ * cdbm_adjoint_forward records, which takes cdbm_step's kernels): on 1-D grids the
  * persistent cluster kernel, and for CDBM_FP64 the stage kernels that split each cell
  * over 16 or two threads (grids of up to about 39000 cells).  Disabled, those grids step
  * with the one-cell-per-thread stage kernel like any other, with the same results bit
@@ -353,9 +354,7 @@ void cdbm_batch_destroy(cdbm_batch *b);
  *   f            : device pointer to the caller's state [16][ny][nx] (for example from
  *                  cdbm_get_state or an equilibrium the caller built), advanced in
  *                  place by nsteps >= 0 two-stage TVD Runge-Kutta steps.  The result
- *                  matches cdbm_step's on the same state to rounding (within 1e-12
- *                  relative max-norm): both apply the same per-cell operations.  On
- *                  2-D grids both run the same stage kernels and agree bit for bit.
+ *                  is cdbm_step's on the same state, bit for bit.
  *   cuda_stream  : stream for the work (NULL = legacy stream).
  * Scratch: the stage-1 buffer and the error flag live in one fixed device array of
  * the library (16 * CDBM_NOALLOC_MAX_CELLS doubles plus 256 bytes, i.e. 4 MiB), which
