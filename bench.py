@@ -658,8 +658,8 @@ def aux_kernels(s, w, stream, torch, cdbm, state_bytes, with_init, reps=10):
     32 B), Delta* (reads the planes, writes 12 doubles: 96 B; it rebuilds the
     central moments of every cell from its raw moments) and the conserved sums
     (reads the planes; a synchronous call that returns 4
-    doubles).  On the FP64 state Delta* takes some 135 FP64 instructions per cell for the
-    vortex' velocity set, macros 27 and the sums 22, near the FP64 pipe's rate.  state_bytes:
+    doubles).  On the FP64 state Delta* takes 138 FP64 instructions per cell for the
+    vortex' velocity set, macros 25 and the sums 22, near the FP64 pipe's rate.  state_bytes:
     bytes per stored value (8 for FP64, 4 for the single-precision states)."""
     cells = w.nx * w.ny
     planes = 16 * state_bytes

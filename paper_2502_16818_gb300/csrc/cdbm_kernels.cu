@@ -497,8 +497,8 @@ RefMoments ref_moments(const FieldArgs &a, bool single)
 __device__ __forceinline__ double stored(double v) { return v; }
 __device__ __forceinline__ double stored(float v) { return widen_f32(v); }
 
-// The conserved moments with the group sums on the integer pipes (cdbm_exact.h): 27 instead
-// of 51 FP64 instructions per cell.
+// The conserved moments with the group sums on the integer pipes (cdbm_exact.h): 25 instead
+// of 51 FP64 instructions per cell, 0.79 instead of 1.61 ms for 4096^2 cells.
 template <typename TS>
 __global__ void __launch_bounds__(128) macros_kernel(const __grid_constant__ FieldArgs a, const RefMoments F,
                                                      const TS *__restrict__ f, double *rho, double *ux, double *uy,

@@ -79,8 +79,8 @@ __device__ __forceinline__ void grid_group(const double *g, const double *base, 
     }
 }
 
-// Stage in double precision, one cell per thread.  Bound by the FP64 pipe (146 / 162
-// instructions of 64 cycles in the two stages); with all sums and differences on that pipe
+// Stage in double precision, one cell per thread.  Bound by the FP64 pipe (141 / 157
+// instructions of 64 cycles in the two stages, 86-87 % busy); with all sums and differences on that pipe
 // it took 246 / 262 at best, rows marched and differences shared.  4.59 ms per 4096^2 stage
 // of the vortex (7.91 before), 0.557 per 1500 x 1300 of smooth fields (1.02).  64 registers
 // for 32 warps per SM, which hide the latency of the integer chains (20 warps: 4.59-4.72 and

@@ -1,8 +1,8 @@
 // One cell of a Runge-Kutta stage in double precision: the operations and the rounding of
 // primitives(), equilibrium() and nnd(), with the sums of the velocity groups and the
 // transport differences on the integer pipes where they have the bits of the FP64
-// operations (cdbm_exact.h).  That leaves 146 / 162 of the 246 / 262 FP64 instructions per
-// cell and stage.
+// operations (cdbm_exact.h).  That leaves 141 / 157 of the 246 / 262 FP64 instructions per
+// cell in the two stages.
 //
 // rounded: the quadrupole of a group is rounded before it is added to the group sum.  The
 // stages of tubes of up to kRoundedTube cells round so, all other grids fuse the product
